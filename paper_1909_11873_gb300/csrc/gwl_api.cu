@@ -278,6 +278,8 @@ int gwl_create(const double* freqs, int64_t n_bins, const double* strain, const 
     if ((e = dev_alloc(c, &c->d_H, (int64_t)n_det * n_bins)) != cudaSuccess) { rc = cuda_fail(e, "alloc"); break; }
     if ((e = dev_alloc(c, &c->d_tab_mixed, n_bins * c->row_floats)) != cudaSuccess) { rc = cuda_fail(e, "alloc"); break; }
     if ((e = dev_alloc(c, &c->d_tab_delta, n_bins * c->row_delta)) != cudaSuccess) { rc = cuda_fail(e, "alloc"); break; }
+    if ((e = dev_alloc(c, &c->d_tab_block, (n_bins + gwl::kAnchor - 1) / gwl::kAnchor * gwl::block_floats(n_det))) !=
+        cudaSuccess) { rc = cuda_fail(e, "alloc"); break; }
     if ((e = dev_alloc(c, &c->d_anchor, (n_bins + gwl::kAnchor - 1) / gwl::kAnchor * gwl::kAnchorRowFloats)) !=
         cudaSuccess) { rc = cuda_fail(e, "alloc"); break; }
     if ((e = dev_alloc(c, &c->d_tab_f64, n_bins * c->row_doubles)) != cudaSuccess) { rc = cuda_fail(e, "alloc"); break; }
@@ -359,7 +361,7 @@ int gwl_loglike(gwl_ctx* c, const double* theta_dev, int64_t B, double* lnl_dev,
   if (B < 0) return fail(GWL_ERR_ARG, "B < 0");
   if (B == 0) return GWL_OK;
   if (!theta_dev || !lnl_dev) return fail(GWL_ERR_ARG, "null device pointer");
-  if ((rc = ensure_scratch(c, B))) return rc;
+  if (!gwl::fused_used(c, B) && (rc = ensure_scratch(c, B))) return rc;  // the one-kernel form needs no scratch
   cudaStream_t st = (cudaStream_t)stream;
   c->last_stream = st;
   cudaError_t e = gwl::launch_loglike(c, theta_dev, B, lnl_dev, st);
@@ -875,6 +877,7 @@ void gwl_destroy(gwl_ctx* c) {
   dev_free(c, c->d_H, (int64_t)c->n_det * c->M);
   dev_free(c, c->d_tab_mixed, c->M * c->row_floats);
   dev_free(c, c->d_tab_delta, c->M * c->row_delta);
+  dev_free(c, c->d_tab_block, (c->M + gwl::kAnchor - 1) / gwl::kAnchor * gwl::block_floats(c->n_det));
   dev_free(c, c->d_anchor, (c->M + gwl::kAnchor - 1) / gwl::kAnchor * gwl::kAnchorRowFloats);
   dev_free(c, c->d_tab_f64, c->M * c->row_doubles);
   dev_free(c, c->d_cal_f, (c->M + 1) * c->row_cal_f);

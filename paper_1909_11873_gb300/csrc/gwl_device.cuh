@@ -49,6 +49,18 @@ __host__ __device__ constexpr int f64_row_doubles(int ndet) { return 2 * odd_uni
 constexpr int kAnchor = 32;
 __host__ __device__ constexpr int delta_row_floats(int ndet) { return 4 * odd_units((16 + 2 * ndet + 3) / 4); }
 constexpr int kAnchorRowFloats = 28;
+// The fused likelihood's copy of what an FP32-delta bin reads, [dB_hi 0..7][G_d]
+// in 16-byte units, blocked by the 32 bins of an anchor block with the bins of
+// a unit side by side ([block][unit][32 bins][4 floats], zeros past the last
+// bin): a warp's vector loads are conflict-free without padding (64 bytes per
+// bin with three or four detectors, 48 with one or two, against 112 and 80-112
+// of a delta row), so that a CTA's shared memory holds more windows.
+__host__ __device__ constexpr int block_units(int ndet) { return (kNBasis + 2 * ndet + 3) / 4; }
+__host__ __device__ constexpr int block_floats(int ndet) { return 4 * kAnchor * block_units(ndet); }
+// Index of float k of bin j in that table.
+__host__ __device__ constexpr int64_t block_index(int64_t j, int k, int ndet) {
+  return j / kAnchor * block_floats(ndet) + (k / 4) * 4 * kAnchor + (j % kAnchor) * 4 + k % 4;
+}
 
 // Calibration model (Section 2.2 of the paper): per detector, amplitude and
 // phase corrections at n_nodes frequency nodes, natural cubic splines in

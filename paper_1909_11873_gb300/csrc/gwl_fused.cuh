@@ -1,0 +1,489 @@
+// gwl_fused.cuh -- the mixed likelihood of a small group of rows on one CTA:
+// coefficients, bin sums and combination with nothing passed through global
+// memory.
+//
+// A CTA of eight warps owns up to 32 rows of theta.  Its warps first play the
+// parts of the float-float prologue (eight parts instead of the four of
+// k_prologue, so that no warp's dependent chain holds two elementary
+// functions in a row where they are independent), while the table rows of the
+// first windows are being copied into shared memory; then all threads form
+// the anchor terms of the rows' 32-bin blocks, one (row, block) per thread;
+// then warps take (row, window) items, longest rows first, and sum them with
+// the lane and block order of k_window, so that every FP32 sum has the bits
+// that k_window gives; then the windows' sums are added in window order and
+// combined in FP64, one row per thread.
+//
+// Against the separate clearing, prologue and bin-loop kernels this takes out
+// two launches with the waits between them, the coefficient records' way
+// through L2, the global claim counters with their ~1 us round trips, two
+// thirds of the anchor work (a short row has 10-19 blocks, and k_window gives
+// each row's blocks a whole warp) and, by the folded warp reduction below,
+// half of the reduction's instructions.
+#pragma once
+
+#include "gwl_bins.cuh"
+#include "gwl_ff.cuh"
+
+namespace gwl {
+
+constexpr int kFusedRows = 32;  // rows per CTA at most (one per lane in the prologue)
+
+// Anchor record of a (row, block): the anchor terms of the detectors, then a
+// flag (nonzero: the block takes the FP32 delta), in 8- or 16-byte units.
+__host__ __device__ constexpr int anchor_rec_floats(int ndet) { return ndet == 1 ? 2 : ndet <= 3 ? 4 : 8; }
+
+// Where the parts of a CTA's dynamic shared memory begin (floats).
+struct FusedLayout {
+  int anchor;   // anchor rows of the staged windows (the table rows begin at 0)
+  int cal;      // calibration rows
+  int rec;      // anchor records [R][blocks]
+  int part;     // FP32 sums [R][windows][S NDET]
+  int total;
+};
+
+__host__ __device__ inline FusedLayout fused_layout(int ndet, int cal_row, int CH, int nwc, int R) {
+  FusedLayout l;
+  const int bins = CH * nwc, blocks = (CH + kAnchor - 1) / kAnchor * nwc;
+  l.anchor = blocks * block_floats(ndet);
+  l.cal = l.anchor + blocks * kAnchorRowFloats;
+  l.rec = l.cal + (cal_row ? (bins + 2) * cal_row : 0);  // calibration rows are staged in pairs
+  l.rec = (l.rec + 3) & ~3;
+  l.part = l.rec + R * blocks * anchor_rec_floats(ndet);
+  l.total = l.part + R * nwc * (cal_row ? 3 : 2) * ndet;
+  return l;
+}
+
+// One event's tables and launch shape, as the group's code needs them.
+struct FusedArgs {
+  SegInfo seg;
+  const float* tab;     // blocked table (FP32-delta bins)
+  const float* rows;    // delta rows, read in place by the blocks with float-float deltas
+  int row_elems;        // floats per delta row
+  const float* anchor;  // anchor rows
+  int CH;               // bins per window (a multiple of 32)
+  int nwc;              // windows staged together
+  float df;
+  // calibration model (instances with CAL only)
+  const float* cal;
+  int cal_row;
+  int cal_par;          // first calibration parameter of a row
+  int nn;
+  const float* calQ;
+  int* status;
+  unsigned long long* ffc;  // diagnostic counter of float-float-delta blocks, or null
+};
+
+// Static shared memory of a group.
+template <int NDET, bool CAL>
+struct FusedSmem {
+  static constexpr int NS = (CAL ? 3 : 2) * NDET;  // sums per row
+  FF lmc[kFusedRows], leta[kFusedRows], eta[kFusedRows], amp[kFusedRows];
+  FF phi[6][kFusedRows];
+  FF sky[4][kFusedRows], ori[3][kFusedRows];
+  FF P[2 * NDET][kFusedRows], ang[2][kFusedRows], hterm[NDET][kFusedRows];
+  double Hc[NDET][kFusedRows], Kr[NDET][kFusedRows], Ki[NDET][kFusedRows];
+  double acc[NS][kFusedRows];
+  PropMixed pm[kFusedRows];
+  int ncut[kFusedRows], flag[kFusedRows];
+  int order[kFusedRows];  // rows by descending cut
+  int next, maxcut;
+  alignas(8) uint64_t bar;
+  alignas(16) float4 nodes[CAL ? 8 * NDET * kMaxCalNodes : 1];
+};
+
+// One thread: the table rows (and anchor and calibration rows) of windows
+// [w0, w0 + nwc) into shared memory, completing on the group's barrier.
+template <int NDET, bool CAL>
+__device__ __forceinline__ void fused_stage(const FusedArgs& a, const FusedLayout& L, float* dyn, int w0,
+                                            uint64_t* bar) {
+  const int64_t j0 = (int64_t)w0 * a.CH;
+  int64_t j1 = j0 + (int64_t)a.nwc * a.CH;
+  if (j1 > a.seg.M) j1 = a.seg.M;
+  const int n = (int)(j1 - j0), nb = (n + kAnchor - 1) / kAnchor;
+  const uint32_t bytes = (uint32_t)nb * (uint32_t)(block_floats(NDET) * 4);
+  const uint32_t abytes = (uint32_t)nb * (uint32_t)(kAnchorRowFloats * 4);
+  const uint32_t cbytes = CAL ? (uint32_t)((n + 1) & ~1) * (uint32_t)a.cal_row * 4u : 0u;
+  mbar_arrive_expect_tx(bar, bytes + abytes + cbytes);
+  bulk_g2s(dyn, a.tab + j0 / kAnchor * block_floats(NDET), bytes, bar);
+  bulk_g2s(dyn + L.anchor, a.anchor + (j0 / kAnchor) * kAnchorRowFloats, abytes, bar);
+  if constexpr (CAL) bulk_g2s(dyn + L.cal, a.cal + j0 * a.cal_row, cbytes, bar);
+}
+
+// The coefficients of rows 0 .. R-1, th(k, lane) giving parameter k of the
+// lane's row (called only for lanes below R): the arithmetic of
+// prologue_rows_ff, operation by operation.  Ends with a CTA barrier after
+// which pm, ncut, flag and maxcut are in place; K_d and the <h|h> terms
+// follow on warps 0 .. NDET-1 and the order of the rows on warp 7, without a
+// barrier after them.
+//   part 0: ln(pi Mc T_sun); c_m         part 4: dec; response and delay of detector 0
+//   part 1: PN coefficients; amplitude   part 5: psi; ... of detector 1
+//   part 2: ln eta; K's phase angle      part 6: iota; ... of detector 2
+//   part 3: ra; cut and H_d there        part 7: checks, prefetch; ... of detector 3
+template <int NDET, bool CAL, class Th>
+__device__ __forceinline__ void fused_coeffs(const SegInfo& s, int R, FusedSmem<NDET, CAL>& sm, Th th) {
+  const int part = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const bool valid = lane < R;
+  // ---- phase 1
+  if (part == 0) {
+    const double mc = valid ? th(0) : 10.0;
+    sm.lmc[lane] = log(ff_from(mc) * (kPi * kTsun));
+  } else if (part == 1) {
+    const double q = valid ? th(1) : 0.5, x1 = valid ? th(2) : 0.0, x2 = valid ? th(3) : 0.0;
+    const PNCoeffs<FF> P = pn_coeffs(ff_from(q), ff_from(x1), ff_from(x2));
+    sm.eta[lane] = P.eta;
+    sm.phi[0][lane] = P.p2;
+    sm.phi[1][lane] = P.p3;
+    sm.phi[2][lane] = P.p4;
+    sm.phi[3][lane] = P.p5c;
+    sm.phi[4][lane] = P.p6c;
+    sm.phi[5][lane] = P.p7;
+  } else if (part == 2) {
+    const FF q = ff_from(valid ? th(1) : 0.5);
+    const FF opq = q + 1.0;
+    sm.leta[lane] = log(q / (opq * opq));
+  } else if (part == 7) {
+    double x[11];
+#pragma unroll
+    for (int k = 0; k < 11; ++k) x[k] = valid ? th(k) : 1.0;
+    const bool ok = valid && physical(x);
+    sm.flag[lane] = ok ? 0 : 1;
+    if (ok) prefetch_cut_H(s, x[0], x[1]);
+  } else {  // parts 3-6: the sine and cosine of one angle
+    const double x = valid ? (part == 3 ? th(7) : part == 4 ? th(8) : part == 5 ? th(6) : th(5)) : 0.0;
+    FF f = ff_from(x);
+    if (part == 3) f = f - s.gmst;
+    FF sn, cs;
+    sincos(f, &sn, &cs);
+    if (part == 3) {
+      sm.sky[0][lane] = sn;
+      sm.sky[1][lane] = cs;
+    } else if (part == 4) {
+      sm.sky[2][lane] = sn;
+      sm.sky[3][lane] = cs;
+    } else if (part == 5) {
+      sm.ori[0][lane] = sn;
+      sm.ori[1][lane] = cs;
+    } else {
+      sm.ori[2][lane] = cs;
+    }
+  }
+  __syncthreads();
+  // ---- phase 2
+  const bool ok = sm.flag[lane] == 0;
+  if (part == 0) {
+    Scale<FF> S;
+    S.la = sm.lmc[lane] - 0.6 * sm.leta[lane];
+    S.a13 = exp(S.la * (1.0 / 3.0));
+    S.amp = ff(0.0f);
+    PNCoeffs<FF> P;
+    P.eta = sm.eta[lane];
+    P.p2 = sm.phi[0][lane];
+    P.p3 = sm.phi[1][lane];
+    P.p4 = sm.phi[2][lane];
+    P.p5c = sm.phi[3][lane];
+    P.p6c = sm.phi[4][lane];
+    P.p7 = sm.phi[5][lane];
+    FF c[kNBasis], ccyc;
+    basis_coeffs(P, S, c, ccyc);
+#pragma unroll
+    for (int m = 0; m < kNBasis; ++m) {
+      sm.pm[lane].ch[m] = ok ? c[m].hi : 0.0f;
+      sm.pm[lane].cl[m] = ok ? c[m].lo : 0.0f;
+    }
+  } else if (part == 1) {
+    const double dl = valid ? th(4) : 100.0;
+    sm.amp[lane] = exp((sm.lmc[lane] - kLnPi) * (5.0 / 6.0)) * s.amp_c_ff / ff_from(dl);
+  } else if (part == 2) {
+    // the same constant-phase cycles as basis_coeffs forms in part 0
+    const double phic = valid ? th(10) : 0.0;
+    const FF la = sm.lmc[lane] - 0.6 * sm.leta[lane];
+    const FF ccyc = const_cycles(cycles_pref(sm.eta[lane]), sm.phi[3][lane], la);
+    FF sa, ca;
+    sincos(ff_from(phic) + 0.25 * kPi - (2.0 * kPi) * frac_near(ccyc), &sa, &ca);
+    sm.ang[0][lane] = sa;
+    sm.ang[1][lane] = ca;
+  } else if (part == 3) {
+    const FF la = sm.lmc[lane] - 0.6 * sm.leta[lane];
+    const FF a13 = exp(la * (1.0 / 3.0));
+    int ncut = 0;
+    if (ok) {
+      ncut = (int)s.M;
+      if (s.fcut_mode == 0) ncut = count_bins_le(s, ff_to_double(1.0 / (kSix32 * (a13 * a13 * a13))));
+    }
+    sm.ncut[lane] = ncut;
+    const int nm = __reduce_max_sync(0xffffffffu, ncut);
+    if (lane == 0) sm.maxcut = nm;
+#pragma unroll
+    for (int d = 0; d < NDET; ++d) sm.Hc[d][lane] = ncut > 0 ? s.H[(int64_t)d * s.M + ncut - 1] : 0.0;
+  } else if (part - 4 < NDET) {
+    const int d = part - 4;
+    Sky<FF> k;
+    k.sl = sm.sky[0][lane];
+    k.cl = sm.sky[1][lane];
+    k.sd = sm.sky[2][lane];
+    k.cd = sm.sky[3][lane];
+    const FF tau = delay_vc(ff_from(valid ? th(9) : 0.0), k, s.vtx_c_ff[d]);
+    sm.pm[lane].th[d] = ok ? tau.hi : 0.0f;
+    sm.pm[lane].tl[d] = ok ? tau.lo : 0.0f;
+    FF Pr, Pi;
+    response(k, sm.ori[0][lane], sm.ori[1][lane], sm.ori[2][lane], s.geom_ff[d], Pr, Pi);
+    sm.P[2 * d][lane] = Pr;
+    sm.P[2 * d + 1][lane] = Pi;
+  }
+  __syncthreads();
+  // ---- phase 3 (no barrier after it)
+  if (part < NDET) {
+    const int d = part;
+    const FF amp = sm.amp[lane], Pr = sm.P[2 * d][lane], Pi = sm.P[2 * d + 1][lane];
+    const FF sa = sm.ang[0][lane], ca = sm.ang[1][lane];
+    const FF kr = amp * (Pr * ca - Pi * sa), ki = amp * (Pr * sa + Pi * ca);
+    sm.Kr[d][lane] = ff_to_double(kr);
+    sm.Ki[d][lane] = ff_to_double(ki);
+    sm.hterm[d][lane] = (kr * kr + ki * ki) * ff_from(sm.Hc[d][lane]);
+  } else if (part == 7) {
+    const int n = valid ? sm.ncut[lane] : -1;
+    int rank = 0;
+#pragma unroll 4
+    for (int l = 0; l < 32; ++l) {
+      const int m = __shfl_sync(0xffffffffu, n, l);
+      rank += (m > n || (m == n && l < lane)) ? 1 : 0;
+    }
+    sm.order[rank] = lane;
+  }
+}
+
+// Warp sums of n FP32 values per lane with the tree of an xor butterfly over
+// 16, 8, 4, 2, 1: at each level a lane keeps one half of its values and hands
+// the other half to its partner, so that value v is added up by the lanes
+// whose upper lane bits spell v, with the same operand pairs, hence the same
+// bits, as the butterfly of every value on every lane (n <= 16; 9 shuffles
+// instead of 30 for six values).  The result of value v is returned on lanes
+// [v W, v W + W), W = 32 / P, P the power of two at or above n.
+template <int N>
+struct FoldP {
+  static constexpr int P = N <= 2 ? 2 : N <= 4 ? 4 : N <= 8 ? 8 : 16;
+  static constexpr int W = 32 / P;
+};
+template <int N>
+__device__ __forceinline__ float warp_fold(const float (&v)[N], int lane) {
+  constexpr int P = FoldP<N>::P;
+  float t[P];
+#pragma unroll
+  for (int k = 0; k < P; ++k) t[k] = k < N ? v[k] : 0.0f;
+  int off = 16;
+#pragma unroll
+  for (int h = P / 2; h >= 1; h >>= 1, off >>= 1) {
+    const bool up = (lane & off) != 0;
+#pragma unroll
+    for (int k = 0; k < h; ++k) {
+      const float send = up ? t[k] : t[k + h];
+      const float keep = up ? t[k + h] : t[k];
+      t[k] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+    }
+  }
+#pragma unroll
+  for (; off >= 1; off >>= 1) t[0] += __shfl_xor_sync(0xffffffffu, t[0], off);
+  return t[0];
+}
+
+// FP32 sums of one row over bins [jl, jl + n) of the staged windows (jl a
+// multiple of 32, in bins from the first staged one; j0 that one's index in
+// the segment): the blocks in order, lanes over a block's bins, as
+// anchored_sums_cal.
+template <int NDET, bool CAL>
+__device__ __forceinline__ void fused_row_sums(const FusedArgs& a, const FusedLayout& L, const float* __restrict__ dyn,
+                                               const PropMixed& P, const float* __restrict__ rec, int j0, int jl, int n,
+                                               int lane, const float4* __restrict__ nodes, float (&U)[NDET],
+                                               float (&V)[NDET], float (&X)[NDET]) {
+  constexpr int RX = 4 * ((kNBasis + 2 * NDET + 3) / 4);
+  constexpr int RXF = 4 * ((2 * kNBasis + 2 * NDET + 3) / 4);
+  constexpr int AR = anchor_rec_floats(NDET);
+  float ch[kNBasis], dtl[NDET];
+#pragma unroll
+  for (int q = 0; q < kNBasis / 4; ++q)
+    *reinterpret_cast<float4*>(&ch[4 * q]) = reinterpret_cast<const float4*>(P.ch)[q];
+  const float lane_df = (float)lane * a.df;
+#pragma unroll
+  for (int d = 0; d < NDET; ++d) {
+    dtl[d] = __fmul_rn(P.th[d], lane_df);
+    U[d] = V[d] = X[d] = 0.0f;
+  }
+  auto record = [&](int b, float (&ad)[NDET]) {
+    float r[AR];
+    if constexpr (AR == 2) {
+      *reinterpret_cast<float2*>(r) = *reinterpret_cast<const float2*>(rec + AR * b);
+    } else {
+#pragma unroll
+      for (int q = 0; q < AR / 4; ++q)
+        *reinterpret_cast<float4*>(&r[4 * q]) = *reinterpret_cast<const float4*>(rec + AR * b + 4 * q);
+    }
+#pragma unroll
+    for (int d = 0; d < NDET; ++d) ad[d] = __fadd_rn(r[d], dtl[d]);
+    return r[NDET] != 0.0f;
+  };
+  constexpr int BF = block_floats(NDET);
+  const float* row = dyn + jl / kAnchor * BF + 4 * lane;
+  const float* crow = CAL ? dyn + L.cal + (jl + lane) * a.cal_row : nullptr;
+  const int cstep = CAL ? kAnchor * a.cal_row : 0;
+  CalBin<NDET, float> cb0, cb1;
+  const int nblk = (n + kAnchor - 1) / kAnchor;
+  for (int b = 0; b < nblk;) {
+    float ad0[NDET], ad1[NDET];
+    const bool f0 = record(b, ad0);
+    bool pair = f0 && (b + 2) * kAnchor <= n;
+    if (pair) pair = record(b + 1, ad1);
+    if (pair) {
+      // two complete blocks with FP32 deltas, in straight-line code so that their chains interleave
+      float v0[RX], v1[RX];
+#pragma unroll
+      for (int k = 0; k < RX / 4; ++k) {
+        *reinterpret_cast<float4*>(&v0[4 * k]) = reinterpret_cast<const float4*>(row)[kAnchor * k];
+        *reinterpret_cast<float4*>(&v1[4 * k]) = reinterpret_cast<const float4*>(row + BF)[kAnchor * k];
+      }
+      if constexpr (CAL) {
+        cal_eval<NDET>(crow, nodes, cb0);
+        cal_eval<NDET>(crow + cstep, nodes, cb1);
+      }
+      bin_anchor<NDET, CAL>(v0, ch, ad0, U, V, cb0, X);
+      bin_anchor<NDET, CAL>(v1, ch, ad1, U, V, cb1, X);
+      b += 2;
+      row += 2 * BF;
+      if (CAL) crow += 2 * cstep;
+      continue;
+    }
+    if (b * kAnchor + lane < n) {  // lanes past the cut sit out
+      if constexpr (CAL) cal_eval<NDET>(crow, nodes, cb0);
+      if (f0) {
+        float v[RX];
+#pragma unroll
+        for (int k = 0; k < RX / 4; ++k)
+          *reinterpret_cast<float4*>(&v[4 * k]) = reinterpret_cast<const float4*>(row)[kAnchor * k];
+        bin_anchor<NDET, CAL>(v, ch, ad0, U, V, cb0, X);
+      } else {
+        if (a.ffc && lane == 0) atomicAdd(a.ffc, 1ull);
+        float v[RXF], cl[kNBasis];
+#pragma unroll
+        for (int q = 0; q < kNBasis / 4; ++q)
+          *reinterpret_cast<float4*>(&cl[4 * q]) = reinterpret_cast<const float4*>(P.cl)[q];
+        const float4* full = reinterpret_cast<const float4*>(a.rows + (int64_t)(j0 + jl + b * kAnchor + lane) * a.row_elems);
+#pragma unroll
+        for (int k = 0; k < RXF / 4; ++k) *reinterpret_cast<float4*>(&v[4 * k]) = __ldg(full + k);
+        bin_anchor_exact<NDET, CAL>(v, ch, cl, ad0, U, V, cb0, X);
+      }
+    }
+    b += 1;
+    row += BF;
+    if (CAL) crow += cstep;
+  }
+}
+
+// Bin sums of the group's rows (all threads; fused_coeffs before it): the
+// windows in groups of nwc, each staged (the first group's copy has been
+// started by the caller), its anchor records, its (row, window) items, its
+// windows' sums added to sm.acc in window order.  parity: the barrier's
+// phase.  crow(r): the calibration parameters of row r in global memory.
+// Returns false when a bounded wait ran out.
+template <int NDET, bool CAL, class Crow>
+__device__ __forceinline__ bool fused_bins(const FusedArgs& a, const FusedLayout& L, float* dyn, int R,
+                                           FusedSmem<NDET, CAL>& sm, uint32_t& parity, bool& staged, Crow crow) {
+  constexpr int NS = FusedSmem<NDET, CAL>::NS, AR = anchor_rec_floats(NDET);
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const int gbins = a.CH * a.nwc, gblk = (a.CH + kAnchor - 1) / kAnchor * a.nwc;
+  const int maxcut = sm.maxcut;
+  for (int i = t; i < NS * kFusedRows; i += 256) (&sm.acc[0][0])[i] = 0.0;
+  for (int w0 = 0; (int64_t)w0 * a.CH < maxcut; w0 += a.nwc) {
+    const int j0 = w0 * a.CH;
+    const int top = maxcut - j0 < gbins ? maxcut - j0 : gbins;  // the longest row's bins in this group
+    if (!staged) {
+      if (t == 0) {
+        fence_proxy_async_smem();
+        fused_stage<NDET, CAL>(a, L, dyn, w0, &sm.bar);
+      }
+    }
+    if (!mbar_wait_bounded(&sm.bar, parity, a.status)) return false;
+    parity ^= 1u;
+    staged = false;
+    // anchor records, blocks of a row on neighbouring threads
+    const int nb = (top + kAnchor - 1) / kAnchor;
+    for (int i = t; i < R * nb; i += 256) {
+      const int r = i / nb, b = i - r * nb;
+      if (j0 + b * kAnchor >= sm.ncut[r]) continue;
+      float ch[kNBasis], cl[kNBasis], th[NDET], tl[NDET], an[NDET];
+      const PropMixed& P = sm.pm[r];
+#pragma unroll
+      for (int m = 0; m < kNBasis; ++m) {
+        ch[m] = P.ch[m];
+        cl[m] = P.cl[m];
+      }
+#pragma unroll
+      for (int d = 0; d < NDET; ++d) {
+        th[d] = P.th[d];
+        tl[d] = P.tl[d];
+      }
+      const bool fast = anchor_terms<NDET>(dyn + L.anchor + b * kAnchorRowFloats, ch, cl, th, tl, an);
+      float* o = dyn + L.rec + (r * gblk + b) * AR;
+#pragma unroll
+      for (int d = 0; d < NDET; ++d) o[d] = an[d];
+      o[NDET] = fast ? 1.0f : 0.0f;
+    }
+    if (t == 0) sm.next = 0;
+    __syncthreads();
+    const int nwa = (top + a.CH - 1) / a.CH;  // windows of the group that hold bins
+    while (true) {
+      int item = 0;
+      if (lane == 0) item = atomicAdd(&sm.next, 1);
+      item = __shfl_sync(0xffffffffu, item, 0);
+      if (item >= R * nwa) break;
+      const int wl = item / R, r = sm.order[item - wl * R];
+      const int jl = wl * a.CH;
+      int n = sm.ncut[r] - j0 - jl;
+      if (n <= 0) continue;
+      if (n > a.CH) n = a.CH;
+      float4* nodes = sm.nodes + (CAL ? warp * NDET * kMaxCalNodes : 0);
+      if constexpr (CAL) cal_nodes_fill<NDET, true>(crow(r), a.nn, a.calQ, lane, nodes);
+      float U[NDET], V[NDET], X[NDET], v[NS];
+      fused_row_sums<NDET, CAL>(a, L, dyn, sm.pm[r], dyn + L.rec + (r * gblk + jl / kAnchor) * AR, j0, jl, n, lane, nodes,
+                                U, V, X);
+#pragma unroll
+      for (int d = 0; d < NDET; ++d) {
+        v[2 * d] = U[d];
+        v[2 * d + 1] = V[d];
+        if constexpr (CAL) v[2 * NDET + d] = X[d];
+      }
+      const float s = warp_fold<NS>(v, lane);
+      constexpr int W = FoldP<NS>::W;
+      if (lane % W == 0 && lane / W < NS) dyn[L.part + (r * a.nwc + wl) * NS + lane / W] = s;
+    }
+    __syncthreads();
+    // the group's window sums, in window order (one thread per row and sum)
+    for (int i = t; i < R * NS; i += 256) {
+      const int r = i / NS, k = i - r * NS;
+      const int left = sm.ncut[r] - j0;
+      double x = sm.acc[k][r];
+      for (int wl = 0; wl < nwa && wl * a.CH < left; ++wl) x += (double)dyn[L.part + (r * a.nwc + wl) * NS + k];
+      sm.acc[k][r] = x;
+    }
+    __syncthreads();
+  }
+  return true;
+}
+
+// lnL of row r from the sums (one thread): -inf for an unphysical row, 0
+// without an in-band bin.
+template <int NDET, bool CAL>
+__device__ __forceinline__ double fused_combine(const FusedSmem<NDET, CAL>& sm, int r) {
+  if (sm.flag[r]) return -INFINITY;
+  if (sm.ncut[r] <= 0) return 0.0;
+  FF hh = ff(0.0f);
+  double acc = 0.0;
+#pragma unroll
+  for (int d = 0; d < NDET; ++d) {
+    hh = hh + sm.hterm[d][r];
+    const double kr = sm.Kr[d][r], ki = sm.Ki[d][r];
+    acc += kr * sm.acc[2 * d][r] - ki * sm.acc[2 * d + 1][r];
+    if constexpr (CAL) acc -= 0.5 * (kr * kr + ki * ki) * sm.acc[2 * NDET + d][r];
+  }
+  return acc - 0.5 * ff_to_double(hh);
+}
+
+}  // namespace gwl

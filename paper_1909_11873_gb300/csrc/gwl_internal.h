@@ -26,6 +26,7 @@ struct gwl_ctx {
   float* d_tab_delta = nullptr;  // [M][delta_row_floats]: basis deltas from the block anchor, G_d
   float* d_anchor = nullptr;     // [ceil(M / kAnchor)][kAnchorRowFloats]
   int row_delta = 0;
+  float* d_tab_block = nullptr;  // [ceil(M / kAnchor)][block_floats]: the FP32-delta bins' part, blocked
   double* d_tab_f64 = nullptr;   // [M][f64_row_doubles]
   int row_floats = 0, row_doubles = 0;
 
@@ -137,6 +138,11 @@ cudaError_t launch_loglike(gwl_ctx* c, const double* theta, int64_t B, double* l
 // ints of d_work) and wrote theta: no clearing kernel
 cudaError_t launch_loglike_cleared(gwl_ctx* c, const double* theta, int64_t B, double* lnl, cudaStream_t st);
 int64_t work_needed(const gwl_ctx* c, int64_t B);
+// the one-kernel form (gwl_fused.cu): its launch shape for a batch (false: not used), launch
+bool fused_shape(const gwl_ctx* c, int64_t B, int* grid, int* rows, int* nwc);
+bool fused_used(const gwl_ctx* c, int64_t B);
+cudaError_t launch_fused(gwl_ctx* c, const double* theta, int64_t B, double* lnl, int grid, int rows, int nwc,
+                         cudaStream_t st);
 // the lane-per-proposal bin loop (gwl_lanes.cu): chunk size (0: not used), scratch sizes, launch
 int lanes_seg(const gwl_ctx* c, int64_t B);
 int64_t lanes_list_ints(const gwl_ctx* c, int64_t B);

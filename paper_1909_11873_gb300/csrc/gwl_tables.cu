@@ -31,8 +31,8 @@ __device__ __forceinline__ void basis_values(double f, double (&b)[kNBasis]) {
 __global__ void k_table_rows(const double* __restrict__ freqs, const double* __restrict__ strain,
                              const double* __restrict__ psd, int64_t M, int n_det, double df, double t_ref,
                              float* __restrict__ tab_m, int row_f, double* __restrict__ tab_d, int row_d,
-                             float* __restrict__ tab_x, int row_x, float* __restrict__ anc,
-                             double* __restrict__ hterm) {
+                             float* __restrict__ tab_x, int row_x, float* __restrict__ tab_b,
+                             float* __restrict__ anc, double* __restrict__ hterm) {
   const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= M) return;
   const double f = freqs[j];
@@ -44,7 +44,11 @@ __global__ void k_table_rows(const double* __restrict__ freqs, const double* __r
   const int lo_off = kNBasis + 2 * n_det;  // low parts after G
   for (int k = lo_off + kNBasis; k < row_x; ++k) rx[k] = 0.0f;
 #pragma unroll
-  for (int m = 0; m < kNBasis; ++m) split_f64(b[m] - ba[m], rx[m], rx[lo_off + m]);
+  for (int m = 0; m < kNBasis; ++m) {
+    split_f64(b[m] - ba[m], rx[m], rx[lo_off + m]);
+    tab_b[block_index(j, m, n_det)] = rx[m];
+  }
+  for (int k = kNBasis; k < 4 * block_units(n_det); ++k) tab_b[block_index(j, k, n_det)] = 0.0f;  // G: k_scale_tables
   if (j == ja) {
     float* ra = anc + (j / kAnchor) * kAnchorRowFloats;
 #pragma unroll
@@ -130,7 +134,7 @@ __global__ void k_prefix_scan(double* __restrict__ H, int64_t M) {
 // Multiply the data weights by 2^-e and the prefix sums by 2^-2e (exact).
 __global__ void k_scale_tables(int64_t M, int n_det, double sg, float* __restrict__ tab_m, int row_f,
                                double* __restrict__ tab_d, int row_d, float* __restrict__ tab_x, int row_x,
-                               double* __restrict__ H) {
+                               float* __restrict__ tab_b, double* __restrict__ H) {
   const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= M) return;
   for (int d = 0; d < n_det; ++d) {
@@ -140,6 +144,8 @@ __global__ void k_scale_tables(int64_t M, int n_det, double sg, float* __restric
     tab_m[j * row_f + 19 + 2 * d] = (float)tab_d[j * row_d + 10 + 2 * d];
     tab_x[j * row_x + kNBasis + 2 * d] = tab_m[j * row_f + 18 + 2 * d];
     tab_x[j * row_x + kNBasis + 2 * d + 1] = tab_m[j * row_f + 19 + 2 * d];
+    tab_b[block_index(j, kNBasis + 2 * d, n_det)] = tab_m[j * row_f + 18 + 2 * d];
+    tab_b[block_index(j, kNBasis + 2 * d + 1, n_det)] = tab_m[j * row_f + 19 + 2 * d];
     H[(int64_t)d * M + j] *= sg * sg;
   }
 }
@@ -148,7 +154,7 @@ cudaError_t launch_scale_tables(gwl_ctx* c, double sg, cudaStream_t st) {
   const int T = 256;
   k_scale_tables<<<(unsigned)((c->M + T - 1) / T), T, 0, st>>>(c->M, c->n_det, sg, c->d_tab_mixed, c->row_floats,
                                                                 c->d_tab_f64, c->row_doubles, c->d_tab_delta,
-                                                                c->row_delta, c->d_H);
+                                                                c->row_delta, c->d_tab_block, c->d_H);
   c->launches++;
   return cudaGetLastError();
 }
@@ -201,11 +207,15 @@ cudaError_t launch_cal_tables(gwl_ctx* c, const double* d_xnode, cudaStream_t st
 cudaError_t launch_build_tables(gwl_ctx* c, const double* d_strain, const double* d_psd, cudaStream_t st) {
   const int T = 256;
   const int64_t nb = (c->M + T - 1) / T;
+  // the bins past the last one in its block
+  const int64_t last = (c->M - 1) / kAnchor * block_floats(c->n_det);
+  cudaError_t e = cudaMemsetAsync(c->d_tab_block + last, 0, sizeof(float) * block_floats(c->n_det), st);
+  if (e != cudaSuccess) return e;
   k_table_rows<<<(unsigned)nb, T, 0, st>>>(c->d_freqs, d_strain, d_psd, c->M, c->n_det, c->df, c->opt.t_ref,
                                             c->d_tab_mixed, c->row_floats, c->d_tab_f64, c->row_doubles,
-                                            c->d_tab_delta, c->row_delta, c->d_anchor, c->d_H);
+                                            c->d_tab_delta, c->row_delta, c->d_tab_block, c->d_anchor, c->d_H);
   c->launches++;
-  cudaError_t e = cudaGetLastError();
+  e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   k_prefix_scan<<<c->n_det, 1024, 0, st>>>(c->d_H, c->M);
   c->launches++;
