@@ -444,6 +444,12 @@ int ns_replace(gwl_ctx* c, const double* live_u, const double* live_lnl, int64_t
   if (n_chains == 0) return GWL_OK;
   if (!live_u || !live_lnl || !chol || !out_u || !out_lnl || !out_nacc) return fail(GWL_ERR_ARG, "null device pointer");
   const int D = (int)gwl::theta_stride(c);
+  cudaError_t e = cudaSuccess;
+  if (gwl::launch_walk_direct(c, live_u, live_lnl, K, worst, lnl_star, seed, counter, n_chains, walk_len, scale, chol,
+                              out_u, out_lnl, out_nacc, out_start, (cudaStream_t)stream, &e)) {
+    c->last_stream = (cudaStream_t)stream;
+    return e == cudaSuccess ? GWL_OK : cuda_fail(e, "ns_replace");
+  }
   if ((rc = ensure_scratch(c, n_chains))) return rc;
   if ((rc = ensure_bytes(c, (void**)&c->d_walk, &c->walk_cap, (int64_t)sizeof(double) * n_chains * (2 * D + 1))))
     return rc;
@@ -451,7 +457,7 @@ int ns_replace(gwl_ctx* c, const double* live_u, const double* live_lnl, int64_t
   c->last_stream = st;
   unsigned char hs[64];
   gwl::set_walk_scalars(hs, lnl_star, scale, worst, counter);
-  cudaError_t e = cudaMemcpyAsync(c->d_wscal, hs, gwl::walk_scalars_bytes(), cudaMemcpyHostToDevice, st);
+  e = cudaMemcpyAsync(c->d_wscal, hs, gwl::walk_scalars_bytes(), cudaMemcpyHostToDevice, st);
   if (e != cudaSuccess) return cuda_fail(e, "ns_replace");
   if (c->walk_kind == GWL_WALK_GALILEAN) {
     if ((rc = ensure_bytes(c, (void**)&c->d_gmc, &c->gmc_cap, (int64_t)sizeof(double) * gwl::gmc_scratch_doubles(n_chains, D))))

@@ -233,14 +233,14 @@ __device__ __forceinline__ FF cos(const FF& x) {
 // operations), then form the curvatures m_k = sum_i Q_ki y_i from the stored
 // values.  Nodes: (dA_k, m^A_k, dphi_k, m^phi_k) per detector and node.
 template <int NDET, bool MIXED, typename Node>
-__device__ __forceinline__ void cal_nodes_fill(const double* __restrict__ y, int nn, const void* __restrict__ calQ,
+__device__ __forceinline__ void cal_nodes_fill(const double* y, int nn, const void* __restrict__ calQ,
                                                int lane, Node* __restrict__ nd) {
   using T = typename std::conditional<MIXED, float, double>::type;
   const T* Q = reinterpret_cast<const T*>(calQ);
   __syncwarp();  // the warp is done with the previous proposal's node data
   for (int o = lane; o < 2 * NDET * nn; o += 32) {
     const int sp = o / nn, k = o - sp * nn;
-    const double yd = __ldg(y + o);
+    const double yd = y[o];
     T yv;
     if constexpr (MIXED) yv = ff_from(yd).hi;
     else yv = yd;

@@ -33,13 +33,13 @@ __global__ void __launch_bounds__(256, 2) k_fused(const __grid_constant__ FusedA
   const int lane = threadIdx.x & 31;
   const double* row = theta + (row0 + lane) * a.seg.stride;
   fused_coeffs<NDET, CAL>(a.seg, n, sm,
-                          [&](int k) { return a.seg.param_pos[k] >= 0 ? row[a.seg.param_pos[k]] : a.seg.fixed[k]; });
-  uint32_t parity = 0;
-  bool staged = true;
-  if (!fused_bins<NDET, CAL>(a, L, dyn, n, sm, parity, staged,
+                          [&](int k) { return a.seg.param_pos[k] >= 0 ? row[a.seg.param_pos[k]] : a.seg.fixed[k]; },
+                          [](int) { return false; });
+  FusedStage st;
+  if (!fused_bins<NDET, CAL>(a, L, dyn, n, sm, st,
                              [&](int r) { return theta + (row0 + r) * a.seg.stride + a.cal_par; }))
     return;
-  if (staged) mbar_wait_bounded(&sm.bar, parity, a.status);  // no copy may outlive the CTA
+  if (st.pending) mbar_wait_bounded(&sm.bar, st.parity, a.status);  // no copy may outlive the CTA
   __syncthreads();
   if (threadIdx.x < n) lnl[row0 + threadIdx.x] = fused_combine<NDET, CAL>(sm, threadIdx.x);
 }
@@ -47,7 +47,7 @@ __global__ void __launch_bounds__(256, 2) k_fused(const __grid_constant__ FusedA
 // ---------------------------------------------------------------- host side
 int lnl_window(const gwl_ctx* c) { return c->window > c->M ? (int)c->M : c->window; }
 
-static size_t fused_bytes(const gwl_ctx* c, int nwc, int R) {
+size_t fused_bytes(const gwl_ctx* c, int nwc, int R) {
   return sizeof(float) * (size_t)fused_layout(c->n_det, c->n_cal_nodes ? c->row_cal_f : 0, lnl_window(c), nwc, R).total;
 }
 
@@ -88,7 +88,8 @@ constexpr size_t kSmemPerSm = 228 * 1024;  // 1 KB of it goes to each resident C
 //     327 / 1014 / 1388 / 2479 against 248 / 895 / 1529 / 3109
 // so segments of up to 32 windows take it at any batch, longer ones where the
 // batch gives every warp of two CTAs per SM a row.
-bool fused_shape(const gwl_ctx* c, int64_t B, int* grid, int* rows, int* nwc) {
+// row_bytes: shared memory that a caller's kernel needs besides, per row.
+bool fused_shape(const gwl_ctx* c, int64_t B, int* grid, int* rows, int* nwc, size_t row_bytes) {
   if (c->opt.precision != GWL_MIXED || B <= 0) return false;
   const int CH = lnl_window(c);
   const int64_t nw = (c->M + CH - 1) / CH;
@@ -99,7 +100,9 @@ bool fused_shape(const gwl_ctx* c, int64_t B, int* grid, int* rows, int* nwc) {
   const int64_t waves = (B + slots * kFusedRows - 1) / (slots * kFusedRows);
   const int64_t R = (B + slots * waves - 1) / (slots * waves);
   const int64_t G = (B + R - 1) / R;
-  const size_t room = (per_sm == 1 ? 227 * 1024 : kSmemPerSm / 2 - 1024) - fused_static(c) - 128;
+  const size_t room = (per_sm == 1 ? 227 * 1024 : kSmemPerSm / 2 - 1024) - fused_static(c) - 1024 -
+                      (size_t)R * row_bytes;
+  if ((size_t)R * row_bytes > 64 * 1024) return false;
   int w = 1;
   if (fused_bytes(c, 1, (int)R) > room) return false;
   while (w < nw && fused_bytes(c, w + 1, (int)R) <= room) ++w;
@@ -115,9 +118,7 @@ bool fused_used(const gwl_ctx* c, int64_t B) {
   return !lanes_seg(c, B) && fused_shape(c, B, &grid, &rows, &nwc);
 }
 
-template <int NDET, bool CAL>
-static cudaError_t run_fused(gwl_ctx* c, const double* theta, int64_t B, double* lnl, int grid, int rows, int nwc,
-                             cudaStream_t st) {
+FusedArgs fused_args(const gwl_ctx* c, int nwc) {
   FusedArgs a;
   a.seg = c->seg;
   a.tab = c->d_tab_block;
@@ -134,6 +135,13 @@ static cudaError_t run_fused(gwl_ctx* c, const double* theta, int64_t B, double*
   a.calQ = c->d_calQ_f;
   a.status = c->d_status;
   a.ffc = c->count_ff ? c->d_ffc : nullptr;
+  return a;
+}
+
+template <int NDET, bool CAL>
+static cudaError_t run_fused(gwl_ctx* c, const double* theta, int64_t B, double* lnl, int grid, int rows, int nwc,
+                             cudaStream_t st) {
+  const FusedArgs a = fused_args(c, nwc);
   const size_t smem = fused_bytes(c, nwc, rows);
   cudaError_t e = raise_smem_limit((const void*)k_fused<NDET, CAL>, c->device, smem);
   if (e != cudaSuccess) return e;

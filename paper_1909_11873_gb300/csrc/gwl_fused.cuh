@@ -73,6 +73,11 @@ struct FusedArgs {
   unsigned long long* ffc;  // diagnostic counter of float-float-delta blocks, or null
 };
 
+// The context's tables and window as such arguments, and a group's dynamic
+// shared memory (gwl_fused.cu).
+FusedArgs fused_args(const gwl_ctx* c, int nwc);
+size_t fused_bytes(const gwl_ctx* c, int nwc, int R);
+
 // Static shared memory of a group.
 template <int NDET, bool CAL>
 struct FusedSmem {
@@ -110,8 +115,9 @@ __device__ __forceinline__ void fused_stage(const FusedArgs& a, const FusedLayou
 }
 
 // The coefficients of rows 0 .. R-1, th(k, lane) giving parameter k of the
-// lane's row (called only for lanes below R): the arithmetic of
-// prologue_rows_ff, operation by operation.  Ends with a CTA barrier after
+// lane's row and out(lane) whether the row is refused whatever its parameters
+// (both called only for lanes below R): the arithmetic of prologue_rows_ff,
+// operation by operation.  Ends with a CTA barrier after
 // which pm, ncut, flag and maxcut are in place; K_d and the <h|h> terms
 // follow on warps 0 .. NDET-1 and the order of the rows on warp 7, without a
 // barrier after them.
@@ -119,8 +125,8 @@ __device__ __forceinline__ void fused_stage(const FusedArgs& a, const FusedLayou
 //   part 1: PN coefficients; amplitude   part 5: psi; ... of detector 1
 //   part 2: ln eta; K's phase angle      part 6: iota; ... of detector 2
 //   part 3: ra; cut and H_d there        part 7: checks, prefetch; ... of detector 3
-template <int NDET, bool CAL, class Th>
-__device__ __forceinline__ void fused_coeffs(const SegInfo& s, int R, FusedSmem<NDET, CAL>& sm, Th th) {
+template <int NDET, bool CAL, class Th, class Out>
+__device__ __forceinline__ void fused_coeffs(const SegInfo& s, int R, FusedSmem<NDET, CAL>& sm, Th th, Out out) {
   const int part = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const bool valid = lane < R;
   // ---- phase 1
@@ -145,7 +151,7 @@ __device__ __forceinline__ void fused_coeffs(const SegInfo& s, int R, FusedSmem<
     double x[11];
 #pragma unroll
     for (int k = 0; k < 11; ++k) x[k] = valid ? th(k) : 1.0;
-    const bool ok = valid && physical(x);
+    const bool ok = valid && physical(x) && !out(lane);
     sm.flag[lane] = ok ? 0 : 1;
     if (ok) prefetch_cut_H(s, x[0], x[1]);
   } else {  // parts 3-6: the sine and cosine of one angle
@@ -378,14 +384,19 @@ __device__ __forceinline__ void fused_row_sums(const FusedArgs& a, const FusedLa
 }
 
 // Bin sums of the group's rows (all threads; fused_coeffs before it): the
-// windows in groups of nwc, each staged (the first group's copy has been
-// started by the caller), its anchor records, its (row, window) items, its
-// windows' sums added to sm.acc in window order.  parity: the barrier's
-// phase.  crow(r): the calibration parameters of row r in global memory.
-// Returns false when a bounded wait ran out.
+// windows in groups of nwc, each staged unless it is in place, its anchor
+// records, its (row, window) items, its windows' sums added to sm.acc in
+// window order.  st: the group that shared memory holds.  crow(r): the
+// calibration parameters of row r.  Returns false when a bounded wait ran out.
+struct FusedStage {
+  int w0 = 0;             // first window of the group in shared memory
+  bool pending = true;    // its copy is in flight (the caller has started the first one)
+  uint32_t parity = 0;    // the barrier's phase
+};
+
 template <int NDET, bool CAL, class Crow>
 __device__ __forceinline__ bool fused_bins(const FusedArgs& a, const FusedLayout& L, float* dyn, int R,
-                                           FusedSmem<NDET, CAL>& sm, uint32_t& parity, bool& staged, Crow crow) {
+                                           FusedSmem<NDET, CAL>& sm, FusedStage& st, Crow crow) {
   constexpr int NS = FusedSmem<NDET, CAL>::NS, AR = anchor_rec_floats(NDET);
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const int gbins = a.CH * a.nwc, gblk = (a.CH + kAnchor - 1) / kAnchor * a.nwc;
@@ -394,15 +405,18 @@ __device__ __forceinline__ bool fused_bins(const FusedArgs& a, const FusedLayout
   for (int w0 = 0; (int64_t)w0 * a.CH < maxcut; w0 += a.nwc) {
     const int j0 = w0 * a.CH;
     const int top = maxcut - j0 < gbins ? maxcut - j0 : gbins;  // the longest row's bins in this group
-    if (!staged) {
-      if (t == 0) {
-        fence_proxy_async_smem();
-        fused_stage<NDET, CAL>(a, L, dyn, w0, &sm.bar);
+    if (st.w0 != w0 || st.pending) {
+      if (st.w0 != w0) {  // (a pending copy is always group 0's, the first one taken)
+        if (t == 0) {
+          fence_proxy_async_smem();
+          fused_stage<NDET, CAL>(a, L, dyn, w0, &sm.bar);
+        }
+        st.w0 = w0;
       }
+      if (!mbar_wait_bounded(&sm.bar, st.parity, a.status)) return false;
+      st.parity ^= 1u;
+      st.pending = false;
     }
-    if (!mbar_wait_bounded(&sm.bar, parity, a.status)) return false;
-    parity ^= 1u;
-    staged = false;
     // anchor records, blocks of a row on neighbouring threads
     const int nb = (top + kAnchor - 1) / kAnchor;
     for (int i = t; i < R * nb; i += 256) {

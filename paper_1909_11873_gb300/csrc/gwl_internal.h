@@ -139,7 +139,7 @@ cudaError_t launch_loglike(gwl_ctx* c, const double* theta, int64_t B, double* l
 cudaError_t launch_loglike_cleared(gwl_ctx* c, const double* theta, int64_t B, double* lnl, cudaStream_t st);
 int64_t work_needed(const gwl_ctx* c, int64_t B);
 // the one-kernel form (gwl_fused.cu): its launch shape for a batch (false: not used), launch
-bool fused_shape(const gwl_ctx* c, int64_t B, int* grid, int* rows, int* nwc);
+bool fused_shape(const gwl_ctx* c, int64_t B, int* grid, int* rows, int* nwc, size_t row_bytes = 0);
 bool fused_used(const gwl_ctx* c, int64_t B);
 cudaError_t launch_fused(gwl_ctx* c, const double* theta, int64_t B, double* lnl, int grid, int rows, int nwc,
                          cudaStream_t st);
@@ -165,6 +165,11 @@ cudaError_t launch_walk(gwl_ctx* c, const double* live_u, const double* live_lnl
                         uint64_t seed, int64_t n_chains, int walk_len, const double* chol, double* out_u,
                         double* out_lnl, int32_t* out_nacc, int32_t* out_start, double* pu, double* pth,
                         double* plnl, cudaStream_t st);
+// the one-kernel walk with its scalars by value and no scratch (false: not used for this shape)
+bool launch_walk_direct(gwl_ctx* c, const double* live_u, const double* live_lnl, int64_t K, int64_t worst,
+                        double lstar, uint64_t seed, uint64_t counter, int64_t n_chains, int walk_len, double scale,
+                        const double* chol, double* out_u, double* out_lnl, int32_t* out_nacc, int32_t* out_start,
+                        cudaStream_t st, cudaError_t* e);
 size_t walk_scalars_bytes();
 size_t gmc_scratch_doubles(int64_t n_chains, int D);
 void set_walk_scalars(void* host_buf, double lstar, double scale, int64_t worst, uint64_t counter);

@@ -20,7 +20,7 @@
 #include <cmath>
 #include <vector>
 
-#include "gwl_internal.h"
+#include "gwl_fused.cuh"
 
 namespace gwl {
 
@@ -174,6 +174,138 @@ __global__ void k_walk_step(PriorInfo pr, const WalkScalars* __restrict__ sc, co
   if (t0 >= n_chains) return;
   if (step > 1) walk_accept_row(sc, pr.D, t0, pu, plnl, cu, cl, cn);
   walk_propose_row(pr, sc, chol, seed, step, t0, cu, pu, ptheta);
+}
+
+// ---------------------------------------------------------------- the whole walk in one kernel
+// A chain depends on no other chain within a round, so a CTA takes a group of
+// chains through all steps of the walk by itself: proposal, the group's
+// likelihood (gwl_fused.cuh, whose table rows stay in shared memory from step
+// to step while one group of windows covers the rows) and accept/reject.  The
+// random numbers and their products L z do not depend on the chain's state:
+// warp 7 forms the next step's while the other warps sum bins.  FP64 warp
+// instructions hold the narrow FP64 pipe however few lanes are active, so the
+// FP64 work is packed over (chain, coordinate) pairs.
+//
+// What bounds it: per step the latency of the coefficients' float-pair chains
+// and of the bin sums of one row per warp.  Measured per step (us, 20-step
+// walks) against three dependent launches a step (proposal, prologue, bin
+// loop), at 1 / 250 / 1000 / 1900 chains: 4 s, 1 detector, 4-D 9.8 / 12.3 /
+// 12.5 / 14.5 against 29.7 / 35.5 / 41.4 / 47.8; 8 s, 3 detectors, 11-D
+// 11.2 / 15.4 / 19.8 / 22.0 against 41.7 / 57.2 / 59.9 / 62.0.
+template <int NDET, bool CAL>
+__global__ void __launch_bounds__(256, 2)
+    k_walk_fused(const __grid_constant__ FusedArgs a, const __grid_constant__ PriorInfo pr, WalkScalars val,
+                 const WalkScalars* __restrict__ sc, const double* __restrict__ live_u,
+                 const double* __restrict__ live_lnl, int64_t K, const double* __restrict__ chol, uint64_t seed,
+                 int64_t n_chains, int walk_len, int R, double* __restrict__ out_u, double* __restrict__ out_lnl,
+                 int32_t* __restrict__ out_nacc, int32_t* __restrict__ out_start) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  __shared__ FusedSmem<NDET, CAL> sm;
+  __shared__ double s_l[kFusedRows], s_cl[kFusedRows];
+  __shared__ int s_n[kFusedRows], s_out[kFusedRows], s_start[kFusedRows];
+  float* dyn = reinterpret_cast<float*>(smem_raw);
+  const FusedLayout L = fused_layout(NDET, CAL ? a.cal_row : 0, a.CH, a.nwc, R);
+  const int D = pr.D, np = (D + 1) / 2;
+  // per chain: the point, the proposal and its parameters, the normals and L z
+  double* s_cu = reinterpret_cast<double*>(dyn + ((L.total + 1) & ~1));
+  double* s_pu = s_cu + R * D;
+  double* s_th = s_pu + R * D;
+  double* s_dz = s_th + R * D;
+  double* s_z = s_dz + R * D;
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  cudaTriggerProgrammaticLaunchCompletion();
+  if (t == 0) {
+    mbar_init(&sm.bar, 1);
+    fence_mbar_init();
+    fused_stage<NDET, CAL>(a, L, dyn, 0, &sm.bar);
+  }
+  cudaGridDependencySynchronize();  // the live set, the step matrix and the scalars are written
+  const WalkScalars w = sc ? *sc : val;
+  const int64_t b0 = (int64_t)blockIdx.x * R;
+  const int n = n_chains - b0 < R ? (int)(n_chains - b0) : R;
+  // normals of step s and their products with the step matrix (one warp)
+  auto draw = [&](uint32_t s) {
+    for (int q = lane; q < n * np; q += 32) {
+      const int r = q / np, k = q - r * np;
+      const uint4 v = philox(make_uint4((uint32_t)(k >> 1), s, (uint32_t)(b0 + r), (uint32_t)w.counter),
+                             (uint32_t)seed, (uint32_t)(seed >> 32));
+      const uint32_t w0 = (k & 1) ? v.z : v.x, w1 = (k & 1) ? v.w : v.y;
+      const double u1 = ((double)w0 + 1.0) * 0x1p-32;
+      const double u2 = (double)w1 * 0x1p-32;
+      const double rr = sqrt(-2.0 * ::log(u1));
+      double sn, cs;
+      sincospi(2.0 * u2, &sn, &cs);
+      s_z[r * 2 * np + 2 * k] = rr * cs;
+      s_z[r * 2 * np + 2 * k + 1] = rr * sn;
+    }
+    __syncwarp();
+    for (int q = lane; q < n * D; q += 32) {
+      const int i = q / n, r = q - i * n;
+      const double* z = s_z + r * 2 * np;
+      double dz = 0.0;
+      for (int k = 0; k <= i; ++k) dz += chol[i * D + k] * z[k];
+      s_dz[r * D + i] = dz;
+    }
+  };
+  // the chains' start points
+  if (t < n) {
+    const uint4 v = philox(make_uint4(0u, 0u, (uint32_t)(b0 + t), (uint32_t)w.counter), (uint32_t)seed,
+                           (uint32_t)(seed >> 32));
+    const int64_t idx = (int64_t)(((uint64_t)v.x * (uint64_t)(K - 1)) >> 32);
+    const int64_t st = idx < w.worst ? idx : idx + 1;
+    s_start[t] = (int)st;
+    s_cl[t] = live_lnl[st];
+    s_n[t] = 0;
+    s_out[t] = 0;
+    s_l[t] = 0.0;
+  }
+  if (warp == 7 && walk_len > 0) draw(1);
+  __syncthreads();
+  for (int q = t; q < n * D; q += 256) {
+    const int i = q / n, r = q - i * n;
+    s_cu[r * D + i] = live_u[(int64_t)s_start[r] * D + i];
+  }
+  FusedStage stg;
+  for (int s = 1; s <= walk_len; ++s) {
+    // the last step's accept (a thread keeps its pairs from step to step), this step's proposal
+    for (int q = t; q < n * D; q += 256) {
+      const int i = q / n, r = q - i * n, e = r * D + i;
+      if (s > 1 && s_l[r] >= w.lstar) s_cu[e] = s_pu[e];
+      double x = s_cu[e] + w.scale * s_dz[e];
+      if (coord_periodic(pr, i)) x -= floor(x);
+      else if (x < 0.0 || x > 1.0) s_out[r] = 1;
+      s_pu[e] = x;
+      s_th[e] = coord_map(pr, i, x);
+    }
+    __syncthreads();
+    fused_coeffs<NDET, CAL>(
+        a.seg, n, sm,
+        [&](int k) { return a.seg.param_pos[k] >= 0 ? s_th[lane * D + a.seg.param_pos[k]] : a.seg.fixed[k]; },
+        [&](int r) { return s_out[r] != 0; });
+    if (warp == 7 && s < walk_len) draw((uint32_t)s + 1);
+    if (!fused_bins<NDET, CAL>(a, L, dyn, n, sm, stg, [&](int r) { return s_th + r * D + a.cal_par; })) return;
+    __syncthreads();
+    if (t < n) {
+      const double l = fused_combine<NDET, CAL>(sm, t);
+      s_l[t] = l;
+      s_out[t] = 0;
+      if (l >= w.lstar) {  // rows outside the cube give -inf
+        s_cl[t] = l;
+        s_n[t] += 1;
+      }
+    }
+    __syncthreads();
+  }
+  if (stg.pending) mbar_wait_bounded(&sm.bar, stg.parity, a.status);  // no copy may outlive the CTA
+  for (int q = t; q < n * D; q += 256) {
+    const int i = q / n, r = q - i * n, e = r * D + i;
+    out_u[(b0 + r) * D + i] = walk_len > 0 && s_l[r] >= w.lstar ? s_pu[e] : s_cu[e];
+  }
+  if (t < n) {
+    out_lnl[b0 + t] = s_cl[t];
+    out_nacc[b0 + t] = s_n[t];
+    if (out_start) out_start[b0 + t] = s_start[t];
+  }
 }
 
 // ---------------------------------------------------------------- Galilean walk
@@ -909,6 +1041,72 @@ static cudaError_t launch_gmc(gwl_ctx* c, const double* live_u, const double* li
   return e;
 }
 
+// Shared memory per chain of k_walk_fused.
+static size_t walk_row_bytes(const gwl_ctx* c) {
+  const size_t D = (size_t)theta_stride(c);
+  return sizeof(double) * (5 * D + 1);
+}
+
+static bool walk_fused_shape(const gwl_ctx* c, int64_t n_chains, int* grid, int* rows, int* nwc) {
+  return c->walk_kind == GWL_WALK_RANDOM && !lanes_seg(c, n_chains) &&
+         fused_shape(c, n_chains, grid, rows, nwc, walk_row_bytes(c));
+}
+
+template <int NDET, bool CAL>
+static cudaError_t run_walk_fused(gwl_ctx* c, const WalkScalars& val, const WalkScalars* sc, const double* live_u,
+                                  const double* live_lnl, int64_t K, uint64_t seed, int64_t n_chains, int walk_len,
+                                  const double* chol, double* out_u, double* out_lnl, int32_t* out_nacc,
+                                  int32_t* out_start, int grid, int rows, int nwc, cudaStream_t st) {
+  const FusedArgs a = fused_args(c, nwc);
+  const size_t smem = fused_bytes(c, nwc, rows) + 8 + (size_t)rows * walk_row_bytes(c);
+  cudaError_t e = raise_smem_limit((const void*)k_walk_fused<NDET, CAL>, c->device, smem);
+  if (e != cudaSuccess) return e;
+  ProfScope ps(c, GWL_KERNEL_WALK, st);
+  e = launch_pdl(k_walk_fused<NDET, CAL>, dim3(grid), dim3(256), smem, st, a, prior_info(c), val, sc, live_u, live_lnl,
+                 K, chol, seed, n_chains, walk_len, rows, out_u, out_lnl, out_nacc, out_start);
+  c->launches++;
+  return e;
+}
+
+static cudaError_t launch_walk_fused(gwl_ctx* c, const WalkScalars& val, const WalkScalars* sc, const double* live_u,
+                                     const double* live_lnl, int64_t K, uint64_t seed, int64_t n_chains, int walk_len,
+                                     const double* chol, double* out_u, double* out_lnl, int32_t* out_nacc,
+                                     int32_t* out_start, int grid, int rows, int nwc, cudaStream_t st) {
+  auto go = [&](auto nd, auto cal) {
+    return run_walk_fused<decltype(nd)::value, decltype(cal)::value>(c, val, sc, live_u, live_lnl, K, seed, n_chains,
+                                                                     walk_len, chol, out_u, out_lnl, out_nacc,
+                                                                     out_start, grid, rows, nwc, st);
+  };
+  auto pick = [&](auto nd) {
+    return c->n_cal_nodes > 0 ? go(nd, std::true_type()) : go(nd, std::false_type());
+  };
+  switch (c->n_det) {
+    case 1: return pick(std::integral_constant<int, 1>());
+    case 2: return pick(std::integral_constant<int, 2>());
+    case 3: return pick(std::integral_constant<int, 3>());
+    default: return pick(std::integral_constant<int, 4>());
+  }
+}
+
+// ns_replace's walk in the one-kernel form, its scalars passed by value; false
+// where the separate kernels run (the line is fused_shape's: the walk's step is
+// that likelihood).
+bool launch_walk_direct(gwl_ctx* c, const double* live_u, const double* live_lnl, int64_t K, int64_t worst,
+                        double lstar, uint64_t seed, uint64_t counter, int64_t n_chains, int walk_len, double scale,
+                        const double* chol, double* out_u, double* out_lnl, int32_t* out_nacc, int32_t* out_start,
+                        cudaStream_t st, cudaError_t* e) {
+  int grid, rows, nwc;
+  if (!walk_fused_shape(c, n_chains, &grid, &rows, &nwc)) return false;
+  WalkScalars v;
+  v.lstar = lstar;
+  v.scale = scale;
+  v.worst = worst;
+  v.counter = counter;
+  *e = launch_walk_fused(c, v, nullptr, live_u, live_lnl, K, seed, n_chains, walk_len, chol, out_u, out_lnl, out_nacc,
+                         out_start, grid, rows, nwc, st);
+  return true;
+}
+
 size_t gmc_scratch_doubles(int64_t n_chains, int D) { return (size_t)n_chains * (5 * D + 2); }
 
 cudaError_t launch_walk(gwl_ctx* c, const double* live_u, const double* live_lnl, int64_t K, const void* scalars,
@@ -919,6 +1117,10 @@ cudaError_t launch_walk(gwl_ctx* c, const double* live_u, const double* live_lnl
   if (c->walk_kind == GWL_WALK_GALILEAN)
     return launch_gmc(c, live_u, live_lnl, K, sc, seed, n_chains, walk_len, chol, out_u, out_lnl, out_nacc,
                       out_start, pu, pth, plnl, st);
+  int grid, rows, nwc;
+  if (walk_fused_shape(c, n_chains, &grid, &rows, &nwc))
+    return launch_walk_fused(c, WalkScalars(), sc, live_u, live_lnl, K, seed, n_chains, walk_len, chol, out_u, out_lnl,
+                             out_nacc, out_start, grid, rows, nwc, st);
   const int D = (int)theta_stride(c);
   const unsigned nb = (unsigned)((n_chains + 127) / 128);
   const PriorInfo pr = prior_info(c);

@@ -82,3 +82,43 @@ def test_one_kernel_matches_separate_kernels(n_det, T, source, fcut, nodes):
     assert torch.equal(many.reshape(9, n), one[None].expand(9, n))
     ctx.gwl_sync()
     ctx.close()
+
+
+@pytest.mark.parametrize("n_det,source,nodes,walk", [(1, "bbh", 0, 6), (3, "bbh", 0, 5), (3, "bbh", 10, 3), (2, "bbh", 0, 0)])
+def test_one_kernel_walk_matches_separate_kernels(n_det, source, nodes, walk):
+    """Chain b's random numbers depend on b alone, so the first chains of a long batch (separate kernels, with the
+    largest windows) are those of a short one (one kernel): same points, acceptances and, rows having one window,
+    the same log-likelihoods bit for bit."""
+    from paper_1909_11873_gb300 import gwl as g
+
+    cfg = dict(n_det=n_det, T=8.0, f_low=20.0, f_high=1024.0, noise=True, source=source, gmst=1.7)
+    ev = custom_event(cfg, 5)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    ctx = g.Context.from_event(ev, g.GWL_MIXED)
+    if nodes:
+        ctx.gwl_set_calibration(I.cal_node_freqs(20.0, 1024.0, nodes))
+    ctx.gwl_set_tuning(window=1440 if nodes else 1696 if n_det == 3 else 2432, bin_kernel=g.GWL_BINS_WARP)
+    D, K = ctx.theta_stride, 64
+    rng = np.random.default_rng(8)
+    u = torch.from_numpy(rng.uniform(0.0, 1.0, (K, D))).cuda()
+    l = torch.from_numpy(np.sort(rng.uniform(-50.0, 0.0, K))).cuda()
+    A = 0.1 * np.tril(rng.standard_normal((D, D))) / np.sqrt(D) + 0.05 * np.eye(D)
+    chol = torch.from_numpy(A).cuda()
+
+    def chains(n):
+        out = [torch.empty((n, D), dtype=torch.float64, device="cuda"), torch.empty(n, dtype=torch.float64, device="cuda"),
+               torch.empty(n, dtype=torch.int32, device="cuda"), torch.empty(n, dtype=torch.int32, device="cuda")]
+        k = ctx.launch_count()
+        ctx.ns_replace(u, l, 0, -200.0, 7, 3, n, walk, 0.5, chol, *out)
+        torch.cuda.synchronize()
+        return out, ctx.launch_count() - k
+
+    ref, k = chains(8 * sms + 9)
+    assert walk == 0 or (k > 1 and int((ref[2] > 0).sum()) > 0)
+    for n in (1, 9, sms + 1, 8 * sms):
+        got, k = chains(n)
+        assert k == 1
+        for a, b in zip(got, ref):
+            assert torch.equal(a, b[:n])
+    ctx.gwl_sync()
+    ctx.close()
