@@ -230,22 +230,34 @@ __device__ __forceinline__ bool physical(const double th[11]) {
   return ok;
 }
 
+// The same test on the doubles' bits: FP64 compares would each wait for the
+// narrow FP64 pipe.
+__device__ __forceinline__ bool physical_bits(const double th[11]) {
+  auto bits = [&](int k) { return __double_as_longlong(th[k]); };
+  bool ok = bits(1) > 0 && bits(1) <= 0x3FF0000000000000ll && bits(0) > 0 && bits(4) > 0;
+#pragma unroll
+  for (int k = 0; k < 11; ++k) ok = ok && ((bits(k) >> 52) & 0x7FF) != 0x7FF;
+  return ok;
+}
+
 // Pull the lines of H_d[j-1 .. j+1] (all detectors) into L2, j an FP32
 // estimate of the last bin at or below the cut frequency 1 / (6^{3/2} pi M
 // T_sun): the exact count that is read later differs from it by at most a bin.
 __device__ __forceinline__ void prefetch_cut_H(const SegInfo& s, double mc, double q) {
-  int64_t j = s.M - 1;
+  const int last = (int)s.M - 1;
+  int j = last;
   if (s.fcut_mode == 0) {
     const float qf = (float)q, opq = 1.0f + qf;
-    const float M = (float)mc * __powf(qf / (opq * opq), -0.6f);
-    const float fc = 1.0f / ((float)(kSix32 * kPi * kTsun) * M);
-    const float x = fminf(fmaxf(floorf((fc - (float)s.f0) * (float)s.inv_df), 0.0f), (float)(s.M - 1));
-    j = (int64_t)x;
+    const float M = (float)mc * __powf(__fdividef(qf, opq * opq), -0.6f);
+    const float fc = __fdividef(1.0f, (float)(kSix32 * kPi * kTsun) * M);
+    j = (int)fminf(fmaxf((fc - (float)s.f0) * (float)s.inv_df, 0.0f), (float)last);
   }
-  const int64_t a = j > 0 ? j - 1 : 0, b = j + 1 < s.M ? j + 1 : s.M - 1;
-  for (int d = 0; d < s.n_det; ++d) {
-    asm volatile("prefetch.global.L2 [%0];" ::"l"(s.H + d * s.M + a));
-    asm volatile("prefetch.global.L2 [%0];" ::"l"(s.H + d * s.M + b));
+  const double* h = s.H + (j > 0 ? j - 1 : 0);
+  const int ahead = j + 1 < last ? 2 : 0;
+#pragma unroll 1
+  for (int d = 0; d < s.n_det; ++d, h += s.M) {
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(h));
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(h + ahead));
   }
 }
 
@@ -254,6 +266,16 @@ __device__ __forceinline__ void prefetch_cut_H(const SegInfo& s, double mc, doub
 // x = (fc - f0) / df is more than 1e-7 from an integer the count follows from
 // x alone; otherwise it is settled against the stored FP64 frequencies.  Either
 // way the decision matches a per-bin comparison exactly.
+static __device__ __noinline__ int count_bins_search(const double* __restrict__ freqs, int64_t M, double x, double fc) {
+  if (!(fc >= freqs[0])) return 0;
+  if (fc >= freqs[M - 1]) return (int)M;
+  int64_t j = (int64_t)floor(x);
+  if (j < 0) j = 0;
+  if (j > M - 1) j = M - 1;
+  while (j + 1 < M && freqs[j + 1] <= fc) ++j;
+  while (j >= 0 && freqs[j] > fc) --j;
+  return (int)(j + 1);
+}
 __device__ __forceinline__ int count_bins_le(const SegInfo& s, double fc) {
   const double x = (fc - s.f0) * s.inv_df;
   const double jf = floor(x), r = x - jf;
@@ -262,14 +284,7 @@ __device__ __forceinline__ int count_bins_le(const SegInfo& s, double fc) {
     if (jf >= (double)(s.M - 1)) return (int)s.M;
     return (int)jf + 1;
   }
-  if (!(fc >= s.freqs[0])) return 0;
-  if (fc >= s.freqs[s.M - 1]) return (int)s.M;
-  int64_t j = (int64_t)floor((fc - s.f0) / s.df);
-  if (j < 0) j = 0;
-  if (j > s.M - 1) j = s.M - 1;
-  while (j + 1 < s.M && s.freqs[j + 1] <= fc) ++j;
-  while (j >= 0 && s.freqs[j] > fc) --j;
-  return (int)(j + 1);
+  return count_bins_search(s.freqs, s.M, x, fc);
 }
 
 // ------------------------------------------------------------- model formulas

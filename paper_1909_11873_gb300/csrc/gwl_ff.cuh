@@ -38,7 +38,10 @@ __device__ __forceinline__ FF ff(float x) { return FF{x, 0.0f}; }
 // by the 2^23 bias trick, then scaled by a power of two): hi + lo = x to about
 // 2^-48.  Zero and subnormal doubles give zero; |x| outside [2^-70, 2^100]
 // (not met by the prologues' inputs) takes the conversion instructions.
-__device__ __forceinline__ FF ff_from(double x) {
+// Out of line, as the division and the elementary functions below: the
+// prologues call each of these many times, once per launch or walk step, and
+// are bound by the instruction cache rather than by the calls.
+static __device__ __noinline__ FF ff_from(double x) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
   const int e = (int)((b >> 52) & 0x7FF);
   if (e == 0) return FF{0.0f, 0.0f};
@@ -87,11 +90,12 @@ __device__ __forceinline__ FF operator*(const FF& a, const FF& b) {
   return ff_norm(p, __fmaf_rn(a.hi, b.lo, __fmaf_rn(a.lo, b.hi, e)));
 }
 // a / b: the FP32 quotient of the high parts, corrected by the quotient of the remainder.
-__device__ __forceinline__ FF operator/(const FF& a, const FF& b) {
+static __device__ __noinline__ FF ff_div(FF a, FF b) {
   const float q1 = __fdiv_rn(a.hi, b.hi);
   const FF r = a - b * ff(q1);
   return ff_norm(q1, __fdiv_rn(r.hi, b.hi));
 }
+__device__ __forceinline__ FF operator/(const FF& a, const FF& b) { return ff_div(a, b); }
 __device__ __forceinline__ FF operator+(const FF& a, double c) { return a + ffc(c); }
 __device__ __forceinline__ FF operator+(double c, const FF& a) { return a + ffc(c); }
 __device__ __forceinline__ FF operator-(const FF& a, double c) { return a + ffc(-c); }
@@ -139,7 +143,7 @@ __device__ __forceinline__ FF ff_reduce(const FF& x, float k, float c1, float c2
 // orders whose FP32 rounding would show at the float-pair level are summed
 // as float pairs: the high orders of a Taylor series are small enough for
 // plain FP32, which takes about a fifth of the instructions.
-static __device__ __noinline__ FF ff_exp(const FF& x) {
+static __device__ __noinline__ FF ff_exp(FF x) {
   const float k = nearest_int(__fmul_rn(x.hi, 1.44269504088896341f));
   const FF r = ff_reduce(x, k, 0x1.62e000p-1f, 0x1.0bfbe8p-15f, 0x1.cf79acp-40f);  // ln 2
   // orders 8..13 in FP32 (r^8 / 8! < 6e-9, so their rounding stays below 1e-15 relative)
@@ -154,13 +158,16 @@ static __device__ __noinline__ FF ff_exp(const FF& x) {
   return FF{__fmul_rn(p.hi, s), __fmul_rn(p.lo, s)};
 }
 
-static __device__ __noinline__ FF ff_log(const FF& x) {
+static __device__ __noinline__ FF ff_log(FF x) {
   const float y0 = logf(x.hi);
   const FF t = x * ff_exp(ff(-y0)) - 1.0;
   return ff(y0) + (t - t * t * 0.5);
 }
 
-static __device__ __noinline__ void ff_sincos(const FF& x, FF* sn, FF* cs) {
+struct FFPair {
+  FF s, c;
+};
+static __device__ __noinline__ FFPair ff_sincos2(FF x) {
   const float k = nearest_int(__fmul_rn(x.hi, 0.636619772367581343f));
   const FF r = ff_reduce(x, k, 0x1.920000p+0f, 0x1.fb5444p-12f, 0x1.68c234p-39f);  // pi / 2
   const FF r2 = r * r;
@@ -179,12 +186,19 @@ static __device__ __noinline__ void ff_sincos(const FF& x, FF* sn, FF* cs) {
     pc = pc * r2 + kCosCoef[n];
   }
   const FF s = r * ps, c = pc;
-  switch ((int)k & 3) {
-    case 0: *sn = s; *cs = c; break;
-    case 1: *sn = c; *cs = -s; break;
-    case 2: *sn = -s; *cs = -c; break;
-    default: *sn = -c; *cs = s; break;
-  }
+  // quadrants 1 and 3 swap them; the sine is negative in 2 and 3, the cosine in 1 and 2
+  const int q = (int)k & 3;
+  FFPair o;
+  o.s = (q & 1) ? c : s;
+  o.c = (q & 1) ? s : c;
+  if (q & 2) o.s = -o.s;
+  if ((q + 1) & 2) o.c = -o.c;
+  return o;
+}
+__device__ __forceinline__ void ff_sincos(const FF& x, FF* sn, FF* cs) {
+  const FFPair o = ff_sincos2(x);
+  *sn = o.s;
+  *cs = o.c;
 }
 
 // Overloads used by the templated model code (gwl_device.cuh).

@@ -16,13 +16,15 @@ template <int NDET, bool CAL>
 __global__ void __launch_bounds__(256, 2) k_fused(const __grid_constant__ FusedArgs a, const double* __restrict__ theta,
                                                   int64_t B, int R, double* __restrict__ lnl) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  __shared__ FusedSmem<NDET, CAL> sm;
+  constexpr int NW = 8;
+  __shared__ FusedSmem<NDET, CAL, NW> sm;
   float* dyn = reinterpret_cast<float*>(smem_raw);
   const FusedLayout L = fused_layout(NDET, CAL ? a.cal_row : 0, a.CH, a.nwc, R);
   // the next call's kernel may become resident as CTAs leave; it stages its
   // table rows and waits for this grid before it reads anything else
   cudaTriggerProgrammaticLaunchCompletion();
   if (threadIdx.x == 0) {
+    sm.fail = 0;
     mbar_init(&sm.bar, 1);
     fence_mbar_init();
     fused_stage<NDET, CAL>(a, L, dyn, 0, &sm.bar);
@@ -32,16 +34,16 @@ __global__ void __launch_bounds__(256, 2) k_fused(const __grid_constant__ FusedA
   const int n = B - row0 < R ? (int)(B - row0) : R;
   const int lane = threadIdx.x & 31;
   const double* row = theta + (row0 + lane) * a.seg.stride;
-  fused_coeffs<NDET, CAL>(a.seg, n, sm,
+  fused_coeffs<NDET, CAL, NW>(a.seg, n, sm,
                           [&](int k) { return a.seg.param_pos[k] >= 0 ? row[a.seg.param_pos[k]] : a.seg.fixed[k]; },
                           [](int) { return false; });
   FusedStage st;
-  if (!fused_bins<NDET, CAL>(a, L, dyn, n, sm, st,
+  if (!fused_bins<NDET, CAL, NW>(a, L, dyn, n, sm, st,
                              [&](int r) { return theta + (row0 + r) * a.seg.stride + a.cal_par; }))
     return;
   if (st.pending) mbar_wait_bounded(&sm.bar, st.parity, a.status);  // no copy may outlive the CTA
   __syncthreads();
-  if (threadIdx.x < n) lnl[row0 + threadIdx.x] = fused_combine<NDET, CAL>(sm, threadIdx.x);
+  if (threadIdx.x < n) lnl[row0 + threadIdx.x] = fused_combine<NDET, CAL, NW>(a, L, dyn, sm, threadIdx.x);
 }
 
 // ---------------------------------------------------------------- host side
@@ -51,10 +53,24 @@ size_t fused_bytes(const gwl_ctx* c, int nwc, int R) {
   return sizeof(float) * (size_t)fused_layout(c->n_det, c->n_cal_nodes ? c->row_cal_f : 0, lnl_window(c), nwc, R).total;
 }
 
+int fused_window_count(const gwl_ctx* c) {
+  const int CH = lnl_window(c);
+  return (int)((c->M + CH - 1) / CH);
+}
+
+// Windows of R rows' groups that fit `room` bytes of dynamic shared memory (0: none).
+int fused_windows(const gwl_ctx* c, int R, size_t room) {
+  const int nw = fused_window_count(c);
+  if ((lnl_window(c) % kAnchor && nw > 1) || fused_bytes(c, 1, R) > room) return 0;
+  int w = 1;
+  while (w < nw && fused_bytes(c, w + 1, R) <= room) ++w;
+  return w;
+}
+
 // Static shared memory of the kernel.
 template <int NDET>
 static size_t static_of(bool cal) {
-  return cal ? sizeof(FusedSmem<NDET, true>) : sizeof(FusedSmem<NDET, false>);
+  return cal ? sizeof(FusedSmem<NDET, true, 8>) : sizeof(FusedSmem<NDET, false, 8>);
 }
 static size_t fused_static(const gwl_ctx* c) {
   const bool cal = c->n_cal_nodes > 0;
@@ -88,24 +104,16 @@ constexpr size_t kSmemPerSm = 228 * 1024;  // 1 KB of it goes to each resident C
 //     327 / 1014 / 1388 / 2479 against 248 / 895 / 1529 / 3109
 // so segments of up to 32 windows take it at any batch, longer ones where the
 // batch gives every warp of two CTAs per SM a row.
-// row_bytes: shared memory that a caller's kernel needs besides, per row.
-bool fused_shape(const gwl_ctx* c, int64_t B, int* grid, int* rows, int* nwc, size_t row_bytes) {
+bool fused_shape(const gwl_ctx* c, int64_t B, int* grid, int* rows, int* nwc) {
   if (c->opt.precision != GWL_MIXED || B <= 0) return false;
-  const int CH = lnl_window(c);
-  const int64_t nw = (c->M + CH - 1) / CH;
-  if (CH % kAnchor && nw > 1) return false;
-  if (nw > 32 && B <= 8 * (int64_t)c->num_sms) return false;
+  if (fused_window_count(c) > 32 && B <= 8 * (int64_t)c->num_sms) return false;
   const int per_sm = B <= 8 * (int64_t)c->num_sms ? 1 : 2;
   const int64_t slots = per_sm * (int64_t)c->num_sms;
   const int64_t waves = (B + slots * kFusedRows - 1) / (slots * kFusedRows);
   const int64_t R = (B + slots * waves - 1) / (slots * waves);
   const int64_t G = (B + R - 1) / R;
-  const size_t room = (per_sm == 1 ? 227 * 1024 : kSmemPerSm / 2 - 1024) - fused_static(c) - 1024 -
-                      (size_t)R * row_bytes;
-  if ((size_t)R * row_bytes > 64 * 1024) return false;
-  int w = 1;
-  if (fused_bytes(c, 1, (int)R) > room) return false;
-  while (w < nw && fused_bytes(c, w + 1, (int)R) <= room) ++w;
+  const int w = fused_windows(c, (int)R, (per_sm == 1 ? 227 * 1024 : kSmemPerSm / 2 - 1024) - fused_static(c) - 128);
+  if (w == 0) return false;
   *grid = (int)G;
   *rows = (int)R;
   *nwc = w;

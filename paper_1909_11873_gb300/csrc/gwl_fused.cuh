@@ -78,22 +78,30 @@ struct FusedArgs {
 FusedArgs fused_args(const gwl_ctx* c, int nwc);
 size_t fused_bytes(const gwl_ctx* c, int nwc, int R);
 
+// The group's warps are the first NW of the CTA's (8 or 16; the coefficients
+// use eight, the bin sums all); other warps of the CTA take no part, so the
+// group has a barrier of its own.
+template <int NW>
+__device__ __forceinline__ void group_sync() {
+  asm volatile("bar.sync 1, %0;" ::"n"(32 * NW) : "memory");
+}
+
 // Static shared memory of a group.
-template <int NDET, bool CAL>
+template <int NDET, bool CAL, int NW>
 struct FusedSmem {
   static constexpr int NS = (CAL ? 3 : 2) * NDET;  // sums per row
   FF lmc[kFusedRows], leta[kFusedRows], eta[kFusedRows], amp[kFusedRows];
   FF phi[6][kFusedRows];
   FF sky[4][kFusedRows], ori[3][kFusedRows];
   FF P[2 * NDET][kFusedRows], ang[2][kFusedRows], hterm[NDET][kFusedRows];
-  double Hc[NDET][kFusedRows], Kr[NDET][kFusedRows], Ki[NDET][kFusedRows];
-  double acc[NS][kFusedRows];
+  double Kr[NDET][kFusedRows], Ki[NDET][kFusedRows];
+  double acc[NS][kFusedRows];  // sums over the window groups before the last one
   PropMixed pm[kFusedRows];
   int ncut[kFusedRows], flag[kFusedRows];
   int order[kFusedRows];  // rows by descending cut
-  int next, maxcut;
+  int next, maxcut, fail;
   alignas(8) uint64_t bar;
-  alignas(16) float4 nodes[CAL ? 8 * NDET * kMaxCalNodes : 1];
+  alignas(16) float4 nodes[CAL ? NW * NDET * kMaxCalNodes : 1];
 };
 
 // One thread: the table rows (and anchor and calibration rows) of windows
@@ -114,68 +122,105 @@ __device__ __forceinline__ void fused_stage(const FusedArgs& a, const FusedLayou
   if constexpr (CAL) bulk_g2s(dyn + L.cal, a.cal + j0 * a.cal_row, cbytes, bar);
 }
 
+// The quadratics in eta of the PN coefficients (pn_coeffs in gwl_device.cuh),
+// a + b eta + c eta^2, summed in that order: of p4, gamma, p6, and the three of
+// p7 (its non-spinning part, its chi_s and its delta chi_a factors).
+constexpr int kPnP4 = 0, kPnGam = 1, kPnP6 = 2, kPnP7 = 3, kPnP7s = 4, kPnP7a = 5;
+static __constant__ FF kPnQuad[6][3] = {
+    {ffc(3058673.0 / 1016064.0), ffc(5429.0 / 1008.0), ffc(617.0 / 144.0)},
+    {ffc(732985.0 / 2268.0), ffc(-(24260.0 / 81.0)), ffc(-(340.0 / 9.0))},
+    {ffc(11583231236531.0 / 4694215680.0 - (640.0 / 3.0) * kPi * kPi - (6848.0 / 21.0) * kGammaE),
+     ffc(-15737765635.0 / 3048192.0 + (2255.0 / 12.0) * kPi * kPi), ffc(76055.0 / 1728.0)},
+    {ffc(77096675.0 / 254016.0), ffc(378515.0 / 1512.0), ffc(-(74045.0 / 756.0))},
+    {ffc(-25150083775.0 / 3048192.0), ffc(10566655595.0 / 762048.0), ffc(-(1042165.0 / 3024.0))},
+    {ffc(-25150083775.0 / 3048192.0), ffc(26804935.0 / 6048.0), ffc(-(1985.0 / 48.0))}};
+static __device__ __noinline__ FF pn_quad(FF eta, FF eta2, int k) {
+  return (kPnQuad[k][0] + eta * kPnQuad[k][1]) + eta2 * kPnQuad[k][2];
+}
+// eta = q / (1 + q)^2 and delta = (1 - q) / (1 + q).
+static __device__ __noinline__ FF pn_eta(FF q) {
+  const FF opq = q + 1.0;
+  return q / (opq * opq);
+}
+static __device__ __noinline__ FF pn_delta(FF q) { return (1.0 - q) / (q + 1.0); }
+
 // The coefficients of rows 0 .. R-1, th(k, lane) giving parameter k of the
 // lane's row and out(lane) whether the row is refused whatever its parameters
 // (both called only for lanes below R): the arithmetic of prologue_rows_ff,
-// operation by operation.  Ends with a CTA barrier after
-// which pm, ncut, flag and maxcut are in place; K_d and the <h|h> terms
-// follow on warps 0 .. NDET-1 and the order of the rows on warp 7, without a
-// barrier after them.
-//   part 0: ln(pi Mc T_sun); c_m         part 4: dec; response and delay of detector 0
-//   part 1: PN coefficients; amplitude   part 5: psi; ... of detector 1
-//   part 2: ln eta; K's phase angle      part 6: iota; ... of detector 2
-//   part 3: ra; cut and H_d there        part 7: checks, prefetch; ... of detector 3
-template <int NDET, bool CAL, class Th, class Out>
-__device__ __forceinline__ void fused_coeffs(const SegInfo& s, int R, FusedSmem<NDET, CAL>& sm, Th th, Out out) {
+// operation by operation, on the first eight warps, no chain longer than it
+// must be.  K_d and the <h|h> terms are left to fused_amplitudes.  Ends with a
+// barrier after which pm, ncut, flag and maxcut are in place; warp 7 then sorts
+// the rows, without a barrier after it.
+//   part 0: ln(pi Mc T_sun); c_m           part 4: dec, H prefetch; response and delay of detector 0
+//   part 1: PN orders 2-4; amplitude       part 5: psi, PN order 5; ... of detector 1
+//   part 2: ln eta; K's phase angle        part 6: iota, checks; ... of detector 2
+//   part 3: ra, PN order 6; cut            part 7: PN order 7; ... of detector 3
+// What bounds it is the fetching of its code (each warp runs straight-line code
+// once per launch or step), so the elementary functions, the division and the
+// quadratics are out of line.
+template <int NDET, bool CAL, int NW, class Th, class Out>
+__device__ __forceinline__ void fused_coeffs(const SegInfo& s, int R, FusedSmem<NDET, CAL, NW>& sm, Th th, Out out) {
   const int part = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const bool valid = lane < R;
   // ---- phase 1
   if (part == 0) {
     const double mc = valid ? th(0) : 10.0;
     sm.lmc[lane] = log(ff_from(mc) * (kPi * kTsun));
-  } else if (part == 1) {
-    const double q = valid ? th(1) : 0.5, x1 = valid ? th(2) : 0.0, x2 = valid ? th(3) : 0.0;
-    const PNCoeffs<FF> P = pn_coeffs(ff_from(q), ff_from(x1), ff_from(x2));
-    sm.eta[lane] = P.eta;
-    sm.phi[0][lane] = P.p2;
-    sm.phi[1][lane] = P.p3;
-    sm.phi[2][lane] = P.p4;
-    sm.phi[3][lane] = P.p5c;
-    sm.phi[4][lane] = P.p6c;
-    sm.phi[5][lane] = P.p7;
   } else if (part == 2) {
-    const FF q = ff_from(valid ? th(1) : 0.5);
-    const FF opq = q + 1.0;
-    sm.leta[lane] = log(q / (opq * opq));
-  } else if (part == 7) {
-    double x[11];
+    const FF eta = pn_eta(ff_from(valid ? th(1) : 0.5));
+    sm.eta[lane] = eta;
+    sm.leta[lane] = log(eta);
+    sm.order[lane] = lane;
+  } else if (part < 8) {
+    if (part >= 3 && part < 7) {  // the sine and cosine of one angle
+      const double x = valid ? (part == 3 ? th(7) : part == 4 ? th(8) : part == 5 ? th(6) : th(5)) : 0.0;
+      FF f = ff_from(x);
+      if (part == 3) f = f - s.gmst;
+      FF sn, cs;
+      sincos(f, &sn, &cs);
+      FF* o = part == 3 ? &sm.sky[0][lane] : part == 4 ? &sm.sky[2][lane] : part == 5 ? &sm.ori[0][lane] : nullptr;
+      if (part < 6) {
+        o[0] = sn;
+        o[kFusedRows] = cs;
+      } else {
+        sm.ori[2][lane] = cs;
+      }
+    }
+    if (part == 4) {
+      if (valid) prefetch_cut_H(s, th(0), th(1));
+    } else if (part == 6) {
+      double x[11];
 #pragma unroll
-    for (int k = 0; k < 11; ++k) x[k] = valid ? th(k) : 1.0;
-    const bool ok = valid && physical(x) && !out(lane);
-    sm.flag[lane] = ok ? 0 : 1;
-    if (ok) prefetch_cut_H(s, x[0], x[1]);
-  } else {  // parts 3-6: the sine and cosine of one angle
-    const double x = valid ? (part == 3 ? th(7) : part == 4 ? th(8) : part == 5 ? th(6) : th(5)) : 0.0;
-    FF f = ff_from(x);
-    if (part == 3) f = f - s.gmst;
-    FF sn, cs;
-    sincos(f, &sn, &cs);
-    if (part == 3) {
-      sm.sky[0][lane] = sn;
-      sm.sky[1][lane] = cs;
-    } else if (part == 4) {
-      sm.sky[2][lane] = sn;
-      sm.sky[3][lane] = cs;
-    } else if (part == 5) {
-      sm.ori[0][lane] = sn;
-      sm.ori[1][lane] = cs;
-    } else {
-      sm.ori[2][lane] = cs;
+      for (int k = 0; k < 11; ++k) x[k] = valid ? th(k) : 1.0;
+      sm.flag[lane] = valid && physical_bits(x) && !out(lane) ? 0 : 1;
+    } else {  // parts 1, 3, 5, 7: the PN coefficients, as pn_coeffs forms them
+      const FF q = ff_from(valid ? th(1) : 0.5), chi1 = ff_from(valid ? th(2) : 0.0),
+               chi2 = ff_from(valid ? th(3) : 0.0);
+      const FF eta = pn_eta(q), eta2 = eta * eta;
+      if (part == 1) {
+        const FF x1 = 1.0 / (q + 1.0), x2 = q * x1;
+        const FF beta = ((113.0 / 12.0) * x1 * x1 + 6.25 * eta) * chi1 + ((113.0 / 12.0) * x2 * x2 + 6.25 * eta) * chi2;
+        sm.phi[0][lane] = (743.0 / 336.0 + (11.0 / 4.0) * eta) * (20.0 / 9.0);
+        sm.phi[1][lane] = 4.0 * beta - 16.0 * kPi;
+        sm.phi[2][lane] = pn_quad(eta, eta2, kPnP4) * 10.0 - (10.0 * 79.0 / 8.0) * eta * chi1 * chi2;
+      } else {
+        const FF delta = pn_delta(q), chis = (chi1 + chi2) * 0.5, chia = (chi1 - chi2) * 0.5;
+        if (part == 5) {
+          const FF gam = pn_quad(eta, eta2, kPnGam) * chis + ((140.0 / 9.0) * eta + 732985.0 / 2268.0) * delta * chia;
+          sm.phi[3][lane] = kPi * (38645.0 / 756.0 - (65.0 / 9.0) * eta) - gam;
+        } else if (part == 3) {
+          sm.phi[4][lane] = pn_quad(eta, eta2, kPnP6) - (127825.0 / 1296.0) * eta2 * eta +
+                            kPi * ((2270.0 / 3.0) * delta * chia + ((2270.0 / 3.0) - 520.0 * eta) * chis);
+        } else {
+          sm.phi[5][lane] = kPi * pn_quad(eta, eta2, kPnP7) +
+                            (pn_quad(eta, eta2, kPnP7s) + (5345.0 / 36.0) * eta2 * eta) * chis +
+                            delta * pn_quad(eta, eta2, kPnP7a) * chia;
+        }
+      }
     }
   }
-  __syncthreads();
+  group_sync<NW>();
   // ---- phase 2
-  const bool ok = sm.flag[lane] == 0;
   if (part == 0) {
     Scale<FF> S;
     S.la = sm.lmc[lane] - 0.6 * sm.leta[lane];
@@ -191,6 +236,7 @@ __device__ __forceinline__ void fused_coeffs(const SegInfo& s, int R, FusedSmem<
     P.p7 = sm.phi[5][lane];
     FF c[kNBasis], ccyc;
     basis_coeffs(P, S, c, ccyc);
+    const bool ok = sm.flag[lane] == 0;
 #pragma unroll
     for (int m = 0; m < kNBasis; ++m) {
       sm.pm[lane].ch[m] = ok ? c[m].hi : 0.0f;
@@ -212,17 +258,16 @@ __device__ __forceinline__ void fused_coeffs(const SegInfo& s, int R, FusedSmem<
     const FF la = sm.lmc[lane] - 0.6 * sm.leta[lane];
     const FF a13 = exp(la * (1.0 / 3.0));
     int ncut = 0;
-    if (ok) {
+    if (sm.flag[lane] == 0) {
       ncut = (int)s.M;
       if (s.fcut_mode == 0) ncut = count_bins_le(s, ff_to_double(1.0 / (kSix32 * (a13 * a13 * a13))));
     }
     sm.ncut[lane] = ncut;
     const int nm = __reduce_max_sync(0xffffffffu, ncut);
     if (lane == 0) sm.maxcut = nm;
-#pragma unroll
-    for (int d = 0; d < NDET; ++d) sm.Hc[d][lane] = ncut > 0 ? s.H[(int64_t)d * s.M + ncut - 1] : 0.0;
   } else if (part - 4 < NDET) {
     const int d = part - 4;
+    const bool ok = sm.flag[lane] == 0;
     Sky<FF> k;
     k.sl = sm.sky[0][lane];
     k.cl = sm.sky[1][lane];
@@ -236,17 +281,9 @@ __device__ __forceinline__ void fused_coeffs(const SegInfo& s, int R, FusedSmem<
     sm.P[2 * d][lane] = Pr;
     sm.P[2 * d + 1][lane] = Pi;
   }
-  __syncthreads();
-  // ---- phase 3 (no barrier after it)
-  if (part < NDET) {
-    const int d = part;
-    const FF amp = sm.amp[lane], Pr = sm.P[2 * d][lane], Pi = sm.P[2 * d + 1][lane];
-    const FF sa = sm.ang[0][lane], ca = sm.ang[1][lane];
-    const FF kr = amp * (Pr * ca - Pi * sa), ki = amp * (Pr * sa + Pi * ca);
-    sm.Kr[d][lane] = ff_to_double(kr);
-    sm.Ki[d][lane] = ff_to_double(ki);
-    sm.hterm[d][lane] = (kr * kr + ki * ki) * ff_from(sm.Hc[d][lane]);
-  } else if (part == 7) {
+  group_sync<NW>();
+  // rows by descending cut, where warps take more than one row
+  if (part == 7 && R > NW) {
     const int n = valid ? sm.ncut[lane] : -1;
     int rank = 0;
 #pragma unroll 4
@@ -256,6 +293,20 @@ __device__ __forceinline__ void fused_coeffs(const SegInfo& s, int R, FusedSmem<
     }
     sm.order[rank] = lane;
   }
+}
+
+// K_d and the <h|h> term of detector d, one row per lane (one warp; after
+// fused_coeffs).
+template <int NDET, bool CAL, int NW>
+__device__ __forceinline__ void fused_amplitudes(const SegInfo& s, FusedSmem<NDET, CAL, NW>& sm, int d, int lane) {
+  const int ncut = sm.ncut[lane];
+  const double H = ncut > 0 ? s.H[(int64_t)d * s.M + ncut - 1] : 0.0;
+  const FF amp = sm.amp[lane], Pr = sm.P[2 * d][lane], Pi = sm.P[2 * d + 1][lane];
+  const FF sa = sm.ang[0][lane], ca = sm.ang[1][lane];
+  const FF kr = amp * (Pr * ca - Pi * sa), ki = amp * (Pr * sa + Pi * ca);
+  sm.Kr[d][lane] = ff_to_double(kr);
+  sm.Ki[d][lane] = ff_to_double(ki);
+  sm.hterm[d][lane] = (kr * kr + ki * ki) * ff_from(H);
 }
 
 // Warp sums of n FP32 values per lane with the tree of an xor butterfly over
@@ -383,25 +434,27 @@ __device__ __forceinline__ void fused_row_sums(const FusedArgs& a, const FusedLa
   }
 }
 
-// Bin sums of the group's rows (all threads; fused_coeffs before it): the
+// Bin sums of the group's rows (all its threads; fused_coeffs before it): the
 // windows in groups of nwc, each staged unless it is in place, its anchor
-// records, its (row, window) items, its windows' sums added to sm.acc in
-// window order.  st: the group that shared memory holds.  crow(r): the
-// calibration parameters of row r.  Returns false when a bounded wait ran out.
+// records, its items.  The first items are the detectors' amplitudes, the
+// others (row, window) pairs.  The windows' sums of every group but the last
+// are added to sm.acc in window order; the last group's are left in place for
+// fused_combine.  st: the group that shared memory holds.  crow(r): the
+// calibration parameters of row r.  Ends without a barrier after the last
+// items; returns false when a bounded wait ran out (the same on every thread).
 struct FusedStage {
   int w0 = 0;             // first window of the group in shared memory
   bool pending = true;    // its copy is in flight (the caller has started the first one)
   uint32_t parity = 0;    // the barrier's phase
 };
 
-template <int NDET, bool CAL, class Crow>
+template <int NDET, bool CAL, int NW, class Crow>
 __device__ __forceinline__ bool fused_bins(const FusedArgs& a, const FusedLayout& L, float* dyn, int R,
-                                           FusedSmem<NDET, CAL>& sm, FusedStage& st, Crow crow) {
-  constexpr int NS = FusedSmem<NDET, CAL>::NS, AR = anchor_rec_floats(NDET);
+                                           FusedSmem<NDET, CAL, NW>& sm, FusedStage& st, Crow crow) {
+  constexpr int NS = FusedSmem<NDET, CAL, NW>::NS, AR = anchor_rec_floats(NDET);
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const int gbins = a.CH * a.nwc, gblk = (a.CH + kAnchor - 1) / kAnchor * a.nwc;
   const int maxcut = sm.maxcut;
-  for (int i = t; i < NS * kFusedRows; i += 256) (&sm.acc[0][0])[i] = 0.0;
   for (int w0 = 0; (int64_t)w0 * a.CH < maxcut; w0 += a.nwc) {
     const int j0 = w0 * a.CH;
     const int top = maxcut - j0 < gbins ? maxcut - j0 : gbins;  // the longest row's bins in this group
@@ -413,13 +466,13 @@ __device__ __forceinline__ bool fused_bins(const FusedArgs& a, const FusedLayout
         }
         st.w0 = w0;
       }
-      if (!mbar_wait_bounded(&sm.bar, st.parity, a.status)) return false;
+      if (!mbar_wait_bounded(&sm.bar, st.parity, a.status)) sm.fail = 1;
       st.parity ^= 1u;
       st.pending = false;
     }
     // anchor records, blocks of a row on neighbouring threads
     const int nb = (top + kAnchor - 1) / kAnchor;
-    for (int i = t; i < R * nb; i += 256) {
+    for (int i = t; i < R * nb; i += 32 * NW) {
       const int r = i / nb, b = i - r * nb;
       if (j0 + b * kAnchor >= sm.ncut[r]) continue;
       float ch[kNBasis], cl[kNBasis], th[NDET], tl[NDET], an[NDET];
@@ -441,13 +494,19 @@ __device__ __forceinline__ bool fused_bins(const FusedArgs& a, const FusedLayout
       o[NDET] = fast ? 1.0f : 0.0f;
     }
     if (t == 0) sm.next = 0;
-    __syncthreads();
+    group_sync<NW>();
+    if (sm.fail) return false;
     const int nwa = (top + a.CH - 1) / a.CH;  // windows of the group that hold bins
+    const int nk = w0 == 0 ? NDET : 0;
     while (true) {
       int item = 0;
       if (lane == 0) item = atomicAdd(&sm.next, 1);
-      item = __shfl_sync(0xffffffffu, item, 0);
+      item = __shfl_sync(0xffffffffu, item, 0) - nk;
       if (item >= R * nwa) break;
+      if (item < 0) {
+        fused_amplitudes<NDET, CAL, NW>(a.seg, sm, item + nk, lane);
+        continue;
+      }
       const int wl = item / R, r = sm.order[item - wl * R];
       const int jl = wl * a.CH;
       int n = sm.ncut[r] - j0 - jl;
@@ -456,8 +515,8 @@ __device__ __forceinline__ bool fused_bins(const FusedArgs& a, const FusedLayout
       float4* nodes = sm.nodes + (CAL ? warp * NDET * kMaxCalNodes : 0);
       if constexpr (CAL) cal_nodes_fill<NDET, true>(crow(r), a.nn, a.calQ, lane, nodes);
       float U[NDET], V[NDET], X[NDET], v[NS];
-      fused_row_sums<NDET, CAL>(a, L, dyn, sm.pm[r], dyn + L.rec + (r * gblk + jl / kAnchor) * AR, j0, jl, n, lane, nodes,
-                                U, V, X);
+      fused_row_sums<NDET, CAL>(a, L, dyn, sm.pm[r], dyn + L.rec + (r * gblk + jl / kAnchor) * AR, j0, jl, n, lane,
+                                nodes, U, V, X);
 #pragma unroll
       for (int d = 0; d < NDET; ++d) {
         v[2 * d] = U[d];
@@ -468,34 +527,51 @@ __device__ __forceinline__ bool fused_bins(const FusedArgs& a, const FusedLayout
       constexpr int W = FoldP<NS>::W;
       if (lane % W == 0 && lane / W < NS) dyn[L.part + (r * a.nwc + wl) * NS + lane / W] = s;
     }
-    __syncthreads();
-    // the group's window sums, in window order (one thread per row and sum)
-    for (int i = t; i < R * NS; i += 256) {
-      const int r = i / NS, k = i - r * NS;
-      const int left = sm.ncut[r] - j0;
-      double x = sm.acc[k][r];
-      for (int wl = 0; wl < nwa && wl * a.CH < left; ++wl) x += (double)dyn[L.part + (r * a.nwc + wl) * NS + k];
-      sm.acc[k][r] = x;
+    if (j0 + gbins < maxcut) {  // another group follows: its sums go on top of these
+      group_sync<NW>();
+      for (int i = t; i < R * NS; i += 32 * NW) {
+        const int r = i / NS, k = i - r * NS;
+        const int left = sm.ncut[r] - j0;
+        double x = w0 == 0 ? 0.0 : sm.acc[k][r];
+        for (int wl = 0; wl < nwa && wl * a.CH < left; ++wl) x += (double)dyn[L.part + (r * a.nwc + wl) * NS + k];
+        sm.acc[k][r] = x;
+      }
+      group_sync<NW>();
     }
-    __syncthreads();
   }
   return true;
 }
 
-// lnL of row r from the sums (one thread): -inf for an unphysical row, 0
-// without an in-band bin.
-template <int NDET, bool CAL>
-__device__ __forceinline__ double fused_combine(const FusedSmem<NDET, CAL>& sm, int r) {
+// lnL of row r from the sums (one thread; a barrier after fused_bins): -inf for
+// an unphysical row, 0 without an in-band bin.
+template <int NDET, bool CAL, int NW>
+__device__ __forceinline__ double fused_combine(const FusedArgs& a, const FusedLayout& L, const float* __restrict__ dyn,
+                                                const FusedSmem<NDET, CAL, NW>& sm, int r) {
+  constexpr int NS = FusedSmem<NDET, CAL, NW>::NS;
+  const int ncut = sm.ncut[r];
   if (sm.flag[r]) return -INFINITY;
-  if (sm.ncut[r] <= 0) return 0.0;
+  if (ncut <= 0) return 0.0;
+  const int gbins = a.CH * a.nwc;
+  const int j0 = (sm.maxcut - 1) / gbins * gbins;  // the last group's first bin
+  const float* part = dyn + L.part + r * a.nwc * NS;
+  const bool one = ncut <= a.CH;  // the row's only window
+  auto sum = [&](int k) {
+    if (one) return (double)part[k];
+    double x = j0 > 0 ? sm.acc[k][r] : 0.0;
+#pragma unroll 1
+    for (int wl = 0; wl < a.nwc && j0 + wl * a.CH < ncut; ++wl) x += (double)part[wl * NS + k];
+    return x;
+  };
   FF hh = ff(0.0f);
   double acc = 0.0;
 #pragma unroll
   for (int d = 0; d < NDET; ++d) {
     hh = hh + sm.hterm[d][r];
     const double kr = sm.Kr[d][r], ki = sm.Ki[d][r];
-    acc += kr * sm.acc[2 * d][r] - ki * sm.acc[2 * d + 1][r];
-    if constexpr (CAL) acc -= 0.5 * (kr * kr + ki * ki) * sm.acc[2 * NDET + d][r];
+    const double U = sum(2 * d), V = sum(2 * d + 1);
+    // the fused multiply-adds that flush_pending's expressions compile to
+    acc = __dadd_rn(acc, __fma_rn(kr, U, -__dmul_rn(ki, V)));
+    if constexpr (CAL) acc = __fma_rn(-0.5 * __fma_rn(kr, kr, __dmul_rn(ki, ki)), sum(2 * NDET + d), acc);
   }
   return acc - 0.5 * ff_to_double(hh);
 }

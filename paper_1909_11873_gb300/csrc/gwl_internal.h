@@ -139,7 +139,9 @@ cudaError_t launch_loglike(gwl_ctx* c, const double* theta, int64_t B, double* l
 cudaError_t launch_loglike_cleared(gwl_ctx* c, const double* theta, int64_t B, double* lnl, cudaStream_t st);
 int64_t work_needed(const gwl_ctx* c, int64_t B);
 // the one-kernel form (gwl_fused.cu): its launch shape for a batch (false: not used), launch
-bool fused_shape(const gwl_ctx* c, int64_t B, int* grid, int* rows, int* nwc, size_t row_bytes = 0);
+bool fused_shape(const gwl_ctx* c, int64_t B, int* grid, int* rows, int* nwc);
+int fused_window_count(const gwl_ctx* c);
+int fused_windows(const gwl_ctx* c, int R, size_t room);
 bool fused_used(const gwl_ctx* c, int64_t B);
 cudaError_t launch_fused(gwl_ctx* c, const double* theta, int64_t B, double* lnl, int grid, int rows, int nwc,
                          cudaStream_t st);

@@ -180,41 +180,121 @@ __global__ void k_walk_step(PriorInfo pr, const WalkScalars* __restrict__ sc, co
 // A chain depends on no other chain within a round, so a CTA takes a group of
 // chains through all steps of the walk by itself: proposal, the group's
 // likelihood (gwl_fused.cuh, whose table rows stay in shared memory from step
-// to step while one group of windows covers the rows) and accept/reject.  The
-// random numbers and their products L z do not depend on the chain's state:
-// warp 7 forms the next step's while the other warps sum bins.  FP64 warp
-// instructions hold the narrow FP64 pipe however few lanes are active, so the
-// FP64 work is packed over (chain, coordinate) pairs.
+// to step while one group of windows covers the rows) and accept/reject.
+//
+// FP64 instructions have a long latency and hold the narrow FP64 pipe however
+// few lanes are active: the normals of a step (logarithm, square root, sine and
+// cosine) take 4 us, the prior maps (cube root, arc sine and cosine) up to
+// 2.5 us.  Four warps beside the likelihood's do both ahead of time, packed
+// over (chain, coordinate) pairs: two form the normals of the step after next
+// and their products L z, which do not depend on the chains' states, and two
+// form the next proposal and its parameters from either state that the chain
+// can be in then, so that a step begins with a choice between two finished
+// proposals.
 //
 // What bounds it: per step the latency of the coefficients' float-pair chains
 // and of the bin sums of one row per warp.  Measured per step (us, 20-step
 // walks) against three dependent launches a step (proposal, prologue, bin
-// loop), at 1 / 250 / 1000 / 1900 chains: 4 s, 1 detector, 4-D 9.8 / 12.3 /
-// 12.5 / 14.5 against 29.7 / 35.5 / 41.4 / 47.8; 8 s, 3 detectors, 11-D
-// 11.2 / 15.4 / 19.8 / 22.0 against 41.7 / 57.2 / 59.9 / 62.0.
-template <int NDET, bool CAL>
-__global__ void __launch_bounds__(256, 2)
+// loop), at 1 / 250 / 1000 / 1900 chains: 4 s, 1 detector, 4-D 6.9 / 9.9 /
+// 10.2 / 10.7 against 29.7 / 35.5 / 41.4 / 47.8; 8 s, 3 detectors, 11-D
+// 6.2 / 11.6 / 11.2 / 11.9 against 41.7 / 57.2 / 59.9 / 62.0.
+constexpr int kWalkHelpers = 4;  // warps beside the likelihood's
+
+// A CTA's walk state in shared memory, for the two functions that the helper
+// warps run (out of line: one copy of their FP64 functions each, beside a
+// likelihood whose code already fills the instruction cache).
+struct WalkGroup {
+  double *cu, *pu;  // [R][D] the points, their proposals
+  double *cx, *ct;  // [2][R][D] the next step's proposals and parameters, from the point kept or the proposal taken
+  double *dz;       // [2][R][D] L z of odd and even steps
+  double *z;        // [2][R][2 np] normals
+  int* cout;        // [2][kFusedRows] whether that proposal left the cube
+  const double* chol;
+  int64_t b0;       // first chain
+  int R, D, n;      // chains per CTA, coordinates, chains of this CTA
+  uint32_t counter, k0, k1;
+  double scale;
+};
+
+// Normals of step s and their products with the step matrix, chains [r0, r1) (one warp).
+static __device__ __noinline__ void walk_draw(const WalkGroup& g, uint32_t s, int r0, int r1) {
+  const int lane = threadIdx.x & 31, D = g.D, np = (D + 1) / 2, m = r1 - r0;
+  double* zs = g.z + (s & 1) * g.R * 2 * np;
+  for (int q = lane; q < m * np; q += 32) {
+    const int k = q % np, r = r0 + q / np;
+    const uint4 v = philox(make_uint4((uint32_t)(k >> 1), s, (uint32_t)(g.b0 + r), g.counter), g.k0, g.k1);
+    const uint32_t w0 = (k & 1) ? v.z : v.x, w1 = (k & 1) ? v.w : v.y;
+    const double u1 = ((double)w0 + 1.0) * 0x1p-32;
+    const double u2 = (double)w1 * 0x1p-32;
+    const double rr = sqrt(-2.0 * ::log(u1));
+    double sn, cs;
+    sincospi(2.0 * u2, &sn, &cs);
+    zs[r * 2 * np + 2 * k] = rr * cs;
+    zs[r * 2 * np + 2 * k + 1] = rr * sn;
+  }
+  __syncwarp();
+  for (int q = lane; q < m * D; q += 32) {
+    const int i = q / m, r = r0 + q - i * m;
+    const double* z = zs + r * 2 * np;
+    const double* row = g.chol + i * D;
+    double dz = 0.0;
+#pragma unroll 1
+    for (int k = 0; k <= i; ++k) dz += row[k] * z[k];
+    g.dz[(s & 1) * g.R * D + r * D + i] = dz;
+  }
+  __syncwarp();
+}
+
+// The proposals of step s from the points kept (v = 0) or the proposals taken
+// (v = 1), threads t0, t0 + nt, ... over (coordinate, chain), coordinates
+// outermost so that a warp's lanes mostly share a prior map.
+template <bool CAL>
+static __device__ __noinline__ void walk_candidates(const WalkGroup& g, const PriorInfo& pr, uint32_t s, int v, int t0,
+                                                    int nt) {
+  const int D = g.D, RD = g.R * D;
+#pragma unroll 1
+  for (int q = t0; q < g.n * D; q += nt) {
+    const int i = q / g.n, r = q - i * g.n, e = r * D + i;
+    double x = (v ? g.pu : g.cu)[e] + g.scale * g.dz[(s & 1) * RD + e];
+    if (coord_periodic(pr, i)) x -= floor(x);
+    else if (x < 0.0 || x > 1.0) g.cout[v * kFusedRows + r] = 1;
+    g.cx[v * RD + e] = x;
+    g.ct[v * RD + e] = CAL ? coord_map(pr, i, x) : prior_map(pr.kind[i], pr.lo[i], pr.hi[i], x);
+  }
+}
+
+template <int NDET, bool CAL, int NW>
+__global__ void __launch_bounds__(32 * (NW + kWalkHelpers), 1)
     k_walk_fused(const __grid_constant__ FusedArgs a, const __grid_constant__ PriorInfo pr, WalkScalars val,
                  const WalkScalars* __restrict__ sc, const double* __restrict__ live_u,
                  const double* __restrict__ live_lnl, int64_t K, const double* __restrict__ chol, uint64_t seed,
                  int64_t n_chains, int walk_len, int R, double* __restrict__ out_u, double* __restrict__ out_lnl,
                  int32_t* __restrict__ out_nacc, int32_t* __restrict__ out_start) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  __shared__ FusedSmem<NDET, CAL> sm;
+  __shared__ FusedSmem<NDET, CAL, NW> sm;
   __shared__ double s_l[kFusedRows], s_cl[kFusedRows];
-  __shared__ int s_n[kFusedRows], s_out[kFusedRows], s_start[kFusedRows];
+  __shared__ int s_n[kFusedRows], s_out[kFusedRows], s_start[kFusedRows], s_cout[2][kFusedRows];
   float* dyn = reinterpret_cast<float*>(smem_raw);
   const FusedLayout L = fused_layout(NDET, CAL ? a.cal_row : 0, a.CH, a.nwc, R);
-  const int D = pr.D, np = (D + 1) / 2;
-  // per chain: the point, the proposal and its parameters, the normals and L z
-  double* s_cu = reinterpret_cast<double*>(dyn + ((L.total + 1) & ~1));
-  double* s_pu = s_cu + R * D;
-  double* s_th = s_pu + R * D;
-  double* s_dz = s_th + R * D;
-  double* s_z = s_dz + R * D;
+  const int D = pr.D, np = (D + 1) / 2, RD = R * D;
+  WalkGroup g;
+  g.cu = reinterpret_cast<double*>(dyn + ((L.total + 1) & ~1));
+  g.pu = g.cu + RD;
+  double* s_th = g.pu + RD;  // parameters of the proposals
+  g.cx = s_th + RD;
+  g.ct = g.cx + 2 * RD;
+  g.dz = g.ct + 2 * RD;
+  g.z = g.dz + 2 * RD;
+  g.cout = &s_cout[0][0];
+  g.chol = chol;
+  g.R = R;
+  g.D = D;
+  g.k0 = (uint32_t)seed;
+  g.k1 = (uint32_t)(seed >> 32);
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   cudaTriggerProgrammaticLaunchCompletion();
   if (t == 0) {
+    sm.fail = 0;
     mbar_init(&sm.bar, 1);
     fence_mbar_init();
     fused_stage<NDET, CAL>(a, L, dyn, 0, &sm.bar);
@@ -223,83 +303,81 @@ __global__ void __launch_bounds__(256, 2)
   const WalkScalars w = sc ? *sc : val;
   const int64_t b0 = (int64_t)blockIdx.x * R;
   const int n = n_chains - b0 < R ? (int)(n_chains - b0) : R;
-  // normals of step s and their products with the step matrix (one warp)
-  auto draw = [&](uint32_t s) {
-    for (int q = lane; q < n * np; q += 32) {
-      const int r = q / np, k = q - r * np;
-      const uint4 v = philox(make_uint4((uint32_t)(k >> 1), s, (uint32_t)(b0 + r), (uint32_t)w.counter),
-                             (uint32_t)seed, (uint32_t)(seed >> 32));
-      const uint32_t w0 = (k & 1) ? v.z : v.x, w1 = (k & 1) ? v.w : v.y;
-      const double u1 = ((double)w0 + 1.0) * 0x1p-32;
-      const double u2 = (double)w1 * 0x1p-32;
-      const double rr = sqrt(-2.0 * ::log(u1));
-      double sn, cs;
-      sincospi(2.0 * u2, &sn, &cs);
-      s_z[r * 2 * np + 2 * k] = rr * cs;
-      s_z[r * 2 * np + 2 * k + 1] = rr * sn;
-    }
-    __syncwarp();
-    for (int q = lane; q < n * D; q += 32) {
-      const int i = q / n, r = q - i * n;
-      const double* z = s_z + r * 2 * np;
-      double dz = 0.0;
-      for (int k = 0; k <= i; ++k) dz += chol[i * D + k] * z[k];
-      s_dz[r * D + i] = dz;
-    }
-  };
+  g.b0 = b0;
+  g.n = n;
+  g.counter = (uint32_t)w.counter;
+  g.scale = w.scale;
   // the chains' start points
   if (t < n) {
-    const uint4 v = philox(make_uint4(0u, 0u, (uint32_t)(b0 + t), (uint32_t)w.counter), (uint32_t)seed,
-                           (uint32_t)(seed >> 32));
+    const uint4 v = philox(make_uint4(0u, 0u, (uint32_t)(b0 + t), g.counter), g.k0, g.k1);
     const int64_t idx = (int64_t)(((uint64_t)v.x * (uint64_t)(K - 1)) >> 32);
     const int64_t st = idx < w.worst ? idx : idx + 1;
     s_start[t] = (int)st;
     s_cl[t] = live_lnl[st];
     s_n[t] = 0;
-    s_out[t] = 0;
+    s_cout[0][t] = s_cout[1][t] = 0;
     s_l[t] = 0.0;
   }
-  if (warp == 7 && walk_len > 0) draw(1);
-  __syncthreads();
-  for (int q = t; q < n * D; q += 256) {
-    const int i = q / n, r = q - i * n;
-    s_cu[r * D + i] = live_u[(int64_t)s_start[r] * D + i];
+  const int half = (n + 1) / 2;
+  if (warp >= NW && walk_len > 0) {
+    const int h = warp - NW;  // the first two steps' draws, by halves of the chains
+    walk_draw(g, (uint32_t)(h < 2 ? 1 : 2), h & 1 ? half : 0, h & 1 ? n : half);
   }
+  __syncthreads();
+  for (int q = t; q < n * D; q += blockDim.x) {
+    const int i = q / n, r = q - i * n;
+    g.cu[r * D + i] = live_u[(int64_t)s_start[r] * D + i];
+  }
+  if (walk_len > 0) walk_candidates<CAL>(g, pr, 1, 0, t, blockDim.x);  // over the pairs that the thread has just set
+  __syncthreads();
   FusedStage stg;
+  bool ok = true;
   for (int s = 1; s <= walk_len; ++s) {
-    // the last step's accept (a thread keeps its pairs from step to step), this step's proposal
-    for (int q = t; q < n * D; q += 256) {
-      const int i = q / n, r = q - i * n, e = r * D + i;
-      if (s > 1 && s_l[r] >= w.lstar) s_cu[e] = s_pu[e];
-      double x = s_cu[e] + w.scale * s_dz[e];
-      if (coord_periodic(pr, i)) x -= floor(x);
-      else if (x < 0.0 || x > 1.0) s_out[r] = 1;
-      s_pu[e] = x;
-      s_th[e] = coord_map(pr, i, x);
+    if (warp < NW) {
+      // the last step's accept, and the proposal that follows from it
+      for (int q = t; q < n * D; q += 32 * NW) {
+        const int i = q / n, r = q - i * n, e = r * D + i;
+        const int v = s > 1 && s_l[r] >= w.lstar ? 1 : 0;
+        if (v) g.cu[e] = g.pu[e];
+        g.pu[e] = g.cx[v * RD + e];
+        s_th[e] = g.ct[v * RD + e];
+        if (i == 0) s_out[r] = s_cout[v][r];
+      }
     }
     __syncthreads();
-    fused_coeffs<NDET, CAL>(
-        a.seg, n, sm,
-        [&](int k) { return a.seg.param_pos[k] >= 0 ? s_th[lane * D + a.seg.param_pos[k]] : a.seg.fixed[k]; },
-        [&](int r) { return s_out[r] != 0; });
-    if (warp == 7 && s < walk_len) draw((uint32_t)s + 1);
-    if (!fused_bins<NDET, CAL>(a, L, dyn, n, sm, stg, [&](int r) { return s_th + r * D + a.cal_par; })) return;
-    __syncthreads();
-    if (t < n) {
-      const double l = fused_combine<NDET, CAL>(sm, t);
-      s_l[t] = l;
-      s_out[t] = 0;
-      if (l >= w.lstar) {  // rows outside the cube give -inf
-        s_cl[t] = l;
-        s_n[t] += 1;
+    if (warp < NW) {
+      fused_coeffs<NDET, CAL, NW>(
+          a.seg, n, sm,
+          [&](int k) { return a.seg.param_pos[k] >= 0 ? s_th[lane * D + a.seg.param_pos[k]] : a.seg.fixed[k]; },
+          [&](int r) { return s_out[r] != 0; });
+      ok = fused_bins<NDET, CAL, NW>(a, L, dyn, n, sm, stg, [&](int r) { return s_th + r * D + a.cal_par; });
+      if (!ok) return;  // a bounded wait ran out
+      group_sync<NW>();
+      if (t < n) {
+        const double l = fused_combine<NDET, CAL, NW>(a, L, dyn, sm, t);
+        s_l[t] = l;
+        if (l >= w.lstar) {  // rows outside the cube give -inf
+          s_cl[t] = l;
+          s_n[t] += 1;
+        }
+      }
+    } else {
+      const int h = warp - NW;
+      if (h < 2) {
+        if (s + 2 <= walk_len) walk_draw(g, (uint32_t)s + 2, h ? half : 0, h ? n : half);
+      } else if (s < walk_len) {
+        const int v = h - 2;
+        for (int r = lane; r < n; r += 32) s_cout[v][r] = 0;
+        __syncwarp();
+        walk_candidates<CAL>(g, pr, (uint32_t)s + 1, v, lane, 32);
       }
     }
     __syncthreads();
   }
-  if (stg.pending) mbar_wait_bounded(&sm.bar, stg.parity, a.status);  // no copy may outlive the CTA
-  for (int q = t; q < n * D; q += 256) {
+  if (t == 0 && stg.pending) mbar_wait_bounded(&sm.bar, stg.parity, a.status);  // no copy may outlive the CTA
+  for (int q = t; q < n * D; q += blockDim.x) {
     const int i = q / n, r = q - i * n, e = r * D + i;
-    out_u[(b0 + r) * D + i] = walk_len > 0 && s_l[r] >= w.lstar ? s_pu[e] : s_cu[e];
+    out_u[(b0 + r) * D + i] = walk_len > 0 && s_l[r] >= w.lstar ? g.pu[e] : g.cu[e];
   }
   if (t < n) {
     out_lnl[b0 + t] = s_cl[t];
@@ -1044,26 +1122,68 @@ static cudaError_t launch_gmc(gwl_ctx* c, const double* live_u, const double* li
 // Shared memory per chain of k_walk_fused.
 static size_t walk_row_bytes(const gwl_ctx* c) {
   const size_t D = (size_t)theta_stride(c);
-  return sizeof(double) * (5 * D + 1);
+  return sizeof(double) * (11 * D + 2);
+}
+template <int NDET, bool CAL, int NW>
+static size_t walk_static() {
+  return sizeof(FusedSmem<NDET, CAL, NW>) + kFusedRows * (2 * sizeof(double) + 5 * sizeof(int)) + 256;
 }
 
-static bool walk_fused_shape(const gwl_ctx* c, int64_t n_chains, int* grid, int* rows, int* nwc) {
-  return c->walk_kind == GWL_WALK_RANDOM && !lanes_seg(c, n_chains) &&
-         fused_shape(c, n_chains, grid, rows, nwc, walk_row_bytes(c));
-}
+// The launch shape of k_walk_fused: one CTA per SM, of eight warps with a chain
+// each, or of sixteen with up to 32 chains in whole waves.
+struct WalkShape {
+  int grid, rows, nwc;
+  bool wide;  // sixteen warps
+};
 
 template <int NDET, bool CAL>
+static bool walk_shape_of(const gwl_ctx* c, int64_t n, WalkShape* o) {
+  o->wide = n > 8 * (int64_t)c->num_sms;
+  const int64_t waves = (n + (int64_t)c->num_sms * kFusedRows - 1) / ((int64_t)c->num_sms * kFusedRows);
+  const int64_t R = (n + c->num_sms * waves - 1) / (c->num_sms * waves);
+  const size_t used = (o->wide ? walk_static<NDET, CAL, 16>() : walk_static<NDET, CAL, 8>()) +
+                      (size_t)R * walk_row_bytes(c);
+  constexpr size_t all = 227 * 1024;
+  o->rows = (int)R;
+  o->grid = (int)((n + R - 1) / R);
+  o->nwc = used < all ? fused_windows(c, (int)R, all - used) : 0;
+  return o->nwc > 0;
+}
+
+// Calls f(std::integral_constant<int, NDET>, std::bool_constant<CAL>) for the context.
+template <class F>
+static auto for_model(const gwl_ctx* c, F f) {
+  auto pick = [&](auto nd) { return c->n_cal_nodes > 0 ? f(nd, std::true_type()) : f(nd, std::false_type()); };
+  switch (c->n_det) {
+    case 1: return pick(std::integral_constant<int, 1>());
+    case 2: return pick(std::integral_constant<int, 2>());
+    case 3: return pick(std::integral_constant<int, 3>());
+    default: return pick(std::integral_constant<int, 4>());
+  }
+}
+
+// Whether the random walk of n chains runs as one kernel: where gwl_loglike of
+// n rows would (gwl_fused.cu gives the line and both sides).
+static bool walk_fused_shape(const gwl_ctx* c, int64_t n, WalkShape* o) {
+  if (c->walk_kind != GWL_WALK_RANDOM || !fused_used(c, n)) return false;
+  return for_model(c, [&](auto nd, auto cal) {
+    return walk_shape_of<decltype(nd)::value, decltype(cal)::value>(c, n, o);
+  });
+}
+
+template <int NDET, bool CAL, int NW>
 static cudaError_t run_walk_fused(gwl_ctx* c, const WalkScalars& val, const WalkScalars* sc, const double* live_u,
                                   const double* live_lnl, int64_t K, uint64_t seed, int64_t n_chains, int walk_len,
                                   const double* chol, double* out_u, double* out_lnl, int32_t* out_nacc,
-                                  int32_t* out_start, int grid, int rows, int nwc, cudaStream_t st) {
-  const FusedArgs a = fused_args(c, nwc);
-  const size_t smem = fused_bytes(c, nwc, rows) + 8 + (size_t)rows * walk_row_bytes(c);
-  cudaError_t e = raise_smem_limit((const void*)k_walk_fused<NDET, CAL>, c->device, smem);
+                                  int32_t* out_start, const WalkShape& sh, cudaStream_t st) {
+  const FusedArgs a = fused_args(c, sh.nwc);
+  const size_t smem = fused_bytes(c, sh.nwc, sh.rows) + 8 + (size_t)sh.rows * walk_row_bytes(c);
+  cudaError_t e = raise_smem_limit((const void*)k_walk_fused<NDET, CAL, NW>, c->device, smem);
   if (e != cudaSuccess) return e;
   ProfScope ps(c, GWL_KERNEL_WALK, st);
-  e = launch_pdl(k_walk_fused<NDET, CAL>, dim3(grid), dim3(256), smem, st, a, prior_info(c), val, sc, live_u, live_lnl,
-                 K, chol, seed, n_chains, walk_len, rows, out_u, out_lnl, out_nacc, out_start);
+  e = launch_pdl(k_walk_fused<NDET, CAL, NW>, dim3(sh.grid), dim3(32 * (NW + kWalkHelpers)), smem, st, a,
+                 prior_info(c), val, sc, live_u, live_lnl, K, chol, seed, n_chains, walk_len, sh.rows, out_u, out_lnl,
+                 out_nacc, out_start);
   c->launches++;
   return e;
 }
@@ -1071,21 +1191,15 @@ static cudaError_t run_walk_fused(gwl_ctx* c, const WalkScalars& val, const Walk
 static cudaError_t launch_walk_fused(gwl_ctx* c, const WalkScalars& val, const WalkScalars* sc, const double* live_u,
                                      const double* live_lnl, int64_t K, uint64_t seed, int64_t n_chains, int walk_len,
                                      const double* chol, double* out_u, double* out_lnl, int32_t* out_nacc,
-                                     int32_t* out_start, int grid, int rows, int nwc, cudaStream_t st) {
-  auto go = [&](auto nd, auto cal) {
-    return run_walk_fused<decltype(nd)::value, decltype(cal)::value>(c, val, sc, live_u, live_lnl, K, seed, n_chains,
-                                                                     walk_len, chol, out_u, out_lnl, out_nacc,
-                                                                     out_start, grid, rows, nwc, st);
-  };
-  auto pick = [&](auto nd) {
-    return c->n_cal_nodes > 0 ? go(nd, std::true_type()) : go(nd, std::false_type());
-  };
-  switch (c->n_det) {
-    case 1: return pick(std::integral_constant<int, 1>());
-    case 2: return pick(std::integral_constant<int, 2>());
-    case 3: return pick(std::integral_constant<int, 3>());
-    default: return pick(std::integral_constant<int, 4>());
-  }
+                                     int32_t* out_start, const WalkShape& sh, cudaStream_t st) {
+  return for_model(c, [&](auto nd, auto cal) {
+    constexpr int N = decltype(nd)::value;
+    constexpr bool C = decltype(cal)::value;
+    return sh.wide ? run_walk_fused<N, C, 16>(c, val, sc, live_u, live_lnl, K, seed, n_chains, walk_len, chol, out_u,
+                                              out_lnl, out_nacc, out_start, sh, st)
+                   : run_walk_fused<N, C, 8>(c, val, sc, live_u, live_lnl, K, seed, n_chains, walk_len, chol, out_u,
+                                             out_lnl, out_nacc, out_start, sh, st);
+  });
 }
 
 // ns_replace's walk in the one-kernel form, its scalars passed by value; false
@@ -1095,15 +1209,15 @@ bool launch_walk_direct(gwl_ctx* c, const double* live_u, const double* live_lnl
                         double lstar, uint64_t seed, uint64_t counter, int64_t n_chains, int walk_len, double scale,
                         const double* chol, double* out_u, double* out_lnl, int32_t* out_nacc, int32_t* out_start,
                         cudaStream_t st, cudaError_t* e) {
-  int grid, rows, nwc;
-  if (!walk_fused_shape(c, n_chains, &grid, &rows, &nwc)) return false;
+  WalkShape sh;
+  if (!walk_fused_shape(c, n_chains, &sh)) return false;
   WalkScalars v;
   v.lstar = lstar;
   v.scale = scale;
   v.worst = worst;
   v.counter = counter;
   *e = launch_walk_fused(c, v, nullptr, live_u, live_lnl, K, seed, n_chains, walk_len, chol, out_u, out_lnl, out_nacc,
-                         out_start, grid, rows, nwc, st);
+                         out_start, sh, st);
   return true;
 }
 
@@ -1117,10 +1231,10 @@ cudaError_t launch_walk(gwl_ctx* c, const double* live_u, const double* live_lnl
   if (c->walk_kind == GWL_WALK_GALILEAN)
     return launch_gmc(c, live_u, live_lnl, K, sc, seed, n_chains, walk_len, chol, out_u, out_lnl, out_nacc,
                       out_start, pu, pth, plnl, st);
-  int grid, rows, nwc;
-  if (walk_fused_shape(c, n_chains, &grid, &rows, &nwc))
+  WalkShape sh;
+  if (walk_fused_shape(c, n_chains, &sh))
     return launch_walk_fused(c, WalkScalars(), sc, live_u, live_lnl, K, seed, n_chains, walk_len, chol, out_u, out_lnl,
-                             out_nacc, out_start, grid, rows, nwc, st);
+                             out_nacc, out_start, sh, st);
   const int D = (int)theta_stride(c);
   const unsigned nb = (unsigned)((n_chains + 127) / 128);
   const PriorInfo pr = prior_info(c);
