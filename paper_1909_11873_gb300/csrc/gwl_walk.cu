@@ -753,11 +753,24 @@ __device__ __forceinline__ double key_lnl(long long k) {
 }
 
 // Consumption of the round's candidates.  The sequential replacement loop
-// (warp 0) touches only shared memory: the order keys of the live lnL and of
-// the candidates' lnL and, per live slot, where its point currently comes from
-// (an original live point or a candidate); it records each dead point's lnL
-// and slot.  The dead points' prior weights, the unit-cube coordinates of
-// dead points and of the replaced slots are then written by the whole CTA.
+// (warp 0) touches only shared memory and registers: the order keys of the
+// live lnL and, per live slot, where its point currently comes from (an
+// original live point or a candidate); it records each dead point's lnL and
+// slot.  Slot k belongs to lane k mod 32, which keeps the smallest of its slots
+// in registers and reads them again only when one of them has been replaced
+// (alone up to kRescanSlots live points, with the whole warp beyond);
+// the worst point is then the smallest of 32 keys (three 32-bit warp
+// reductions: the key's halves and the slot), and the next candidate above it
+// comes from a ballot over 32 candidates held in registers.  What bounds it is
+// that chain of one warp per dead point.  A round of the 4 s event (250 live
+// points, 250 chains, walk 20) outside its walk, consumption and statistics in
+// one launch: 63 us against 142 with every slot read again per dead point and
+// two launches.  Whole rounds of 1000 / 4000 live points and chains: 0.52 / 2.5
+// ms against 0.68 / 6.0 with one lane reading its slots again, and 1.55 / 9.1
+// with every slot read per dead point (and the walk in separate kernels).  The
+// dead points' prior weights, the unit-cube coordinates of dead points and of the
+// replaced slots are then written by the whole CTA.
+constexpr int kRescanSlots = 384;
 __device__ void ns_consume_body(const NsDev& s) {
   if (s.stats[NS_DONE] > 0.5) return;
   extern __shared__ __align__(16) unsigned char smc[];
@@ -778,38 +791,74 @@ __device__ void ns_consume_body(const NsDev& s) {
   __syncthreads();
   const int64_t nd0 = (int64_t)s.stats[NS_NDEAD];
   if (t < 32) {
-    int64_t ptr = 0;
-    int nrep = 0;
-    while (true) {
-      long long bv = 0x7fffffffffffffffll;
-      int bi = 0;
-      for (int k = lane; k < s.K; k += 32) {
+    const int K = (int)s.K, n = (int)s.n_chains;
+    // the lane's smallest slot (the lowest index among equal keys)
+    long long mv = 0x7fffffffffffffffll;
+    int mi = 0x7fffffff;
+    auto rescan = [&]() {
+      mv = 0x7fffffffffffffffll;
+      mi = 0x7fffffff;
+#pragma unroll 4
+      for (int k = lane; k < K; k += 32) {
         const long long v = ll[k];
-        if (v < bv || (v == bv && k < bi)) {
-          bv = v;
-          bi = k;
+        if (v < mv || mi == 0x7fffffff) {
+          mv = v;
+          mi = k;
         }
       }
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) {
-        const long long v = __shfl_xor_sync(0xffffffffu, bv, off);
-        const int i = __shfl_xor_sync(0xffffffffu, bi, off);
-        if (v < bv || (v == bv && i < bi)) {
-          bv = v;
-          bi = i;
-        }
+    };
+    rescan();
+    int nrep = 0, base = 0;         // candidates [base, base + 32) are in registers
+    unsigned left = 0xffffffffu;    // those not yet passed over
+    long long cv = lane < n ? cl[lane] : 0;
+    while (true) {
+      const int hi = (int)(mv >> 32);
+      const int mh = __reduce_min_sync(0xffffffffu, hi);
+      const unsigned lo = hi == mh ? (unsigned)mv : 0xffffffffu;
+      const unsigned ml = __reduce_min_sync(0xffffffffu, lo);
+      const bool at = hi == mh && (unsigned)mv == ml;
+      const int bi = __reduce_min_sync(0xffffffffu, at ? mi : 0x7fffffff);
+      const long long bv = (long long)(((unsigned long long)(unsigned)mh << 32) | ml);
+      // the next candidate above the worst live point
+      unsigned up;
+      while (true) {
+        up = __ballot_sync(0xffffffffu, base + lane < n && cv > bv) & left;
+        if (up || base + 32 >= n) break;
+        base += 32;
+        left = 0xffffffffu;
+        cv = base + lane < n ? cl[base + lane] : 0;
       }
-      while (ptr < s.n_chains && !(cl[ptr] > bv)) ++ptr;
-      if (ptr >= s.n_chains) break;
-      if (lane == 0) {
+      if (!up) break;
+      const int c = __ffs(up) - 1;
+      left = c == 31 ? 0u : 0xffffffffu << (c + 1);
+      const long long nv = __shfl_sync(0xffffffffu, cv, c);
+      if (lane == (bi & 31)) {  // the slot's lane records the dead point and takes the candidate
         s.rl[nrep] = key_lnl(bv);
         rslot[nrep] = bi;
         rsrc[nrep] = src[bi];
-        src[bi] = (int)ptr;
-        ll[bi] = cl[ptr];
+        src[bi] = base + c;
+        ll[bi] = nv;
+        if (K <= kRescanSlots) rescan();
       }
       __syncwarp();
-      ++ptr;
+      if (K > kRescanSlots) {  // the warp reads that lane's slots together
+        long long v = 0x7fffffffffffffffll;
+        int vi = 0x7fffffff;
+        for (int k = (bi & 31) + 32 * lane; k < K; k += 1024) {
+          const long long x = ll[k];
+          if (x < v || vi == 0x7fffffff) {
+            v = x;
+            vi = k;
+          }
+        }
+        const int h2 = __reduce_min_sync(0xffffffffu, (int)(v >> 32));
+        const unsigned l2 = __reduce_min_sync(0xffffffffu, (int)(v >> 32) == h2 ? (unsigned)v : 0xffffffffu);
+        const int i2 = __reduce_min_sync(0xffffffffu, (int)(v >> 32) == h2 && (unsigned)v == l2 ? vi : 0x7fffffff);
+        if (lane == (bi & 31)) {
+          mv = (long long)(((unsigned long long)(unsigned)h2 << 32) | l2);
+          mi = i2;
+        }
+      }
       ++nrep;
     }
     if (lane == 0) sh_nrep = nrep;
@@ -964,12 +1013,19 @@ __device__ void ns_final_body(const NsDev& s) {
 
 // One event (parameters by value) or E events (one CTA per event).
 __global__ void __launch_bounds__(256) k_ns_prep(NsDev s) { ns_prep_body(s); }
-__global__ void __launch_bounds__(256) k_ns_consume(NsDev s) { ns_consume_body(s); }
-__global__ void __launch_bounds__(256) k_ns_stats(NsDev s, int walk_len, double dlogz) { ns_stats_body(s, walk_len, dlogz); }
+// The round's consumption and its statistics: one launch.  Dynamic shared
+// memory above kCloseSmem needs the raised limit (48 KB less the statics).
+constexpr size_t kCloseSmem = 40 * 1024;
+__global__ void __launch_bounds__(256) k_ns_close(NsDev s, int walk_len, double dlogz) {
+  ns_consume_body(s);
+  __syncthreads();
+  ns_stats_body(s, walk_len, dlogz);
+}
 __global__ void __launch_bounds__(256) k_ns_final(NsDev s) { ns_final_body(s); }
 __global__ void __launch_bounds__(256) k_mns_prep(const NsDev* a) { ns_prep_body(a[blockIdx.x]); }
-__global__ void __launch_bounds__(256) k_mns_consume(const NsDev* a) { ns_consume_body(a[blockIdx.x]); }
-__global__ void __launch_bounds__(256) k_mns_stats(const NsDev* a, int walk_len, double dlogz) {
+__global__ void __launch_bounds__(256) k_mns_close(const NsDev* a, int walk_len, double dlogz) {
+  ns_consume_body(a[blockIdx.x]);
+  __syncthreads();
   ns_stats_body(a[blockIdx.x], walk_len, dlogz);
 }
 __global__ void __launch_bounds__(256) k_mns_final(const NsDev* a) { ns_final_body(a[blockIdx.x]); }
@@ -1280,10 +1336,9 @@ cudaError_t launch_ns_round(gwl_ctx* c, const NsDev& s, uint64_t seed, int walk_
                   plnl, st);
   if (e != cudaSuccess) return e;
   const size_t csm = consume_smem_bytes(s.K, s.n_chains);
-  if (csm > 48 * 1024 && (e = raise_smem_limit((const void*)k_ns_consume, c->device, csm)) != cudaSuccess) return e;
-  k_ns_consume<<<1, 256, csm, st>>>(s);
-  k_ns_stats<<<1, 256, 0, st>>>(s, walk_len, dlogz);
-  c->launches += 2;
+  if (csm > kCloseSmem && (e = raise_smem_limit((const void*)k_ns_close, c->device, csm)) != cudaSuccess) return e;
+  k_ns_close<<<1, 256, csm, st>>>(s, walk_len, dlogz);
+  c->launches++;
   return cudaGetLastError();
 }
 
@@ -1672,8 +1727,8 @@ static int multi_ns_run_on(Multi* m, int64_t K, int64_t n_chains, int walk_len, 
     }
     // one round, captured
     const size_t csm = consume_smem_bytes(K, n_chains);
-    if (csm > 48 * 1024) {
-      if ((e = cudaFuncSetAttribute(k_mns_consume, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csm)) !=
+    if (csm > kCloseSmem) {
+      if ((e = cudaFuncSetAttribute(k_mns_close, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csm)) !=
           cudaSuccess)
         break;
     }
@@ -1691,8 +1746,7 @@ static int multi_ns_run_on(Multi* m, int64_t K, int64_t n_chains, int walk_len, 
         er = multi_loglike(m, pth, n_chains, plnl, st);
         k_mwalk_accept<<<nb, 128, 0, st>>>(d_ns, n_chains, E, pu, plnl);
       }
-      k_mns_consume<<<E, 256, csm, st>>>(d_ns);
-      k_mns_stats<<<E, 256, 0, st>>>(d_ns, walk_len, dlogz);
+      k_mns_close<<<E, 256, csm, st>>>(d_ns, walk_len, dlogz);
       cudaError_t ec = cudaStreamEndCapture(st, &graph);
       e = er != cudaSuccess ? er : ec;
     }
@@ -1705,7 +1759,7 @@ static int multi_ns_run_on(Multi* m, int64_t K, int64_t n_chains, int walk_len, 
       const int64_t todo = (max_rounds - r) < check ? (max_rounds - r) : check;
       for (int64_t i = 0; i < todo && e == cudaSuccess; ++i) {
         e = cudaGraphLaunch(gexec, st);
-        multi_count(m, 5 + 5 * (int64_t)walk_len);
+        multi_count(m, 4 + 5 * (int64_t)walk_len);
       }
       if (e != cudaSuccess) break;
       r += todo;
