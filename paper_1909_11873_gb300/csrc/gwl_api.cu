@@ -361,7 +361,7 @@ int gwl_loglike(gwl_ctx* c, const double* theta_dev, int64_t B, double* lnl_dev,
   if (B < 0) return fail(GWL_ERR_ARG, "B < 0");
   if (B == 0) return GWL_OK;
   if (!theta_dev || !lnl_dev) return fail(GWL_ERR_ARG, "null device pointer");
-  if (!gwl::fused_used(c, B) && (rc = ensure_scratch(c, B))) return rc;  // the one-kernel form needs no scratch
+  if (!gwl::fused_used(c, B) && !gwl::fused64_used(c, B) && (rc = ensure_scratch(c, B))) return rc;  // the one-kernel form needs no scratch
   cudaStream_t st = (cudaStream_t)stream;
   c->last_stream = st;
   cudaError_t e = gwl::launch_loglike(c, theta_dev, B, lnl_dev, st);

@@ -143,6 +143,9 @@ bool fused_shape(const gwl_ctx* c, int64_t B, int* grid, int* rows, int* nwc);
 int fused_window_count(const gwl_ctx* c);
 int fused_windows(const gwl_ctx* c, int R, size_t room);
 bool fused_used(const gwl_ctx* c, int64_t B);
+// the FP64 one-kernel form (gwl_fused64.cu)
+bool fused64_used(const gwl_ctx* c, int64_t B);
+cudaError_t launch_fused64(gwl_ctx* c, const double* theta, int64_t B, double* lnl, cudaStream_t st);
 cudaError_t launch_fused(gwl_ctx* c, const double* theta, int64_t B, double* lnl, int grid, int rows, int nwc,
                          cudaStream_t st);
 // the lane-per-proposal bin loop (gwl_lanes.cu): chunk size (0: not used), scratch sizes, launch

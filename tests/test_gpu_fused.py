@@ -122,3 +122,41 @@ def test_one_kernel_walk_matches_separate_kernels(n_det, source, nodes, walk):
             assert torch.equal(a, b[:n])
     ctx.gwl_sync()
     ctx.close()
+
+
+@pytest.mark.parametrize("n_det,T,source,fcut", [(3, 8.0, "bbh", 0), (1, 4.0, "bbh", 0), (4, 4.0, "bns", 1), (2, 16.0, "bbh", 0)])
+def test_one_kernel_fp64_at_every_shape(n_det, T, source, fcut):
+    """The FP64 one-kernel form at the batch sizes where its shape changes (clusters of eight, four and two CTAs,
+    one CTA per group, 32 rows, two waves) against one batch in another shape: on the 16 s segment the separate
+    kernels.  FP64 sums in another order: about 1e4 terms of up to 10 each, 1e4 * 2^-53 * 1e3 < 2e-9."""
+    from paper_1909_11873_gb300 import gwl as g
+
+    cfg = dict(n_det=n_det, T=T, f_low=20.0, f_high=1024.0, noise=True, source=source, gmst=1.7)
+    ev = custom_event(cfg, 4, fcut_mode=fcut)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    n = 8 * sms - 1
+    th = I.reduced(I.proposals(ev, n, 10), ev.sampling)
+    th[5, 1] = 1.5
+    th[-1, 0] = np.nan
+    th[31, 0] = 400.0
+    x = torch.from_numpy(th).cuda()
+    ctx = g.Context.from_event(ev, g.GWL_FP64)
+    ref, k = launches(ctx, lambda: g.loglike(ctx, x))
+    assert k == (3 if T == 16.0 else 1)
+    ok = ~torch.isinf(ref)
+    sizes = [1, 2, sms * 2 // 19, sms * 2 // 19 + 1, sms * 4 // 19 + 1, sms // 2, sms // 2 + 1, sms, sms + 1, 2 * sms, 2 * sms + 1]
+    for B in sizes if T != 16.0 else []:
+        got, k = launches(ctx, lambda: g.loglike(ctx, x[:B].contiguous()))
+        again = g.loglike(ctx, x[:B].contiguous())
+        assert k == 1 and torch.equal(got, again)
+        assert torch.equal(torch.isinf(got), ~ok[:B])
+        d = (got - ref[:B])[ok[:B]].abs()
+        assert d.numel() == 0 or float(d.max()) < 2e-9, f"B={B}: {float(d.max()):.3e}"
+    for times in (2, 5, 33):  # from a row per warp to two waves of 32 rows per SM
+        got, k = launches(ctx, lambda: g.loglike(ctx, x.repeat(times, 1)[: times * n if times < 33 else 32 * sms + 5]))
+        assert k == 1
+        want = ref.repeat(times)[: got.numel()]
+        assert torch.equal(torch.isinf(got), torch.isinf(want))
+        assert float((got - want)[~torch.isinf(want)].abs().max()) < 2e-9
+    ctx.gwl_sync()
+    ctx.close()
