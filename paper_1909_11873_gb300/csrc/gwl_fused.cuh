@@ -309,6 +309,27 @@ __device__ __forceinline__ void fused_amplitudes(const SegInfo& s, FusedSmem<NDE
   sm.hterm[d][lane] = (kr * kr + ki * ki) * ff_from(H);
 }
 
+// The anchor record of a (row, block): the row's anchor terms at the block's
+// anchor row ra, and whether the block takes the FP32 delta.
+template <int NDET>
+__device__ __forceinline__ void anchor_record(const PropMixed& P, const float* __restrict__ ra, float* __restrict__ o) {
+  float ch[kNBasis], cl[kNBasis], th[NDET], tl[NDET], an[NDET];
+#pragma unroll
+  for (int m = 0; m < kNBasis; ++m) {
+    ch[m] = P.ch[m];
+    cl[m] = P.cl[m];
+  }
+#pragma unroll
+  for (int d = 0; d < NDET; ++d) {
+    th[d] = P.th[d];
+    tl[d] = P.tl[d];
+  }
+  const bool fast = anchor_terms<NDET>(ra, ch, cl, th, tl, an);
+#pragma unroll
+  for (int d = 0; d < NDET; ++d) o[d] = an[d];
+  o[NDET] = fast ? 1.0f : 0.0f;
+}
+
 // Warp sums of n FP32 values per lane with the tree of an xor butterfly over
 // 16, 8, 4, 2, 1: at each level a lane keeps one half of its values and hands
 // the other half to its partner, so that value v is added up by the lanes
@@ -346,9 +367,10 @@ __device__ __forceinline__ float warp_fold(const float (&v)[N], int lane) {
 // FP32 sums of one row over bins [jl, jl + n) of the staged windows (jl a
 // multiple of 32, in bins from the first staged one; j0 that one's index in
 // the segment): the blocks in order, lanes over a block's bins, as
-// anchored_sums_cal.
-template <int NDET, bool CAL>
-__device__ __forceinline__ void fused_row_sums(const FusedArgs& a, const FusedLayout& L, const float* __restrict__ dyn,
+// anchored_sums_cal.  cal: the staged windows' calibration rows.  A: the
+// segment's delta rows (rows, row_elems), df, cal_row and ffc.
+template <int NDET, bool CAL, class A>
+__device__ __forceinline__ void fused_row_sums(const A& a, const float* __restrict__ dyn, const float* __restrict__ cal,
                                                const PropMixed& P, const float* __restrict__ rec, int j0, int jl, int n,
                                                int lane, const float4* __restrict__ nodes, float (&U)[NDET],
                                                float (&V)[NDET], float (&X)[NDET]) {
@@ -380,7 +402,7 @@ __device__ __forceinline__ void fused_row_sums(const FusedArgs& a, const FusedLa
   };
   constexpr int BF = block_floats(NDET);
   const float* row = dyn + jl / kAnchor * BF + 4 * lane;
-  const float* crow = CAL ? dyn + L.cal + (jl + lane) * a.cal_row : nullptr;
+  const float* crow = CAL ? cal + (jl + lane) * a.cal_row : nullptr;
   const int cstep = CAL ? kAnchor * a.cal_row : 0;
   CalBin<NDET, float> cb0, cb1;
   const int nblk = (n + kAnchor - 1) / kAnchor;
@@ -474,24 +496,8 @@ __device__ __forceinline__ bool fused_bins(const FusedArgs& a, const FusedLayout
     const int nb = (top + kAnchor - 1) / kAnchor;
     for (int i = t; i < R * nb; i += 32 * NW) {
       const int r = i / nb, b = i - r * nb;
-      if (j0 + b * kAnchor >= sm.ncut[r]) continue;
-      float ch[kNBasis], cl[kNBasis], th[NDET], tl[NDET], an[NDET];
-      const PropMixed& P = sm.pm[r];
-#pragma unroll
-      for (int m = 0; m < kNBasis; ++m) {
-        ch[m] = P.ch[m];
-        cl[m] = P.cl[m];
-      }
-#pragma unroll
-      for (int d = 0; d < NDET; ++d) {
-        th[d] = P.th[d];
-        tl[d] = P.tl[d];
-      }
-      const bool fast = anchor_terms<NDET>(dyn + L.anchor + b * kAnchorRowFloats, ch, cl, th, tl, an);
-      float* o = dyn + L.rec + (r * gblk + b) * AR;
-#pragma unroll
-      for (int d = 0; d < NDET; ++d) o[d] = an[d];
-      o[NDET] = fast ? 1.0f : 0.0f;
+      if (j0 + b * kAnchor < sm.ncut[r])
+        anchor_record<NDET>(sm.pm[r], dyn + L.anchor + b * kAnchorRowFloats, dyn + L.rec + (r * gblk + b) * AR);
     }
     if (t == 0) sm.next = 0;
     group_sync<NW>();
@@ -515,7 +521,7 @@ __device__ __forceinline__ bool fused_bins(const FusedArgs& a, const FusedLayout
       float4* nodes = sm.nodes + (CAL ? warp * NDET * kMaxCalNodes : 0);
       if constexpr (CAL) cal_nodes_fill<NDET, true>(crow(r), a.nn, a.calQ, lane, nodes);
       float U[NDET], V[NDET], X[NDET], v[NS];
-      fused_row_sums<NDET, CAL>(a, L, dyn, sm.pm[r], dyn + L.rec + (r * gblk + jl / kAnchor) * AR, j0, jl, n, lane,
+      fused_row_sums<NDET, CAL>(a, dyn, dyn + L.cal, sm.pm[r], dyn + L.rec + (r * gblk + jl / kAnchor) * AR, j0, jl, n, lane,
                                 nodes, U, V, X);
 #pragma unroll
       for (int d = 0; d < NDET; ++d) {

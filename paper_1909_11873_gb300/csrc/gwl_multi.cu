@@ -7,7 +7,8 @@
 // persistent: its CTAs take (event, window) tasks from one atomic queue,
 // stage that event's window of table rows in shared memory (cp.async.bulk on
 // an mbarrier, bounded wait) and drain that event's per-window proposal
-// counter; events with 4 s and 128 s segments thus share one launch.  With
+// counter (FP64), or take (event, window, part of the proposals) tasks (mixed);
+// events with 4 s and 128 s segments thus share one launch.  With
 // the calibration model (every context of the batch with the same number of
 // nodes, each with its own node frequencies and tables) the window's
 // calibration rows are staged beside its table rows and each proposal's
@@ -18,8 +19,7 @@
 #include <cmath>
 #include <vector>
 
-#include "gwl_bins.cuh"
-#include "gwl_ff.cuh"
+#include "gwl_fused.cuh"
 
 namespace gwl {
 
@@ -27,6 +27,7 @@ struct EvDesc {
   SegInfo seg;
   const void* tab;     // delta table (mixed) or FP64 table of this event
   const float* anchor; // anchor rows (mixed)
+  const float* blk;    // blocked table (mixed)
   float df;
   int row_elems;
   int CH;              // window (bins)
@@ -247,35 +248,237 @@ __global__ void __launch_bounds__(256, 2) k_mwindow(MultiArgs a) {
   }
 }
 
+// ---------------------------------------------------------------- mixed bin loop
+// The same sums for the mixed path, with the row code of gwl_fused.cuh.  A task
+// is up to kTaskRows proposals of one (event, window): the CTA stages the
+// window's part of the blocked table, reads the proposals' coefficients, forms
+// their anchor records one (proposal, block) per thread, and its warps take
+// proposals.  Tasks come from one counter through prefix sums over the events,
+// formed once per CTA.
+//
+// Against whole (event, window) tasks with per-proposal claims, whose 500
+// proposals kept one CTA busy for 250 us (the last tasks ended alone), and the
+// bin loop's per-proposal work (a warp's anchor pass, 30-shuffle reductions):
+// 500 proposals of each of 12 events of 4 to 128 s, 3 detectors, the bin loop 718
+// -> 430 us (cold, serialised; issue active 66 %, short-scoreboard the top stall:
+// the hardware sine and cosine and the shared-memory reads), the call 631-730 ->
+// 356-395 us with the finalisation below and a warp per CTA in the prologue.
+constexpr int kTaskRows = 64;
+constexpr size_t kRowsSmem = 200 * 1024;  // its dynamic shared memory at most (227 KB less the statics)
+constexpr int kMaxPrefix = 1024;  // events whose prefix sums fit shared memory
+
+// What fused_row_sums needs of an event.
+struct RowTab {
+  const float* rows;
+  int row_elems;
+  float df;
+  int cal_row;
+  unsigned long long* ffc;
+};
+
+template <int NDET, bool CAL>
+__global__ void __launch_bounds__(256, 2) k_mrows(MultiArgs a, int CHmax, int calmax) {
+  constexpr int S = CAL ? 3 : 2, NS = S * NDET, AR = anchor_rec_floats(NDET);
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  __shared__ __align__(8) uint64_t bar;
+  __shared__ int s_pre[kMaxPrefix + 1];  // (event, window) pairs before event e
+  __shared__ int s_task, s_next, s_fail;
+  __shared__ PropMixed s_pm[kTaskRows];
+  __shared__ int s_cut[kTaskRows];
+  __shared__ __align__(16) float4 s_nodes[CAL ? 8 * NDET * kMaxCalNodes : 1];
+  const int blocks = CHmax / kAnchor + (CHmax % kAnchor != 0);
+  float* tab = reinterpret_cast<float*>(smem_raw);
+  float* anc = tab + blocks * block_floats(NDET);
+  float* cal = anc + blocks * kAnchorRowFloats;
+  float* rec = cal + (CAL ? ((CHmax + 2) * calmax + 3) / 4 * 4 : 0);
+  const int t = threadIdx.x, lane = t & 31;
+  auto windows = [&](int e) {
+    const EvDesc& d = a.ev[e];
+    const int nw = (a.work[d.work_off] + d.CH - 1) / d.CH;
+    return nw < d.nw_total ? nw : d.nw_total;
+  };
+  const bool prefix = a.E <= kMaxPrefix;
+  if (prefix) {
+    for (int e = t; e < a.E; e += 256) s_pre[e + 1] = windows(e);
+    __syncthreads();
+    if (t < 32) {  // inclusive sums, 32 events at a time
+      int run = 0;
+      for (int e0 = 0; e0 < a.E; e0 += 32) {
+        int v = e0 + lane < a.E ? s_pre[e0 + lane + 1] : 0;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+          const int y = __shfl_up_sync(0xffffffffu, v, off);
+          if (lane >= off) v += y;
+        }
+        if (e0 + lane < a.E) s_pre[e0 + lane + 1] = run + v;
+        run += __shfl_sync(0xffffffffu, v, 31);
+      }
+      if (lane == 0) s_pre[0] = 0;
+    }
+  }
+  if (t == 0) {
+    s_fail = 0;
+    mbar_init(&bar, 1);
+    fence_mbar_init();
+    s_task = atomicAdd(a.task_counter, 1);
+  }
+  __syncthreads();
+  const int parts = (int)((a.n_per + kTaskRows - 1) / kTaskRows);
+  uint32_t parity = 0;
+  while (true) {
+    const int task = s_task;
+    // task -> (event, window, part), the parts of a window next to each other
+    const int pair = task / parts, part = task - pair * parts;
+    int e = -1, w = 0;
+    if (prefix) {
+      if (pair < s_pre[a.E]) {
+        int lo = 0, hi = a.E;
+        while (hi - lo > 1) {
+          const int mid = (lo + hi) >> 1;
+          if (s_pre[mid] <= pair) lo = mid;
+          else hi = mid;
+        }
+        e = lo;
+        w = pair - s_pre[lo];
+      }
+    } else {
+      int q = pair;
+      for (int k = 0; k < a.E && e < 0; ++k) {
+        const int nw = windows(k);
+        if (q < nw) {
+          e = k;
+          w = q;
+        }
+        q -= nw;
+      }
+    }
+    if (e < 0) break;  // no task left (uniform across the CTA)
+    const EvDesc& d = a.ev[e];
+    const int maxn = a.work[d.work_off];
+    const int j0 = w * d.CH;
+    int64_t j1l = (int64_t)j0 + d.CH;
+    if (j1l > d.seg.M) j1l = d.seg.M;
+    if (j1l > maxn) j1l = maxn;
+    const int nbins = (int)j1l - j0, nb = (nbins + kAnchor - 1) / kAnchor;
+    if (t == 0) {
+      fence_proxy_async_smem();
+      const uint32_t bytes = (uint32_t)nb * (uint32_t)(block_floats(NDET) * 4);
+      const uint32_t abytes = (uint32_t)nb * (uint32_t)(kAnchorRowFloats * 4);
+      // calibration rows in pairs: a bulk copy moves whole 16-byte units (the table has a row past the last bin)
+      const uint32_t cbytes = CAL ? (uint32_t)((nbins + 1) & ~1) * (uint32_t)d.cal_row * 4u : 0u;
+      mbar_arrive_expect_tx(&bar, bytes + abytes + cbytes);
+      bulk_g2s(tab, d.blk + (int64_t)(j0 / kAnchor) * block_floats(NDET), bytes, &bar);
+      bulk_g2s(anc, d.anchor + (int64_t)(j0 / kAnchor) * kAnchorRowFloats, abytes, &bar);
+      if constexpr (CAL) bulk_g2s(cal, reinterpret_cast<const float*>(d.cal) + (int64_t)j0 * d.cal_row, cbytes, &bar);
+      s_next = 0;
+    }
+    const int64_t r0 = (int64_t)part * kTaskRows, p0 = (int64_t)e * a.n_per + r0;
+    const int n = a.n_per - r0 < kTaskRows ? (int)(a.n_per - r0) : kTaskRows;
+    for (int i = t; i < n * (int)(sizeof(PropMixed) / 16); i += 256)
+      reinterpret_cast<float4*>(s_pm)[i] = reinterpret_cast<const float4*>(reinterpret_cast<const PropMixed*>(a.prop) + p0)[i];
+    for (int i = t; i < n; i += 256) s_cut[i] = a.pc[p0 + i].ncut;
+    __syncthreads();
+    if (!mbar_wait_bounded(&bar, parity, a.status)) s_fail = 1;
+    parity ^= 1u;
+    for (int i = t; i < n * nb; i += 256) {
+      const int r = i / nb, b = i - r * nb;
+      if (j0 + b * kAnchor < s_cut[r])
+        anchor_record<NDET>(s_pm[r], anc + b * kAnchorRowFloats, rec + (r * blocks + b) * AR);
+    }
+    __syncthreads();
+    if (s_fail) return;
+    if (t == 0) s_task = atomicAdd(a.task_counter, 1);
+    const RowTab rt{reinterpret_cast<const float*>(d.tab), d.row_elems, d.df, d.cal_row, nullptr};
+    while (true) {
+      int r = 0;
+      if (lane == 0) r = atomicAdd(&s_next, 1);
+      r = __shfl_sync(0xffffffffu, r, 0);
+      if (r >= n) break;
+      int nr = s_cut[r] - j0;
+      if (nr <= 0) continue;
+      if (nr > nbins) nr = nbins;
+      float4* nodes = s_nodes + (CAL ? (t >> 5) * NDET * kMaxCalNodes : 0);
+      if constexpr (CAL) cal_nodes_fill<NDET, true>(a.theta + (p0 + r) * a.stride + a.cal_par, d.nn, d.calQ, lane, nodes);
+      float U[NDET], V[NDET], X[NDET], v[NS];
+      fused_row_sums<NDET, CAL>(rt, tab, cal, s_pm[r], rec + r * blocks * AR, j0, 0, nr, lane, nodes, U, V, X);
+#pragma unroll
+      for (int q = 0; q < NDET; ++q) {
+        v[S * q] = U[q];
+        v[S * q + 1] = V[q];
+        if constexpr (CAL) v[S * q + 2] = X[q];
+      }
+      const float s = warp_fold<NS>(v, lane);
+      constexpr int W = FoldP<NS>::W;
+      if (lane % W == 0 && lane / W < NS)
+        reinterpret_cast<float*>(a.partials)[d.part_off + ((r0 + r) * d.nw_total + w) * NS + lane / W] = s;
+    }
+    __syncthreads();  // all warps are done with this task's rows
+  }
+}
+
+// A window sum widened to FP64; a normal float by its bits, as the conversion
+// instruction holds the narrow FP64 unit.
+__device__ __forceinline__ double widen(float f) {
+  const unsigned e = (__float_as_uint(f) >> 23) & 0xFFu;
+  return e == 0u || e == 0xFFu ? (double)f : f2d_bits(f);
+}
+__device__ __forceinline__ double widen(double f) { return f; }
+
+// lnL of a proposal from its windows' sums: one warp, lanes over windows, then
+// a fixed fold over the lanes (FP64; value k ends on the lanes whose upper
+// bits spell k, see warp_fold).  Bound by the FP64 pipe: one add per lane and
+// window, nine for the fold.  (One thread per proposal walking its up to 200
+// windows took 112 us for 6000 proposals; 27 us now.)
 template <int NDET, typename Acc, bool CAL>
-__global__ void k_mfinalize(const EvDesc* __restrict__ ev, int64_t n_per, int64_t B, const PropCommon* __restrict__ pc,
-                            const Acc* __restrict__ partials, double* __restrict__ lnl) {
-  constexpr int S = CAL ? 3 : 2;
-  const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(256) k_mfinalize(const EvDesc* __restrict__ ev, int64_t n_per, int64_t B,
+                                                   const PropCommon* __restrict__ pc,
+                                                   const Acc* __restrict__ partials, double* __restrict__ lnl) {
+  constexpr int S = CAL ? 3 : 2, NS = S * NDET;
+  const int64_t p = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
   if (p >= B) return;
   const int e = (int)(p / n_per);
   const int64_t pi = p - (int64_t)e * n_per;
   const EvDesc& d = ev[e];
   const PropCommon c = pc[p];
   if (c.flag) {
-    lnl[p] = -INFINITY;
+    if (lane == 0) lnl[p] = -INFINITY;
     return;
   }
   const int nwp = (c.ncut + d.CH - 1) / d.CH;
-  const Acc* q = partials + d.part_off + pi * d.nw_total * (S * NDET);
+  const Acc* q = partials + d.part_off + pi * d.nw_total * NS;
+  double x[NS];
+#pragma unroll
+  for (int k = 0; k < NS; ++k) x[k] = 0.0;
+  for (int w = lane; w < nwp; w += 32)
+#pragma unroll
+    for (int k = 0; k < NS; ++k) x[k] += widen(q[w * NS + k]);
+  constexpr int P = FoldP<NS>::P, W = FoldP<NS>::W;
+  double t[P];
+#pragma unroll
+  for (int k = 0; k < P; ++k) t[k] = k < NS ? x[k < NS ? k : 0] : 0.0;
+  int off = 16;
+#pragma unroll
+  for (int h = P / 2; h >= 1; h >>= 1, off >>= 1) {
+    const bool up = (lane & off) != 0;
+#pragma unroll
+    for (int k = 0; k < h; ++k) {
+      const double send = up ? t[k] : t[k + h];
+      const double keep = up ? t[k + h] : t[k];
+      t[k] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+    }
+  }
+#pragma unroll
+  for (; off >= 1; off >>= 1) t[0] += __shfl_xor_sync(0xffffffffu, t[0], off);
+#pragma unroll
+  for (int k = 0; k < NS; ++k) x[k] = __shfl_sync(0xffffffffu, t[0], k * W);
   double acc = 0.0;
 #pragma unroll
   for (int k = 0; k < NDET; ++k) {
-    double U = 0.0, V = 0.0, X = 0.0;
-    for (int w = 0; w < nwp; ++w) {
-      U += (double)q[w * (S * NDET) + S * k];
-      V += (double)q[w * (S * NDET) + S * k + 1];
-      if constexpr (CAL) X += (double)q[w * (S * NDET) + S * k + 2];
-    }
-    acc += c.Kr[k] * U - c.Ki[k] * V;
-    if constexpr (CAL) acc -= 0.5 * (c.Kr[k] * c.Kr[k] + c.Ki[k] * c.Ki[k]) * X;
+    acc += c.Kr[k] * x[S * k] - c.Ki[k] * x[S * k + 1];
+    if constexpr (CAL) acc -= 0.5 * (c.Kr[k] * c.Kr[k] + c.Ki[k] * c.Ki[k]) * x[S * k + 2];
   }
-  lnl[p] = acc - 0.5 * c.hh;
+  if (lane == 0) lnl[p] = acc - 0.5 * c.hh;
 }
 
 // ---------------------------------------------------------------- host side
@@ -339,6 +542,7 @@ cudaError_t multi_prepare(Multi* m, int64_t n_per) {
     d.seg = c->seg;
     d.tab = mixed ? (const void*)c->d_tab_delta : (const void*)c->d_tab_f64;
     d.anchor = c->d_anchor;
+    d.blk = c->d_tab_block;
     d.df = (float)c->df;
     d.row_elems = mixed ? c->row_delta : c->row_doubles;
     int CH = c->window;
@@ -383,7 +587,8 @@ static cudaError_t multi_run(Multi* m, const double* theta, int64_t n_per, doubl
   const int64_t B = n_per * m->E;
   cudaError_t e = cudaMemsetAsync(m->work, 0, sizeof(int) * m->work_len, st);
   if (e != cudaSuccess) return e;
-  k_mprologue<MIXED><<<(unsigned)((B + 127) / 128), 128, 0, st>>>(m->d_ev, n_per, B, theta, m->pm, m->pf, m->pc,
+  // a warp per CTA: the rows' FP64 chains spread over all SMs' FP64 pipes
+  k_mprologue<MIXED><<<(unsigned)((B + 31) / 32), 32, 0, st>>>(m->d_ev, n_per, B, theta, m->pm, m->pf, m->pc,
                                                                    m->work);
   m->launches++;
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
@@ -396,8 +601,6 @@ static cudaError_t multi_run(Multi* m, const double* theta, int64_t n_per, doubl
   // the window's table rows, then (calibration) its calibration rows, staged in pairs
   const int64_t cal_smem = (int64_t)CHmax * rowmax;
   const size_t smem = (size_t)(cal_smem + (CAL ? (int64_t)(CHmax + 1) * calmax : 0)) * sizeof(Elem);
-  if ((e = raise_smem_limit((const void*)k_mwindow<NDET, MIXED, CAL>, m->ctxs[0]->device, smem)) != cudaSuccess)
-    return e;
   MultiArgs a;
   a.ev = m->d_ev;
   a.E = m->E;
@@ -412,10 +615,27 @@ static cudaError_t multi_run(Multi* m, const double* theta, int64_t n_per, doubl
   a.stride = m->D;
   a.cal_par = m->n_dim;
   a.cal_smem = (int)cal_smem;
-  k_mwindow<NDET, MIXED, CAL><<<m->num_sms * 2, 256, smem, st>>>(a);
+  bool rows = false;
+  if constexpr (MIXED) {
+    // the mixed bin loop, where two CTAs' windows and anchor records fit an SM (else one's)
+    const size_t blocks = (size_t)((CHmax + kAnchor - 1) / kAnchor);
+    const size_t rsmem = sizeof(float) * (blocks * (block_floats(NDET) + kAnchorRowFloats) +
+                                          (CAL ? (size_t)((CHmax + 2) * calmax + 3) / 4 * 4 : 0) +
+                                          (size_t)kTaskRows * blocks * anchor_rec_floats(NDET));
+    rows = rsmem <= kRowsSmem;
+    if (rows) {
+      if ((e = raise_smem_limit((const void*)k_mrows<NDET, CAL>, m->ctxs[0]->device, rsmem)) != cudaSuccess) return e;
+      k_mrows<NDET, CAL><<<m->num_sms * 2, 256, rsmem, st>>>(a, CHmax, calmax);
+    }
+  }
+  if (!rows) {
+    if ((e = raise_smem_limit((const void*)k_mwindow<NDET, MIXED, CAL>, m->ctxs[0]->device, smem)) != cudaSuccess)
+      return e;
+    k_mwindow<NDET, MIXED, CAL><<<m->num_sms * 2, 256, smem, st>>>(a);
+  }
   m->launches++;
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  k_mfinalize<NDET, Elem, CAL><<<(unsigned)((B + 63) / 64), 64, 0, st>>>(m->d_ev, n_per, B, m->pc,
+  k_mfinalize<NDET, Elem, CAL><<<(unsigned)((B + 7) / 8), 256, 0, st>>>(m->d_ev, n_per, B, m->pc,
                                                                            (const Elem*)m->partials, lnl);
   m->launches++;
   return cudaGetLastError();
