@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(128) k_mprologue(const EvDesc* __restrict__ ev
   if (ncut > 0) atomicMax(&work[ev[e].work_off], ncut);
 }
 
-// ---------------------------------------------------------------- persistent bin loop
+// ---------------------------------------------------------------- FP64 bin loop
 struct MultiArgs {
   const EvDesc* ev;
   int E;
@@ -129,10 +129,10 @@ struct MultiArgs {
   int cal_smem;         // element offset of the window's calibration rows in shared memory
 };
 
-template <int NDET, bool MIXED, bool CAL>
+template <int NDET, bool CAL>
 __global__ void __launch_bounds__(256, 2) k_mwindow(MultiArgs a) {
-  using Elem = typename std::conditional<MIXED, float, double>::type;
-  using Node = typename std::conditional<MIXED, float4, CalNodeD>::type;
+  using Elem = double;
+  using Node = CalNodeD;
   constexpr int S = CAL ? 3 : 2;  // sums per detector in a partial
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t bar;
@@ -198,14 +198,10 @@ __global__ void __launch_bounds__(256, 2) k_mwindow(MultiArgs a) {
 #pragma unroll
       for (int q = 0; q < NDET; ++q) U[q] = V[q] = X[q] = (Elem)0;
       if constexpr (CAL) {
-        cal_nodes_fill<NDET, MIXED>(a.theta + p * a.stride + a.cal_par, d.nn, d.calQ, lane, nodes);
+        cal_nodes_fill<NDET, false>(a.theta + p * a.stride + a.cal_par, d.nn, d.calQ, lane, nodes);
         __syncwarp();
       }
-      if constexpr (MIXED) {
-        anchored_sums_cal<NDET, CAL>(sm, d.row_elems, d.anchor + (int64_t)(j0 / kAnchor) * kAnchorRowFloats, d.df,
-                                     reinterpret_cast<const PropMixed*>(a.prop) + p, j0, jend, lane, U, V,
-                                     sm + a.cal_smem, d.cal_row, reinterpret_cast<const float4*>(nodes), X, nullptr);
-      } else {
+      {
         const PropF64* P = reinterpret_cast<const PropF64*>(a.prop) + p;
         double c[kNBasis], tau[NDET];
 #pragma unroll
@@ -263,8 +259,8 @@ __global__ void __launch_bounds__(256, 2) k_mwindow(MultiArgs a) {
 // -> 430 us (cold, serialised; issue active 66 %, short-scoreboard the top stall:
 // the hardware sine and cosine and the shared-memory reads), the call 631-730 ->
 // 356-395 us with the finalisation below and a warp per CTA in the prologue.
-constexpr int kTaskRows = 64;
-constexpr size_t kRowsSmem = 200 * 1024;  // its dynamic shared memory at most (227 KB less the statics)
+template <int NDET>
+constexpr int kTaskRows = NDET < 4 ? 64 : 32;  // (so that every accepted window fits shared memory)
 constexpr int kMaxPrefix = 1024;  // events whose prefix sums fit shared memory
 
 // What fused_row_sums needs of an event.
@@ -283,8 +279,8 @@ __global__ void __launch_bounds__(256, 2) k_mrows(MultiArgs a, int CHmax, int ca
   __shared__ __align__(8) uint64_t bar;
   __shared__ int s_pre[kMaxPrefix + 1];  // (event, window) pairs before event e
   __shared__ int s_task, s_next, s_fail;
-  __shared__ PropMixed s_pm[kTaskRows];
-  __shared__ int s_cut[kTaskRows];
+  __shared__ PropMixed s_pm[kTaskRows<NDET>];
+  __shared__ int s_cut[kTaskRows<NDET>];
   __shared__ __align__(16) float4 s_nodes[CAL ? 8 * NDET * kMaxCalNodes : 1];
   const int blocks = CHmax / kAnchor + (CHmax % kAnchor != 0);
   float* tab = reinterpret_cast<float*>(smem_raw);
@@ -323,7 +319,7 @@ __global__ void __launch_bounds__(256, 2) k_mrows(MultiArgs a, int CHmax, int ca
     s_task = atomicAdd(a.task_counter, 1);
   }
   __syncthreads();
-  const int parts = (int)((a.n_per + kTaskRows - 1) / kTaskRows);
+  const int parts = (int)((a.n_per + kTaskRows<NDET> - 1) / kTaskRows<NDET>);
   uint32_t parity = 0;
   while (true) {
     const int task = s_task;
@@ -372,8 +368,8 @@ __global__ void __launch_bounds__(256, 2) k_mrows(MultiArgs a, int CHmax, int ca
       if constexpr (CAL) bulk_g2s(cal, reinterpret_cast<const float*>(d.cal) + (int64_t)j0 * d.cal_row, cbytes, &bar);
       s_next = 0;
     }
-    const int64_t r0 = (int64_t)part * kTaskRows, p0 = (int64_t)e * a.n_per + r0;
-    const int n = a.n_per - r0 < kTaskRows ? (int)(a.n_per - r0) : kTaskRows;
+    const int64_t r0 = (int64_t)part * kTaskRows<NDET>, p0 = (int64_t)e * a.n_per + r0;
+    const int n = a.n_per - r0 < kTaskRows<NDET> ? (int)(a.n_per - r0) : kTaskRows<NDET>;
     for (int i = t; i < n * (int)(sizeof(PropMixed) / 16); i += 256)
       reinterpret_cast<float4*>(s_pm)[i] = reinterpret_cast<const float4*>(reinterpret_cast<const PropMixed*>(a.prop) + p0)[i];
     for (int i = t; i < n; i += 256) s_cut[i] = a.pc[p0 + i].ncut;
@@ -598,9 +594,6 @@ static cudaError_t multi_run(Multi* m, const double* theta, int64_t n_per, doubl
     rowmax = d.row_elems > rowmax ? d.row_elems : rowmax;
     calmax = d.cal_row > calmax ? d.cal_row : calmax;
   }
-  // the window's table rows, then (calibration) its calibration rows, staged in pairs
-  const int64_t cal_smem = (int64_t)CHmax * rowmax;
-  const size_t smem = (size_t)(cal_smem + (CAL ? (int64_t)(CHmax + 1) * calmax : 0)) * sizeof(Elem);
   MultiArgs a;
   a.ev = m->d_ev;
   a.E = m->E;
@@ -614,24 +607,19 @@ static cudaError_t multi_run(Multi* m, const double* theta, int64_t n_per, doubl
   a.theta = theta;
   a.stride = m->D;
   a.cal_par = m->n_dim;
-  a.cal_smem = (int)cal_smem;
-  bool rows = false;
   if constexpr (MIXED) {
-    // the mixed bin loop, where two CTAs' windows and anchor records fit an SM (else one's)
     const size_t blocks = (size_t)((CHmax + kAnchor - 1) / kAnchor);
-    const size_t rsmem = sizeof(float) * (blocks * (block_floats(NDET) + kAnchorRowFloats) +
-                                          (CAL ? (size_t)((CHmax + 2) * calmax + 3) / 4 * 4 : 0) +
-                                          (size_t)kTaskRows * blocks * anchor_rec_floats(NDET));
-    rows = rsmem <= kRowsSmem;
-    if (rows) {
-      if ((e = raise_smem_limit((const void*)k_mrows<NDET, CAL>, m->ctxs[0]->device, rsmem)) != cudaSuccess) return e;
-      k_mrows<NDET, CAL><<<m->num_sms * 2, 256, rsmem, st>>>(a, CHmax, calmax);
-    }
-  }
-  if (!rows) {
-    if ((e = raise_smem_limit((const void*)k_mwindow<NDET, MIXED, CAL>, m->ctxs[0]->device, smem)) != cudaSuccess)
-      return e;
-    k_mwindow<NDET, MIXED, CAL><<<m->num_sms * 2, 256, smem, st>>>(a);
+    const size_t smem = sizeof(float) * (blocks * (block_floats(NDET) + kAnchorRowFloats) +
+                                         (CAL ? (size_t)((CHmax + 2) * calmax + 3) / 4 * 4 : 0) +
+                                         (size_t)kTaskRows<NDET> * blocks * anchor_rec_floats(NDET));
+    if ((e = raise_smem_limit((const void*)k_mrows<NDET, CAL>, m->ctxs[0]->device, smem)) != cudaSuccess) return e;
+    k_mrows<NDET, CAL><<<m->num_sms * 2, 256, smem, st>>>(a, CHmax, calmax);
+  } else {
+    // the window's table rows, then (calibration) its calibration rows, staged in pairs
+    a.cal_smem = CHmax * rowmax;
+    const size_t smem = ((size_t)a.cal_smem + (CAL ? (size_t)(CHmax + 1) * calmax : 0)) * sizeof(double);
+    if ((e = raise_smem_limit((const void*)k_mwindow<NDET, CAL>, m->ctxs[0]->device, smem)) != cudaSuccess) return e;
+    k_mwindow<NDET, CAL><<<m->num_sms * 2, 256, smem, st>>>(a);
   }
   m->launches++;
   if ((e = cudaGetLastError()) != cudaSuccess) return e;

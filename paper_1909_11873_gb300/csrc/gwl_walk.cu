@@ -276,7 +276,7 @@ __global__ void __launch_bounds__(32 * (NW + kWalkHelpers), 1)
   __shared__ int s_n[kFusedRows], s_out[kFusedRows], s_start[kFusedRows], s_cout[2][kFusedRows];
   float* dyn = reinterpret_cast<float*>(smem_raw);
   const FusedLayout L = fused_layout(NDET, CAL ? a.cal_row : 0, a.CH, a.nwc, R);
-  const int D = pr.D, np = (D + 1) / 2, RD = R * D;
+  const int D = pr.D, RD = R * D;
   WalkGroup g;
   g.cu = reinterpret_cast<double*>(dyn + ((L.total + 1) & ~1));
   g.pu = g.cu + RD;
@@ -413,59 +413,130 @@ __device__ __forceinline__ double coord_jac(const PriorInfo& pr, int i, double t
   return sg * 2.5066282746310002 * exp(0.5 * z * z);
 }
 
-__global__ void k_gmc_init(PriorInfo pr, const double* __restrict__ live_u, const double* __restrict__ live_lnl,
-                           int64_t K, const WalkScalars* __restrict__ sc, const double* __restrict__ chol,
-                           uint64_t seed, int64_t n_chains, double* __restrict__ cu, double* __restrict__ cl,
-                           int32_t* __restrict__ cn, int32_t* __restrict__ cstart, double* __restrict__ vel) {
-  const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= n_chains) return;
-  const int D = pr.D;
-  const uint4 w = philox(make_uint4(0u, 0u, (uint32_t)b, (uint32_t)sc->counter), (uint32_t)seed,
-                         (uint32_t)(seed >> 32));
-  const int64_t idx = (int64_t)(((uint64_t)w.x * (uint64_t)(K - 1)) >> 32);
-  const int64_t st = idx < sc->worst ? idx : idx + 1;
-  for (int i = 0; i < D; ++i) cu[b * D + i] = live_u[st * D + i];
-  cl[b] = live_lnl[st];
-  cn[b] = 0;
-  if (cstart) cstart[b] = (int32_t)st;
-  double z[kMaxWalkDim];
-  walk_normals(seed, sc->counter, (uint32_t)b, 0x40000000u, D, z);
-  for (int i = 0; i < D; ++i) {
-    double dz = 0.0;
-    for (int k = 0; k <= i; ++k) dz += chol[i * D + k] * z[k];
-    vel[b * D + i] = sc->scale * dz;
+// A warp per chain, lanes over its coordinates, one warp per CTA so that the
+// chains' FP64 work spreads over all SMs.  Sums over coordinates that the
+// chain needs whole (g.Sigma g, v.g) are added in coordinate order on every lane.
+// (One thread per chain took 31 / 40 / 40 / 8 us for init, step, reflection and
+// move at 250 chains in 11-D: serial FP64 functions and triangular products on
+// two SMs.  Now @G1@.)
+struct GmcArgs {
+  const WalkScalars* sc;
+  const double* chol;
+  uint64_t seed;
+  int64_t n;
+  double *cu, *cl;   // chains: points, lnL
+  int32_t* cn;       // moves
+  double *vel, *vel2;
+  double *x1, *th1, *x2, *th2;
+  const double *l1, *g1, *l2;
+  int32_t* mode;
+};
+
+// Normals of a step word times the step matrix, times a factor: s_dz[i] = f (L z)_i (one warp).
+__device__ __forceinline__ void gmc_draw(const GmcArgs& a, uint32_t chain, uint32_t word, int D, double* s_z,
+                                         double* s_dz) {
+  const int lane = threadIdx.x & 31, np = (D + 1) / 2;
+  const uint32_t k0 = (uint32_t)a.seed, k1 = (uint32_t)(a.seed >> 32), counter = (uint32_t)a.sc->counter;
+  for (int k = lane; k < np; k += 32) {
+    const uint4 w = philox(make_uint4((uint32_t)(k >> 1), word, chain, counter), k0, k1);
+    const uint32_t w0 = (k & 1) ? w.z : w.x, w1 = (k & 1) ? w.w : w.y;
+    const double u1 = ((double)w0 + 1.0) * 0x1p-32;
+    const double u2 = (double)w1 * 0x1p-32;
+    const double r = sqrt(-2.0 * ::log(u1));
+    double sn, cs;
+    sincospi(2.0 * u2, &sn, &cs);
+    s_z[2 * k] = r * cs;
+    s_z[2 * k + 1] = r * sn;
   }
+  __syncwarp();
+  for (int i = lane; i < D; i += 32) {
+    double dz = 0.0;
+    for (int k = 0; k <= i; ++k) dz += a.chol[i * D + k] * s_z[k];
+    s_dz[i] = dz;
+  }
+  __syncwarp();
 }
 
-// From the second step on, the velocity is partly refreshed,
+__global__ void __launch_bounds__(32) k_gmc_init(PriorInfo pr, GmcArgs a, const double* __restrict__ live_u,
+                                                 const double* __restrict__ live_lnl, int64_t K,
+                                                 int32_t* __restrict__ cstart) {
+  __shared__ double s_z[kMaxWalkDim + 1], s_dz[kMaxWalkDim];
+  cudaTriggerProgrammaticLaunchCompletion();
+  cudaGridDependencySynchronize();
+  const int64_t b = blockIdx.x;
+  const int D = pr.D, lane = threadIdx.x;
+  const uint4 w = philox(make_uint4(0u, 0u, (uint32_t)b, (uint32_t)a.sc->counter), (uint32_t)a.seed,
+                         (uint32_t)(a.seed >> 32));
+  const int64_t idx = (int64_t)(((uint64_t)w.x * (uint64_t)(K - 1)) >> 32);
+  const int64_t st = idx < a.sc->worst ? idx : idx + 1;
+  for (int i = lane; i < D; i += 32) a.cu[b * D + i] = live_u[st * D + i];
+  if (lane == 0) {
+    a.cl[b] = live_lnl[st];
+    a.cn[b] = 0;
+    if (cstart) cstart[b] = (int32_t)st;
+  }
+  gmc_draw(a, (uint32_t)b, 0x40000000u, D, s_z, s_dz);
+  for (int i = lane; i < D; i += 32) a.vel[b * D + i] = a.sc->scale * s_dz[i];
+}
+
+// The end of a step: move to x2 with v' (mode 1, lnL(x2) >= L*), or stay and
+// reverse v (mode 1 below L*, mode 2).
+__device__ __forceinline__ void gmc_end(const GmcArgs& a, int64_t b, int D) {
+  const int lane = threadIdx.x & 31, mode = a.mode[b];
+  if (mode == 0) return;
+  if (mode == 1 && a.l2[b] >= a.sc->lstar) {
+    for (int i = lane; i < D; i += 32) {
+      a.cu[b * D + i] = a.x2[b * D + i];
+      a.vel[b * D + i] = a.vel2[b * D + i];
+    }
+    if (lane == 0) {
+      a.cl[b] = a.l2[b];
+      a.cn[b] += 1;
+    }
+  } else {
+    for (int i = lane; i < D; i += 32) a.vel[b * D + i] = -a.vel[b * D + i];
+  }
+}
+__global__ void __launch_bounds__(32) k_gmc_end(GmcArgs a, int D) {
+  cudaTriggerProgrammaticLaunchCompletion();
+  cudaGridDependencySynchronize();
+  gmc_end(a, blockIdx.x, D);
+}
+
+// The end of the step before (step > 1), then from the second step on the
+// velocity is partly refreshed,
 //   v <- rho v + sqrt(1 - rho^2) scale L z  (z: the normals of this step's word),
 // which keeps its distribution N(0, scale^2 L L^T); then x1 = u + v and
-// theta1 (NaN rows outside the cube).
-__global__ void k_gmc_step1(PriorInfo pr, const WalkScalars* __restrict__ sc, const double* __restrict__ chol,
-                            uint64_t seed, uint32_t step, double rho, int64_t n_chains,
-                            const double* __restrict__ cu, double* __restrict__ vel, double* __restrict__ x1,
-                            double* __restrict__ th1) {
-  const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= n_chains) return;
-  const int D = pr.D;
-  if (step > 1 && rho < 1.0) {
-    double z[kMaxWalkDim];
-    walk_normals(seed, sc->counter, (uint32_t)b, step, D, z);
-    const double a = sqrt(1.0 - rho * rho) * sc->scale;
-    for (int i = 0; i < D; ++i) {
-      double dz = 0.0;
-      for (int k = 0; k <= i; ++k) dz += chol[i * D + k] * z[k];
-      vel[b * D + i] = rho * vel[b * D + i] + a * dz;
-    }
+// theta1 (NaN rows outside the cube).  The normals, which depend on no other
+// kernel of the step, are formed before the wait for the likelihood.
+__global__ void __launch_bounds__(32) k_gmc_step1(PriorInfo pr, GmcArgs a, uint32_t step, double rho) {
+  __shared__ double s_z[kMaxWalkDim + 1], s_dz[kMaxWalkDim];
+  cudaTriggerProgrammaticLaunchCompletion();
+  const int64_t b = blockIdx.x;
+  const int D = pr.D, lane = threadIdx.x;
+  const bool fresh = step > 1 && rho < 1.0;
+  if (step == 1) cudaGridDependencySynchronize();
+  if (fresh) gmc_draw(a, (uint32_t)b, step, D, s_z, s_dz);
+  if (step > 1) {
+    cudaGridDependencySynchronize();
+    gmc_end(a, b, D);
   }
+  const double f = sqrt(1.0 - rho * rho) * a.sc->scale;
   bool inside = true;
-  for (int i = 0; i < D; ++i) {
-    double x = cu[b * D + i] + vel[b * D + i];
+  for (int i = lane; i < D; i += 32) {
+    const int64_t e = b * D + i;
+    double v = a.vel[e];
+    if (fresh) {
+      v = rho * v + f * s_dz[i];
+      a.vel[e] = v;
+    }
+    double x = a.cu[e] + v;
     if (coord_periodic(pr, i)) x -= floor(x);
     else if (x < 0.0 || x > 1.0) inside = false;
-    x1[b * D + i] = x;
+    a.x1[e] = x;
   }
-  for (int i = 0; i < D; ++i) th1[b * D + i] = inside ? coord_map(pr, i, x1[b * D + i]) : NAN;
+  inside = __all_sync(0xffffffffu, inside);
+  for (int i = lane; i < D; i += 32) a.th1[b * D + i] = inside ? coord_map(pr, i, a.x1[b * D + i]) : NAN;
 }
 
 // Accept x1, or reflect off the surface at x1 and set up the second trial.
@@ -478,81 +549,62 @@ __global__ void k_gmc_step1(PriorInfo pr, const WalkScalars* __restrict__ sc, co
 // so that it keeps the velocity distribution and undoes itself.  v' goes to
 // vel2 and theta2 = theta(x1 + v') is written for the chains that try x2.
 // mode: 0 moved to x1; 1 try x2; 2 stay and reverse v.
-__global__ void k_gmc_reflect(PriorInfo pr, const WalkScalars* __restrict__ sc, int64_t n_chains,
-                              const double* __restrict__ chol, const double* __restrict__ x1,
-                              const double* __restrict__ th1, const double* __restrict__ l1,
-                              const double* __restrict__ g1, double* __restrict__ cu, double* __restrict__ cl,
-                              int32_t* __restrict__ cn, const double* __restrict__ vel, double* __restrict__ vel2,
-                              double* __restrict__ x2, double* __restrict__ th2, int32_t* __restrict__ mode) {
-  const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= n_chains) return;
-  const int D = pr.D;
+__global__ void __launch_bounds__(32) k_gmc_reflect(PriorInfo pr, GmcArgs a) {
+  __shared__ double s_g[kMaxWalkDim], s_m[kMaxWalkDim];
+  cudaTriggerProgrammaticLaunchCompletion();
+  cudaGridDependencySynchronize();
+  const int64_t b = blockIdx.x, o = b * pr.D;
+  const int D = pr.D, lane = threadIdx.x;
   bool inside = true;
-  for (int i = 0; i < D; ++i) inside = inside && !isnan(th1[b * D + i]);
-  for (int i = 0; i < D; ++i) th2[b * D + i] = NAN;
-  if (inside && l1[b] >= sc->lstar) {  // move
-    for (int i = 0; i < D; ++i) cu[b * D + i] = x1[b * D + i];
-    cl[b] = l1[b];
-    cn[b] += 1;
-    mode[b] = 0;
+  for (int i = lane; i < D; i += 32) inside = inside && !isnan(a.th1[o + i]);
+  inside = __all_sync(0xffffffffu, inside);
+  for (int i = lane; i < D; i += 32) a.th2[o + i] = NAN;
+  if (inside && a.l1[b] >= a.sc->lstar) {  // move
+    for (int i = lane; i < D; i += 32) a.cu[o + i] = a.x1[o + i];
+    if (lane == 0) {
+      a.cl[b] = a.l1[b];
+      a.cn[b] += 1;
+      a.mode[b] = 0;
+    }
     return;
   }
-  double g[kMaxWalkDim], m[kMaxWalkDim];
-  for (int i = 0; i < D; ++i) {
-    const double x = x1[b * D + i];
-    g[i] = inside ? g1[b * D + i] * coord_jac(pr, i, th1[b * D + i])
-                  : (coord_periodic(pr, i) ? 0.0 : (x > 1.0 ? 1.0 : (x < 0.0 ? -1.0 : 0.0)));
+  for (int i = lane; i < D; i += 32) {
+    const double x = a.x1[o + i];
+    s_g[i] = inside ? a.g1[o + i] * coord_jac(pr, i, a.th1[o + i])
+                    : (coord_periodic(pr, i) ? 0.0 : (x > 1.0 ? 1.0 : (x < 0.0 ? -1.0 : 0.0)));
   }
-  double gsg = 0.0, vg = 0.0;
-  for (int k = 0; k < D; ++k) {  // m = L^T g
+  __syncwarp();
+  for (int k = lane; k < D; k += 32) {  // m = L^T g
     double t = 0.0;
-    for (int i = k; i < D; ++i) t += chol[i * D + k] * g[i];
-    m[k] = t;
-    gsg += t * t;
-    vg += vel[b * D + k] * g[k];
+    for (int i = k; i < D; ++i) t += a.chol[i * D + k] * s_g[i];
+    s_m[k] = t;
+  }
+  __syncwarp();
+  double gsg = 0.0, vg = 0.0;
+  for (int k = 0; k < D; ++k) {
+    gsg += s_m[k] * s_m[k];
+    vg += a.vel[o + k] * s_g[k];
   }
   if (!(gsg > 0.0) || !isfinite(gsg) || !isfinite(vg)) {
-    mode[b] = 2;
+    if (lane == 0) a.mode[b] = 2;
     return;
   }
   const double f = 2.0 * vg / gsg;
   bool in2 = true;
-  for (int i = 0; i < D; ++i) {
+  for (int i = lane; i < D; i += 32) {
     double sgi = 0.0;  // (Sigma g)_i = (L m)_i
-    for (int k = 0; k <= i; ++k) sgi += chol[i * D + k] * m[k];
-    const double v2 = vel[b * D + i] - f * sgi;
-    double x = x1[b * D + i] + v2;
+    for (int k = 0; k <= i; ++k) sgi += a.chol[i * D + k] * s_m[k];
+    const double v2 = a.vel[o + i] - f * sgi;
+    double x = a.x1[o + i] + v2;
     if (coord_periodic(pr, i)) x -= floor(x);
     else if (x < 0.0 || x > 1.0) in2 = false;
-    x2[b * D + i] = x;
-    vel2[b * D + i] = v2;
+    a.x2[o + i] = x;
+    a.vel2[o + i] = v2;
   }
-  if (!in2) {
-    mode[b] = 2;
-    return;
-  }
-  for (int i = 0; i < D; ++i) th2[b * D + i] = coord_map(pr, i, x2[b * D + i]);
-  mode[b] = 1;
-}
-
-// Move to x2 with v' (mode 1, lnL(x2) >= L*), or stay and reverse v (mode 1
-// below L*, mode 2).
-__global__ void k_gmc_step2(int D, const WalkScalars* __restrict__ sc, int64_t n_chains, const double* __restrict__ x2,
-                            const double* __restrict__ l2, const int32_t* __restrict__ mode,
-                            const double* __restrict__ vel2, double* __restrict__ cu, double* __restrict__ cl,
-                            int32_t* __restrict__ cn, double* __restrict__ vel) {
-  const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= n_chains || mode[b] == 0) return;
-  if (mode[b] == 1 && l2[b] >= sc->lstar) {
-    for (int i = 0; i < D; ++i) {
-      cu[b * D + i] = x2[b * D + i];
-      vel[b * D + i] = vel2[b * D + i];
-    }
-    cl[b] = l2[b];
-    cn[b] += 1;
-  } else {
-    for (int i = 0; i < D; ++i) vel[b * D + i] = -vel[b * D + i];
-  }
+  in2 = __all_sync(0xffffffffu, in2);
+  if (in2)
+    for (int i = lane; i < D; i += 32) a.th2[o + i] = coord_map(pr, i, a.x2[o + i]);
+  if (lane == 0) a.mode[b] = in2 ? 1 : 2;
 }
 
 // ---------------------------------------------------------------- nested-sampling state kernels
@@ -1139,38 +1191,49 @@ static cudaError_t launch_gmc(gwl_ctx* c, const double* live_u, const double* li
                               double* out_u, double* out_lnl, int32_t* out_nacc, int32_t* out_start, double* pu,
                               double* pth, double* plnl, cudaStream_t st) {
   const int D = (int)theta_stride(c);
-  const unsigned nb = (unsigned)((n_chains + 127) / 128);
   const PriorInfo pr = prior_info(c);
   // scratch after the random-walk proposal buffers: velocity, reflected velocity, x2, theta2, gradient,
   // l2, mode
-  double* vel = c->d_gmc;
-  double* vel2 = vel + n_chains * D;
-  double* x2 = vel2 + n_chains * D;
-  double* th2 = x2 + n_chains * D;
-  double* g1 = th2 + n_chains * D;
+  GmcArgs a;
+  a.sc = sc;
+  a.chol = chol;
+  a.seed = seed;
+  a.n = n_chains;
+  a.cu = out_u;
+  a.cl = out_lnl;
+  a.cn = out_nacc;
+  a.vel = c->d_gmc;
+  a.vel2 = a.vel + n_chains * D;
+  a.x1 = pu;
+  a.th1 = pth;
+  a.x2 = a.vel2 + n_chains * D;
+  a.th2 = a.x2 + n_chains * D;
+  double* g1 = a.th2 + n_chains * D;
   double* l2 = g1 + n_chains * D;
-  int32_t* mode = reinterpret_cast<int32_t*>(l2 + n_chains);
+  a.l1 = plnl;
+  a.g1 = g1;
+  a.l2 = l2;
+  a.mode = reinterpret_cast<int32_t*>(l2 + n_chains);
+  const dim3 grid((unsigned)n_chains), block(32);
+  cudaError_t e;
   {
     ProfScope ps(c, GWL_KERNEL_WALK, st);
-    k_gmc_init<<<nb, 128, 0, st>>>(pr, live_u, live_lnl, K, sc, chol, seed, n_chains, out_u, out_lnl, out_nacc,
-                                   out_start, vel);
+    e = launch_pdl(k_gmc_init, grid, block, 0, st, pr, a, live_u, live_lnl, K, out_start);
     c->launches++;
   }
-  cudaError_t e = cudaGetLastError();
   for (int s = 1; s <= walk_len && e == cudaSuccess; ++s) {
-    k_gmc_step1<<<nb, 128, 0, st>>>(pr, sc, chol, seed, (uint32_t)s, c->gmc_persistence, n_chains, out_u, vel, pu,
-                                    pth);
+    e = launch_pdl(k_gmc_step1, grid, block, 0, st, pr, a, (uint32_t)s, c->gmc_persistence);
     c->launches++;
-    if ((e = cudaGetLastError()) != cudaSuccess) break;
+    if (e != cudaSuccess) break;
     if ((e = launch_grad(c, pth, n_chains, plnl, g1, st)) != cudaSuccess) break;
-    k_gmc_reflect<<<nb, 128, 0, st>>>(pr, sc, n_chains, chol, pu, pth, plnl, g1, out_u, out_lnl, out_nacc, vel,
-                                      vel2, x2, th2, mode);
+    e = launch_pdl(k_gmc_reflect, grid, block, 0, st, pr, a);
     c->launches++;
-    if ((e = cudaGetLastError()) != cudaSuccess) break;
-    if ((e = launch_loglike(c, th2, n_chains, l2, st)) != cudaSuccess) break;
-    k_gmc_step2<<<nb, 128, 0, st>>>(D, sc, n_chains, x2, l2, mode, vel2, out_u, out_lnl, out_nacc, vel);
+    if (e != cudaSuccess) break;
+    e = launch_loglike(c, a.th2, n_chains, l2, st);
+  }
+  if (e == cudaSuccess && walk_len > 0) {  // the last step's end
+    e = launch_pdl(k_gmc_end, grid, block, 0, st, a, D);
     c->launches++;
-    e = cudaGetLastError();
   }
   return e;
 }
