@@ -109,6 +109,13 @@ int ensure_bytes(gwl_ctx* c, void** p, int64_t* cap, int64_t need) {
   return GWL_OK;
 }
 
+// The gradient's counters (new ones are not clear).
+int ensure_gwork(gwl_ctx* c) {
+  const int64_t need = gwl::grad_work_ints(c) * (int64_t)sizeof(int);
+  if (need > c->gwork_cap) c->gwork_clean = 0;
+  return ensure_bytes(c, (void**)&c->d_gwork, &c->gwork_cap, need);
+}
+
 int ensure_io(gwl_ctx* c, int64_t n) {
   if (n <= c->io_cap) return GWL_OK;
   dev_free(c, c->d_io, c->io_cap);
@@ -423,6 +430,7 @@ int gwl_grad(gwl_ctx* c, const double* theta_dev, int64_t B, double* lnl_dev, do
   if ((rc = ensure_scratch(c, B))) return rc;
   if ((rc = ensure_bytes(c, &c->d_pgrad, &c->pgrad_cap, gwl::prop_grad_bytes(c) * B))) return rc;
   if ((rc = ensure_bytes(c, &c->d_gpartials, &c->gpartials_cap, gwl::grad_partials_bytes(c, B)))) return rc;
+  if ((rc = ensure_gwork(c))) return rc;
   cudaStream_t st = (cudaStream_t)stream;
   c->last_stream = st;
   cudaError_t e = gwl::launch_grad(c, theta_dev, B, lnl_dev, grad_dev, st);
@@ -464,6 +472,7 @@ int ns_replace(gwl_ctx* c, const double* live_u, const double* live_lnl, int64_t
       return rc;
     if ((rc = ensure_bytes(c, &c->d_pgrad, &c->pgrad_cap, gwl::prop_grad_bytes(c) * n_chains))) return rc;
     if ((rc = ensure_bytes(c, &c->d_gpartials, &c->gpartials_cap, gwl::grad_partials_bytes(c, n_chains)))) return rc;
+    if ((rc = ensure_gwork(c))) return rc;
   }
   double* pu = c->d_walk;
   double* pth = pu + n_chains * D;
@@ -512,6 +521,7 @@ int ns_run_resumable(gwl_ctx* c, int64_t K, int64_t n_chains, int walk_len, uint
       return rc;
     if ((rc = ensure_bytes(c, &c->d_pgrad, &c->pgrad_cap, gwl::prop_grad_bytes(c) * nb))) return rc;
     if ((rc = ensure_bytes(c, &c->d_gpartials, &c->gpartials_cap, gwl::grad_partials_bytes(c, nb)))) return rc;
+    if ((rc = ensure_gwork(c))) return rc;
   }
   cudaStream_t st = (cudaStream_t)stream;
   c->last_stream = st;
@@ -900,6 +910,7 @@ void gwl_destroy(gwl_ctx* c) {
   dev_free(c, c->d_status, 4);
   dev_free(c, c->d_ffc, 1);
   if (c->d_pgrad) cudaFree(c->d_pgrad);
+  if (c->d_gwork) cudaFree(c->d_gwork);
   if (c->d_walk) cudaFree(c->d_walk);
   if (c->d_gmc) cudaFree(c->d_gmc);
   if (c->d_wscal) cudaFree(c->d_wscal);

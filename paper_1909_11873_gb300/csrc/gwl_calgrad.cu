@@ -181,6 +181,10 @@ __global__ void __launch_bounds__(256, 1) k_cal_moments(CalGradArgs a) {
     fence_mbar_init();
   }
   __syncthreads();
+  // This grid may run beside the gradient's bin loop, whose CTAs let it launch
+  // once they have seen the prologue complete: it reads nothing of theirs.  It
+  // waits for them at its end, so that the combination, which waits for this
+  // grid, finds both done.
   const int maxn = *a.maxcut;
   int nw = (maxn + a.CH - 1) / a.CH;
   if (nw > a.nw_total) nw = a.nw_total;
@@ -369,6 +373,7 @@ __global__ void __launch_bounds__(256, 1) k_cal_moments(CalGradArgs a) {
     });
     n_w -= __ldcg(&a.hist[w]);
   }
+  cudaGridDependencySynchronize();
 }
 
 // ---------------------------------------------------------------- launch
@@ -392,8 +397,8 @@ int64_t calgrad_part_elems(const gwl_ctx* c, int64_t B) {
 }
 
 template <int NDET, bool MIXED>
-static cudaError_t run_cal_moments(gwl_ctx* c, int64_t B, int* ctr, const int* hist, void* cpart, double* grad,
-                                   const double* theta, cudaStream_t st) {
+static cudaError_t run_cal_moments(gwl_ctx* c, int64_t B, const int* maxcut, const int* hist, int* ctr, void* cpart,
+                                   double* grad, const double* theta, cudaStream_t st) {
   using Elem = typename std::conditional<MIXED, float, double>::type;
   using Node = typename std::conditional<MIXED, float4, CalNodeD>::type;
   int CH = c->grad_window;
@@ -411,7 +416,7 @@ static cudaError_t run_cal_moments(gwl_ctx* c, int64_t B, int* ctr, const int* h
   a.prop = MIXED ? (const void*)c->d_pm : (const void*)c->d_pf;
   a.ctr = ctr;
   a.hist = hist;
-  a.maxcut = c->d_work;
+  a.maxcut = maxcut;
   a.status = c->d_status;
   a.cal = MIXED ? (const void*)c->d_cal_f : (const void*)c->d_cal_d;
   a.cal_row = MIXED ? c->row_cal_f : c->row_cal_d;
@@ -435,23 +440,23 @@ static cudaError_t run_cal_moments(gwl_ctx* c, int64_t B, int* ctr, const int* h
   int grid = c->num_sms;
   if (want < grid) grid = (int)(want > 0 ? want : 1);
   ProfScope ps(c, GWL_KERNEL_CALGRAD, st);
-  k_cal_moments<NDET, MIXED><<<grid, 256, smem, st>>>(a);
+  e = launch_pdl(k_cal_moments<NDET, MIXED>, dim3(grid), dim3(256), smem, st, a);
   c->launches++;
-  return cudaGetLastError();
+  return e;
 }
 
-cudaError_t launch_cal_moments(gwl_ctx* c, int64_t B, int* ctr, const int* hist, void* cpart, double* grad,
-                               const double* theta, cudaStream_t st) {
+cudaError_t launch_cal_moments(gwl_ctx* c, int64_t B, const int* maxcut, const int* hist, int* ctr, void* cpart,
+                               double* grad, const double* theta, cudaStream_t st) {
   const bool mixed = c->opt.precision == GWL_MIXED;
   switch (c->n_det) {
-    case 1: return mixed ? run_cal_moments<1, true>(c, B, ctr, hist, cpart, grad, theta, st)
-                         : run_cal_moments<1, false>(c, B, ctr, hist, cpart, grad, theta, st);
-    case 2: return mixed ? run_cal_moments<2, true>(c, B, ctr, hist, cpart, grad, theta, st)
-                         : run_cal_moments<2, false>(c, B, ctr, hist, cpart, grad, theta, st);
-    case 3: return mixed ? run_cal_moments<3, true>(c, B, ctr, hist, cpart, grad, theta, st)
-                         : run_cal_moments<3, false>(c, B, ctr, hist, cpart, grad, theta, st);
-    default: return mixed ? run_cal_moments<4, true>(c, B, ctr, hist, cpart, grad, theta, st)
-                          : run_cal_moments<4, false>(c, B, ctr, hist, cpart, grad, theta, st);
+    case 1: return mixed ? run_cal_moments<1, true>(c, B, maxcut, hist, ctr, cpart, grad, theta, st)
+                         : run_cal_moments<1, false>(c, B, maxcut, hist, ctr, cpart, grad, theta, st);
+    case 2: return mixed ? run_cal_moments<2, true>(c, B, maxcut, hist, ctr, cpart, grad, theta, st)
+                         : run_cal_moments<2, false>(c, B, maxcut, hist, ctr, cpart, grad, theta, st);
+    case 3: return mixed ? run_cal_moments<3, true>(c, B, maxcut, hist, ctr, cpart, grad, theta, st)
+                         : run_cal_moments<3, false>(c, B, maxcut, hist, ctr, cpart, grad, theta, st);
+    default: return mixed ? run_cal_moments<4, true>(c, B, maxcut, hist, ctr, cpart, grad, theta, st)
+                          : run_cal_moments<4, false>(c, B, maxcut, hist, ctr, cpart, grad, theta, st);
   }
 }
 

@@ -642,6 +642,11 @@ __global__ void __launch_bounds__(256, 2) k_window_grad(GradArgs a) {
   bool w0_pending = true;
   uint32_t parity = 0;
   cudaGridDependencySynchronize();
+  // The calibration's moments, which follow, need the prologue alone: their CTAs
+  // may take this grid's places as its CTAs leave (2048 rows with the
+  // calibration model 73 -> 64.5 us a call, 250 rows 53.6 -> 37.6).  Without
+  // them nothing is let in early: the combination's waiting CTAs cost 0.5-2 us.
+  if constexpr (CAL) cudaTriggerProgrammaticLaunchCompletion();
   const int maxn = a.work[0];
   int nw = (maxn + a.CH - 1) / a.CH;
   if (nw > a.nw_total) nw = a.nw_total;
@@ -744,11 +749,14 @@ __global__ void k_finalize_grad(const PropCommon* __restrict__ pc,
                                 const PropGrad<typename std::conditional<MIXED, float, double>::type>* __restrict__ pg,
                                 const void* __restrict__ partials_v, const void* __restrict__ xpart_v,
                                 const void* __restrict__ cpart_v, int64_t B, int CH, int nw_total, int n_dim,
-                                int gstride, int nq, double* __restrict__ lnl, double* __restrict__ grad) {
+                                int gstride, int nq, double* __restrict__ lnl, double* __restrict__ grad,
+                                int* __restrict__ work, int nwork) {
   cudaGridDependencySynchronize();
   using G = typename std::conditional<MIXED, float, double>::type;
   // the directions of a proposal are adjacent threads, so their loads of its window sums coincide
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  // the bin loops are done: their counters are left cleared for the next call
+  for (int64_t k = t; k < nwork; k += (int64_t)gridDim.x * blockDim.x) work[k] = 0;
   const int64_t p = t / gstride;
   const int i = (int)(t % gstride);
   if (p >= B) return;
@@ -800,8 +808,8 @@ __global__ void k_finalize_grad(const PropCommon* __restrict__ pc,
 // Per-window sums of the bin loop, then (calibration model) the X_d
 // corrections and the calibration directions' per-window derivatives.
 int64_t calgrad_part_elems(const gwl_ctx* c, int64_t B);
-cudaError_t launch_cal_moments(gwl_ctx* c, int64_t B, int* ctr, const int* hist, void* cpart, double* grad,
-                               const double* theta, cudaStream_t st);
+cudaError_t launch_cal_moments(gwl_ctx* c, int64_t B, const int* maxcut, const int* hist, int* ctr, void* cpart,
+                               double* grad, const double* theta, cudaStream_t st);
 
 static int grad_window_of(const gwl_ctx* c) { return c->grad_window > c->M ? (int)c->M : c->grad_window; }
 static int64_t grad_sums_bytes(const gwl_ctx* c, int64_t B) {
@@ -823,9 +831,11 @@ int64_t grad_partials_bytes(const gwl_ctx* c, int64_t B) {
 int64_t prop_grad_bytes(const gwl_ctx* c) {
   return c->opt.precision == GWL_MIXED ? (int64_t)sizeof(PropGrad<float>) : (int64_t)sizeof(PropGrad<double>);
 }
-int64_t work_needed(const gwl_ctx* c, int64_t B);
-int* window_hist(const gwl_ctx* c);
-int* calgrad_counters(const gwl_ctx* c, int64_t B);
+// Counters of the gradient's bin loops (run_grad), in ints.
+int64_t grad_work_ints(const gwl_ctx* c) {
+  const int CH = grad_window_of(c);
+  return 1 + 3 * ((c->M + CH - 1) / CH);
+}
 
 // Directions per CTA of the role-form tangent prologue, and how many of its
 // CTAs an SM holds (from the kernel's registers and shared memory).
@@ -852,8 +862,21 @@ static cudaError_t run_grad(gwl_ctx* c, const double* theta, int64_t B, double* 
   using G = typename std::conditional<MIXED, float, double>::type;
   const int CH = grad_window_of(c);
   const int nw_total = (int)((c->M + CH - 1) / CH);
-  cudaError_t e = cudaMemsetAsync(c->d_work, 0, sizeof(int) * (size_t)work_needed(c, B), st);
-  if (e != cudaSuccess) return e;
+  // The counters (largest cut, window counters, histogram, the moments' window
+  // counters) are the gradient's own, and every call leaves them cleared (the
+  // combination kernel, after the bin loops): with a clearing launch before the
+  // prologue the call took 44.0 us against 40.6 at 4096 rows, 25.2 against 23.1
+  // at 250.  They are cleared here when they are
+  // new, after a change of the window count and after a call that failed.
+  const int nwork = 1 + 3 * nw_total;
+  int* work = c->d_gwork;
+  int* hist = work + 1 + nw_total;
+  cudaError_t e = cudaSuccess;
+  if (c->gwork_clean != nwork) {
+    e = cudaMemsetAsync(work, 0, sizeof(int) * (size_t)nwork, st);
+    if (e != cudaSuccess) return e;
+  }
+  c->gwork_clean = 0;
   {
     ProfScope ps(c, GWL_KERNEL_PROLOGUE, st);
     // the role form, three directions per CTA, while its CTAs fit one wave
@@ -865,16 +888,16 @@ static cudaError_t run_grad(gwl_ctx* c, const double* theta, int64_t B, double* 
     if (MIXED && role_ctas <= (int64_t)role_ctas_per_sm(c->device) * c->num_sms) {
       const dim3 grid((unsigned)((B + 31) / 32), (unsigned)((c->opt.n_dim + kRoleTangents - 1) / kRoleTangents));
       k_prologue_grad_roles<kRoleTangents><<<grid, 128, 0, st>>>(c->seg, theta, B, c->d_pm, c->d_pc,
-                                                                 reinterpret_cast<PropGrad<float>*>(c->d_pgrad),
-                                                                 c->d_work, window_hist(c), CH);
+                                                                 reinterpret_cast<PropGrad<float>*>(c->d_pgrad), work,
+                                                                 hist, CH);
     } else {
       constexpr int kTanGroup = tan_group<MIXED>();
       const int ngrp = (c->opt.n_dim + kTanGroup - 1) / kTanGroup;
       const int64_t nt = B * ngrp;
       k_prologue_grad<MIXED><<<(unsigned)((nt + 63) / 64), 64, 0, st>>>(c->seg, theta, B, ngrp, c->d_pm, c->d_pf,
-                                                                            c->d_pc,
-                                                                            reinterpret_cast<PropGrad<G>*>(c->d_pgrad),
-                                                                            c->d_work, window_hist(c), CH);
+                                                                        c->d_pc,
+                                                                        reinterpret_cast<PropGrad<G>*>(c->d_pgrad),
+                                                                        work, hist, CH);
     }
     c->launches++;
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
@@ -894,8 +917,8 @@ static cudaError_t run_grad(gwl_ctx* c, const double* theta, int64_t B, double* 
   a.pc = c->d_pc;
   a.prop = MIXED ? (const void*)c->d_pm : (const void*)c->d_pf;
   a.partials = c->d_gpartials;
-  a.work = c->d_work;
-  a.hist = window_hist(c);
+  a.work = work;
+  a.hist = hist;
   a.status = c->d_status;
   a.pg = c->d_pgrad;
   a.lnl = lnl;
@@ -929,7 +952,7 @@ static cudaError_t run_grad(gwl_ctx* c, const double* theta, int64_t B, double* 
     if (e != cudaSuccess) return e;
   }
   if (CAL) {
-    e = launch_cal_moments(c, B, calgrad_counters(c, B), window_hist(c), cpart, grad, theta, st);
+    e = launch_cal_moments(c, B, work, hist, hist + nw_total, cpart, grad, theta, st);
     if (e != cudaSuccess) return e;
   }
   {
@@ -938,9 +961,10 @@ static cudaError_t run_grad(gwl_ctx* c, const double* theta, int64_t B, double* 
     e = launch_pdl(k_finalize_grad<NDET, MIXED, CAL>, dim3((unsigned)((nt + 63) / 64)), dim3(64), 0, st,
                    (const PropCommon*)c->d_pc, (const PropGrad<G>*)c->d_pgrad, (const void*)c->d_gpartials,
                    (const void*)xpart, (const void*)cpart, B, CH, nw_total, c->opt.n_dim, a.gstride,
-                   2 * c->n_cal_nodes, lnl, grad);
+                   2 * c->n_cal_nodes, lnl, grad, work, nwork);
     c->launches++;
   }
+  if (e == cudaSuccess) c->gwork_clean = nwork;
   return e;
 }
 

@@ -893,11 +893,9 @@ static int64_t nw_max(const gwl_ctx* c) {
 // [0] largest cut, [1 + w] proposal (or item) counter of window w,
 // [1 + nw_max + w] histogram of last windows, [1 + 2 nw_max + p] windows (or
 // chunks) of proposal p summed, [1 + 2 nw_max + B + K] bucket counts of the
-// lane kernel (chunks of at least 32 bins), then the window counters of the
-// calibrated gradient's second bin loop.
+// lane kernel (chunks of at least 32 bins).  (A third block of nw_max ints is
+// unused; the size is part of what gwl_loglike_static accepts.)
 int64_t work_needed(const gwl_ctx* c, int64_t B) { return 1 + 3 * nw_max(c) + B + (c->M + 31) / 32; }
-int* window_hist(const gwl_ctx* c) { return c->d_work + 1 + nw_max(c); }
-int* calgrad_counters(const gwl_ctx* c, int64_t B) { return c->d_work + 1 + 2 * nw_max(c) + B + (c->M + 31) / 32; }
 
 template <int NDET, bool MIXED, bool CAL, bool F64PH = false>
 static cudaError_t run_window(gwl_ctx* c, const WinArgs& a, int grid, size_t smem, bool pdl, cudaStream_t st) {
