@@ -287,6 +287,8 @@ int gwl_create(const double* freqs, int64_t n_bins, const double* strain, const 
     if ((e = dev_alloc(c, &c->d_tab_delta, n_bins * c->row_delta)) != cudaSuccess) { rc = cuda_fail(e, "alloc"); break; }
     if ((e = dev_alloc(c, &c->d_tab_block, (n_bins + gwl::kAnchor - 1) / gwl::kAnchor * gwl::block_floats(n_det))) !=
         cudaSuccess) { rc = cuda_fail(e, "alloc"); break; }
+    if ((e = dev_alloc(c, &c->d_tab_low, (n_bins + gwl::kAnchor - 1) / gwl::kAnchor * gwl::kLowFloats)) !=
+        cudaSuccess) { rc = cuda_fail(e, "alloc"); break; }
     if ((e = dev_alloc(c, &c->d_anchor, (n_bins + gwl::kAnchor - 1) / gwl::kAnchor * gwl::kAnchorRowFloats)) !=
         cudaSuccess) { rc = cuda_fail(e, "alloc"); break; }
     if ((e = dev_alloc(c, &c->d_tab_f64, n_bins * c->row_doubles)) != cudaSuccess) { rc = cuda_fail(e, "alloc"); break; }
@@ -894,6 +896,7 @@ void gwl_destroy(gwl_ctx* c) {
   dev_free(c, c->d_tab_mixed, c->M * c->row_floats);
   dev_free(c, c->d_tab_delta, c->M * c->row_delta);
   dev_free(c, c->d_tab_block, (c->M + gwl::kAnchor - 1) / gwl::kAnchor * gwl::block_floats(c->n_det));
+  dev_free(c, c->d_tab_low, (c->M + gwl::kAnchor - 1) / gwl::kAnchor * gwl::kLowFloats);
   dev_free(c, c->d_anchor, (c->M + gwl::kAnchor - 1) / gwl::kAnchor * gwl::kAnchorRowFloats);
   dev_free(c, c->d_tab_f64, c->M * c->row_doubles);
   dev_free(c, c->d_cal_f, (c->M + 1) * c->row_cal_f);

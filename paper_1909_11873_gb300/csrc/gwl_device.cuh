@@ -57,9 +57,18 @@ constexpr int kAnchorRowFloats = 28;
 // of a delta row), so that a CTA's shared memory holds more windows.
 __host__ __device__ constexpr int block_units(int ndet) { return (kNBasis + 2 * ndet + 3) / 4; }
 __host__ __device__ constexpr int block_floats(int ndet) { return 4 * kAnchor * block_units(ndet); }
-// Index of float k of bin j in that table.
+// The low parts dB_lo of the float-float blocks, blocked in the same way in a
+// table of their own, which those blocks read in place: 16-byte loads of 32
+// neighbours, where the delta rows of 80-112 bytes took seven loads of 28 lines
+// each and set the time of batches of long segments.
+constexpr int kLowUnits = kNBasis / 4;
+constexpr int kLowFloats = 4 * kAnchor * kLowUnits;
+// Index of float k of bin j in the first table, and in the second.
 __host__ __device__ constexpr int64_t block_index(int64_t j, int k, int ndet) {
   return j / kAnchor * block_floats(ndet) + (k / 4) * 4 * kAnchor + (j % kAnchor) * 4 + k % 4;
+}
+__host__ __device__ constexpr int64_t low_index(int64_t j, int k) {
+  return j / kAnchor * kLowFloats + (k / 4) * 4 * kAnchor + (j % kAnchor) * 4 + k % 4;
 }
 
 // Calibration model (Section 2.2 of the paper): per detector, amplitude and

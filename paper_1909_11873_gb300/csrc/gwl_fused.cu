@@ -130,9 +130,8 @@ FusedArgs fused_args(const gwl_ctx* c, int nwc) {
   FusedArgs a;
   a.seg = c->seg;
   a.tab = c->d_tab_block;
-  a.rows = c->d_tab_delta;
+  a.low = c->d_tab_low;
   a.anchor = c->d_anchor;
-  a.row_elems = c->row_delta;
   a.CH = lnl_window(c);
   a.nwc = nwc;
   a.df = (float)c->df;

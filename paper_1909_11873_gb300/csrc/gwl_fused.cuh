@@ -57,8 +57,7 @@ __host__ __device__ inline FusedLayout fused_layout(int ndet, int cal_row, int C
 struct FusedArgs {
   SegInfo seg;
   const float* tab;     // blocked table (FP32-delta bins)
-  const float* rows;    // delta rows, read in place by the blocks with float-float deltas
-  int row_elems;        // floats per delta row
+  const float* low;     // blocked low parts, read in place by the blocks with float-float deltas
   const float* anchor;  // anchor rows
   int CH;               // bins per window (a multiple of 32)
   int nwc;              // windows staged together
@@ -364,53 +363,62 @@ __device__ __forceinline__ float warp_fold(const float (&v)[N], int lane) {
   return t[0];
 }
 
-// FP32 sums of one row over bins [jl, jl + n) of the staged windows (jl a
-// multiple of 32, in bins from the first staged one; j0 that one's index in
-// the segment): the blocks in order, lanes over a block's bins, as
-// anchored_sums_cal.  cal: the staged windows' calibration rows.  A: the
-// segment's delta rows (rows, row_elems), df, cal_row and ffc.
-template <int NDET, bool CAL, class A>
-__device__ __forceinline__ void fused_row_sums(const A& a, const float* __restrict__ dyn, const float* __restrict__ cal,
-                                               const PropMixed& P, const float* __restrict__ rec, int j0, int jl, int n,
-                                               int lane, const float4* __restrict__ nodes, float (&U)[NDET],
-                                               float (&V)[NDET], float (&X)[NDET]) {
-  constexpr int RX = 4 * ((kNBasis + 2 * NDET + 3) / 4);
-  constexpr int RXF = 4 * ((2 * kNBasis + 2 * NDET + 3) / 4);
-  constexpr int AR = anchor_rec_floats(NDET);
+// The part of a row's coefficients that its bins use, and its running sums.
+template <int NDET>
+struct RowState {
   float ch[kNBasis], dtl[NDET];
+  float U[NDET], V[NDET], X[NDET];
+  __device__ __forceinline__ void start(const PropMixed& P, float df, int lane) {
 #pragma unroll
-  for (int q = 0; q < kNBasis / 4; ++q)
-    *reinterpret_cast<float4*>(&ch[4 * q]) = reinterpret_cast<const float4*>(P.ch)[q];
-  const float lane_df = (float)lane * a.df;
+    for (int q = 0; q < kNBasis / 4; ++q)
+      *reinterpret_cast<float4*>(&ch[4 * q]) = reinterpret_cast<const float4*>(P.ch)[q];
+    const float lane_df = (float)lane * df;
 #pragma unroll
-  for (int d = 0; d < NDET; ++d) {
-    dtl[d] = __fmul_rn(P.th[d], lane_df);
-    U[d] = V[d] = X[d] = 0.0f;
+    for (int d = 0; d < NDET; ++d) {
+      dtl[d] = __fmul_rn(P.th[d], lane_df);
+      U[d] = V[d] = X[d] = 0.0f;
+    }
   }
-  auto record = [&](int b, float (&ad)[NDET]) {
+  // The lane's anchor terms of the block with anchor record rec; whether the block takes the FP32 delta.
+  __device__ __forceinline__ bool record(const float* __restrict__ rec, float (&ad)[NDET]) const {
+    constexpr int AR = anchor_rec_floats(NDET);
     float r[AR];
     if constexpr (AR == 2) {
-      *reinterpret_cast<float2*>(r) = *reinterpret_cast<const float2*>(rec + AR * b);
+      *reinterpret_cast<float2*>(r) = *reinterpret_cast<const float2*>(rec);
     } else {
 #pragma unroll
       for (int q = 0; q < AR / 4; ++q)
-        *reinterpret_cast<float4*>(&r[4 * q]) = *reinterpret_cast<const float4*>(rec + AR * b + 4 * q);
+        *reinterpret_cast<float4*>(&r[4 * q]) = *reinterpret_cast<const float4*>(rec + 4 * q);
     }
 #pragma unroll
     for (int d = 0; d < NDET; ++d) ad[d] = __fadd_rn(r[d], dtl[d]);
     return r[NDET] != 0.0f;
-  };
+  }
+};
+
+// FP32 sums of one row over blocks [b, bend) of its bins [jl, jl + n) of the
+// staged windows (jl a multiple of 32, in bins from the first staged one; j0
+// that one's index in the segment): the blocks in order, lanes over a block's
+// bins, as anchored_sums_cal.  cal: the staged windows' calibration rows.  A:
+// the segment's low parts (low), df, cal_row and ffc.
+template <int NDET, bool CAL, class A>
+__device__ __forceinline__ void fused_row_blocks(const A& a, const float* __restrict__ dyn, const float* __restrict__ cal,
+                                                 const PropMixed& P, RowState<NDET>& R, const float* __restrict__ rec,
+                                                 int j0, int jl, int n, int b, int bend, int lane,
+                                                 const float4* __restrict__ nodes) {
+  constexpr int RX = 4 * ((kNBasis + 2 * NDET + 3) / 4);
+  constexpr int LO = kNBasis + 2 * NDET, RXF = 4 * ((LO + kNBasis + 3) / 4);
+  constexpr int AR = anchor_rec_floats(NDET);
   constexpr int BF = block_floats(NDET);
-  const float* row = dyn + jl / kAnchor * BF + 4 * lane;
-  const float* crow = CAL ? cal + (jl + lane) * a.cal_row : nullptr;
+  const float* row = dyn + (jl / kAnchor + b) * BF + 4 * lane;
+  const float* crow = CAL ? cal + (jl + b * kAnchor + lane) * a.cal_row : nullptr;
   const int cstep = CAL ? kAnchor * a.cal_row : 0;
   CalBin<NDET, float> cb0, cb1;
-  const int nblk = (n + kAnchor - 1) / kAnchor;
-  for (int b = 0; b < nblk;) {
+  while (b < bend) {
     float ad0[NDET], ad1[NDET];
-    const bool f0 = record(b, ad0);
-    bool pair = f0 && (b + 2) * kAnchor <= n;
-    if (pair) pair = record(b + 1, ad1);
+    const bool f0 = R.record(rec + AR * b, ad0);
+    bool pair = f0 && b + 2 <= bend && (b + 2) * kAnchor <= n;
+    if (pair) pair = R.record(rec + AR * (b + 1), ad1);
     if (pair) {
       // two complete blocks with FP32 deltas, in straight-line code so that their chains interleave
       float v0[RX], v1[RX];
@@ -423,8 +431,8 @@ __device__ __forceinline__ void fused_row_sums(const A& a, const float* __restri
         cal_eval<NDET>(crow, nodes, cb0);
         cal_eval<NDET>(crow + cstep, nodes, cb1);
       }
-      bin_anchor<NDET, CAL>(v0, ch, ad0, U, V, cb0, X);
-      bin_anchor<NDET, CAL>(v1, ch, ad1, U, V, cb1, X);
+      bin_anchor<NDET, CAL>(v0, R.ch, ad0, R.U, R.V, cb0, R.X);
+      bin_anchor<NDET, CAL>(v1, R.ch, ad1, R.U, R.V, cb1, R.X);
       b += 2;
       row += 2 * BF;
       if (CAL) crow += 2 * cstep;
@@ -432,27 +440,105 @@ __device__ __forceinline__ void fused_row_sums(const A& a, const float* __restri
     }
     if (b * kAnchor + lane < n) {  // lanes past the cut sit out
       if constexpr (CAL) cal_eval<NDET>(crow, nodes, cb0);
-      if (f0) {
-        float v[RX];
+      float v[RX];
 #pragma unroll
-        for (int k = 0; k < RX / 4; ++k)
-          *reinterpret_cast<float4*>(&v[4 * k]) = reinterpret_cast<const float4*>(row)[kAnchor * k];
-        bin_anchor<NDET, CAL>(v, ch, ad0, U, V, cb0, X);
+      for (int k = 0; k < RX / 4; ++k)
+        *reinterpret_cast<float4*>(&v[4 * k]) = reinterpret_cast<const float4*>(row)[kAnchor * k];
+      if (f0) {
+        bin_anchor<NDET, CAL>(v, R.ch, ad0, R.U, R.V, cb0, R.X);
       } else {
         if (a.ffc && lane == 0) atomicAdd(a.ffc, 1ull);
-        float v[RXF], cl[kNBasis];
+        float x[RXF], cl[kNBasis], lo[kNBasis];
 #pragma unroll
         for (int q = 0; q < kNBasis / 4; ++q)
           *reinterpret_cast<float4*>(&cl[4 * q]) = reinterpret_cast<const float4*>(P.cl)[q];
-        const float4* full = reinterpret_cast<const float4*>(a.rows + (int64_t)(j0 + jl + b * kAnchor + lane) * a.row_elems);
+        const float4* low = reinterpret_cast<const float4*>(a.low + (int64_t)((j0 + jl) / kAnchor + b) * kLowFloats) + lane;
 #pragma unroll
-        for (int k = 0; k < RXF / 4; ++k) *reinterpret_cast<float4*>(&v[4 * k]) = __ldg(full + k);
-        bin_anchor_exact<NDET, CAL>(v, ch, cl, ad0, U, V, cb0, X);
+        for (int k = 0; k < kLowUnits; ++k) *reinterpret_cast<float4*>(&lo[4 * k]) = __ldg(low + kAnchor * k);
+#pragma unroll
+        for (int k = 0; k < RXF; ++k) x[k] = k < LO ? v[k] : k < LO + kNBasis ? lo[k - LO] : 0.0f;
+        bin_anchor_exact<NDET, CAL>(x, R.ch, cl, ad0, R.U, R.V, cb0, R.X);
       }
     }
     b += 1;
     row += BF;
     if (CAL) crow += cstep;
+  }
+}
+
+// All blocks of a row's bins [jl, jl + n).
+template <int NDET, bool CAL, class A>
+__device__ __forceinline__ void fused_row_sums(const A& a, const float* __restrict__ dyn, const float* __restrict__ cal,
+                                               const PropMixed& P, const float* __restrict__ rec, int j0, int jl, int n,
+                                               int lane, const float4* __restrict__ nodes, RowState<NDET>& R) {
+  R.start(P, a.df, lane);
+  fused_row_blocks<NDET, CAL>(a, dyn, cal, P, R, rec, j0, jl, n, 0, (n + kAnchor - 1) / kAnchor, lane, nodes);
+}
+
+// The sums of NR rows over the first n[k] bins of a staged window by one warp,
+// without calibration: blocks that are complete and take the FP32 delta for
+// every row read the table once for all of them, the others row by row, so
+// that each row's blocks keep their order.  rec[k]: row k's anchor records.
+template <int NDET, int NR, class A>
+__device__ __forceinline__ void fused_shared_sums(const A& a, const float* __restrict__ dyn,
+                                                  const PropMixed* (&P)[NR], const float* (&rec)[NR], int j0, int (&n)[NR],
+                                                  int lane, RowState<NDET> (&R)[NR]) {
+  constexpr int RX = 4 * ((kNBasis + 2 * NDET + 3) / 4), AR = anchor_rec_floats(NDET), BF = block_floats(NDET);
+  int full = n[0] / kAnchor, end = 0;  // blocks complete in every row; blocks of the longest row
+#pragma unroll
+  for (int k = 0; k < NR; ++k) {
+    R[k].start(*P[k], a.df, lane);
+    full = n[k] / kAnchor < full ? n[k] / kAnchor : full;
+    const int e = (n[k] + kAnchor - 1) / kAnchor;
+    end = e > end ? e : end;
+  }
+  int b = 0;
+  while (b < end) {
+    const float* row = dyn + b * BF + 4 * lane;
+    for (; b < full; ++b, row += BF) {
+      float ad[NR][NDET];
+      bool fast = true;
+#pragma unroll
+      for (int k = 0; k < NR; ++k) fast &= R[k].record(rec[k] + AR * b, ad[k]);
+      if (!fast) break;
+      float v[RX];
+#pragma unroll
+      for (int k = 0; k < RX / 4; ++k)
+        *reinterpret_cast<float4*>(&v[4 * k]) = reinterpret_cast<const float4*>(row)[kAnchor * k];
+      CalBin<NDET, float> none;
+#pragma unroll
+      for (int k = 0; k < NR; ++k) bin_anchor<NDET, false>(v, R[k].ch, ad[k], R[k].U, R[k].V, none, R[k].X);
+    }
+    int e = b;  // up to the next block that all rows share, or to the end
+    for (; e < full; ++e) {
+      bool fast = true;
+#pragma unroll
+      for (int k = 0; k < NR; ++k) fast &= rec[k][AR * e + NDET] != 0.0f;
+      if (fast) break;
+    }
+    if (e >= full) e = end;
+    if (b == e) break;
+#pragma unroll 1
+    for (int k = 0; k < NR; ++k) {  // row 0, then the rows move up: one copy of the code
+      const int ek = (n[0] + kAnchor - 1) / kAnchor;
+      fused_row_blocks<NDET, false>(a, dyn, nullptr, *P[0], R[0], rec[0], j0, 0, n[0], b, e < ek ? e : ek, lane, nullptr);
+      const PropMixed* p0 = P[0];
+      const float* rec0 = rec[0];
+      const int n0 = n[0];
+      const RowState<NDET> R0 = R[0];
+#pragma unroll
+      for (int q = 0; q + 1 < NR; ++q) {
+        P[q] = P[q + 1];
+        rec[q] = rec[q + 1];
+        n[q] = n[q + 1];
+        R[q] = R[q + 1];
+      }
+      P[NR - 1] = p0;
+      rec[NR - 1] = rec0;
+      n[NR - 1] = n0;
+      R[NR - 1] = R0;
+    }
+    b = e;
   }
 }
 
@@ -520,14 +606,15 @@ __device__ __forceinline__ bool fused_bins(const FusedArgs& a, const FusedLayout
       if (n > a.CH) n = a.CH;
       float4* nodes = sm.nodes + (CAL ? warp * NDET * kMaxCalNodes : 0);
       if constexpr (CAL) cal_nodes_fill<NDET, true>(crow(r), a.nn, a.calQ, lane, nodes);
-      float U[NDET], V[NDET], X[NDET], v[NS];
+      float v[NS];
+      RowState<NDET> rs;
       fused_row_sums<NDET, CAL>(a, dyn, dyn + L.cal, sm.pm[r], dyn + L.rec + (r * gblk + jl / kAnchor) * AR, j0, jl, n, lane,
-                                nodes, U, V, X);
+                                nodes, rs);
 #pragma unroll
       for (int d = 0; d < NDET; ++d) {
-        v[2 * d] = U[d];
-        v[2 * d + 1] = V[d];
-        if constexpr (CAL) v[2 * NDET + d] = X[d];
+        v[2 * d] = rs.U[d];
+        v[2 * d + 1] = rs.V[d];
+        if constexpr (CAL) v[2 * NDET + d] = rs.X[d];
       }
       const float s = warp_fold<NS>(v, lane);
       constexpr int W = FoldP<NS>::W;

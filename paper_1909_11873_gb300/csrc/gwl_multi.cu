@@ -27,7 +27,8 @@ struct EvDesc {
   SegInfo seg;
   const void* tab;     // delta table (mixed) or FP64 table of this event
   const float* anchor; // anchor rows (mixed)
-  const float* blk;    // blocked table (mixed)
+  const float* blk;    // blocked table and low parts (mixed)
+  const float* low;
   float df;
   int row_elems;
   int CH;              // window (bins)
@@ -252,21 +253,29 @@ __global__ void __launch_bounds__(256, 2) k_mwindow(MultiArgs a) {
 // proposals.  Tasks come from one counter through prefix sums over the events,
 // formed once per CTA.
 //
+// A warp takes kSharedRows proposals together (without calibration), in order of
+// their cuts, and reads a table block once for all of them: alone, every
+// proposal's 64 bytes per bin kept the shared-memory pipe busy 82 % of the time.
+//
 // Against whole (event, window) tasks with per-proposal claims, whose 500
 // proposals kept one CTA busy for 250 us (the last tasks ended alone), and the
 // bin loop's per-proposal work (a warp's anchor pass, 30-shuffle reductions):
 // 500 proposals of each of 12 events of 4 to 128 s, 3 detectors, the bin loop 718
-// -> 430 us (cold, serialised; issue active 66 %, short-scoreboard the top stall:
-// the hardware sine and cosine and the shared-memory reads), the call 631-730 ->
-// 356-395 us with the finalisation below and a warp per CTA in the prologue.
+// -> 430 us (cold, serialised), the call 631-730 -> 356-395 us with the
+// finalisation below and a warp per CTA in the prologue.  Of that, shared reads:
+// 12 x 500 rows of another draw 539 -> 492 us with two rows, 492 with three, 478
+// with four; 12 x 2000 rows 2005 -> 1744 us; 12 x 500 with two detectors 461 -> 392
+// us.  Now bound by the issue of the bins' instructions and the hardware sine and
+// cosine (57 % of its rate on 2048 rows of a 128 s event).  The float-float blocks'
+// low parts from a blocked table: 12 x 64 rows 147 -> 136 us.
 template <int NDET>
 constexpr int kTaskRows = NDET < 4 ? 64 : 32;  // (so that every accepted window fits shared memory)
+constexpr int kSharedRows = 4;    // rows a warp takes together (118 registers with three detectors)
 constexpr int kMaxPrefix = 1024;  // events whose prefix sums fit shared memory
 
 // What fused_row_sums needs of an event.
 struct RowTab {
-  const float* rows;
-  int row_elems;
+  const float* low;
   float df;
   int cal_row;
   unsigned long long* ffc;
@@ -275,12 +284,13 @@ struct RowTab {
 template <int NDET, bool CAL>
 __global__ void __launch_bounds__(256, 2) k_mrows(MultiArgs a, int CHmax, int calmax) {
   constexpr int S = CAL ? 3 : 2, NS = S * NDET, AR = anchor_rec_floats(NDET);
+  constexpr int NR = CAL ? 1 : kSharedRows;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t bar;
   __shared__ int s_pre[kMaxPrefix + 1];  // (event, window) pairs before event e
   __shared__ int s_task, s_next, s_fail;
   __shared__ PropMixed s_pm[kTaskRows<NDET>];
-  __shared__ int s_cut[kTaskRows<NDET>];
+  __shared__ int s_cut[kTaskRows<NDET>], s_order[kTaskRows<NDET>];
   __shared__ __align__(16) float4 s_nodes[CAL ? 8 * NDET * kMaxCalNodes : 1];
   const int blocks = CHmax / kAnchor + (CHmax % kAnchor != 0);
   float* tab = reinterpret_cast<float*>(smem_raw);
@@ -381,32 +391,66 @@ __global__ void __launch_bounds__(256, 2) k_mrows(MultiArgs a, int CHmax, int ca
       if (j0 + b * kAnchor < s_cut[r])
         anchor_record<NDET>(s_pm[r], anc + b * kAnchorRowFloats, rec + (r * blocks + b) * AR);
     }
+    if (t < n) {  // the rows by descending cut: those that share the table's reads end together
+      const int c = s_cut[t];
+      int rank = 0;
+      for (int r = 0; r < n; ++r) {
+        const int m = s_cut[r];
+        rank += m > c || (m == c && r < t) ? 1 : 0;
+      }
+      s_order[rank] = t;
+    }
     __syncthreads();
     if (s_fail) return;
     if (t == 0) s_task = atomicAdd(a.task_counter, 1);
-    const RowTab rt{reinterpret_cast<const float*>(d.tab), d.row_elems, d.df, d.cal_row, nullptr};
-    while (true) {
-      int r = 0;
-      if (lane == 0) r = atomicAdd(&s_next, 1);
-      r = __shfl_sync(0xffffffffu, r, 0);
-      if (r >= n) break;
-      int nr = s_cut[r] - j0;
-      if (nr <= 0) continue;
-      if (nr > nbins) nr = nbins;
-      float4* nodes = s_nodes + (CAL ? (t >> 5) * NDET * kMaxCalNodes : 0);
-      if constexpr (CAL) cal_nodes_fill<NDET, true>(a.theta + (p0 + r) * a.stride + a.cal_par, d.nn, d.calQ, lane, nodes);
-      float U[NDET], V[NDET], X[NDET], v[NS];
-      fused_row_sums<NDET, CAL>(rt, tab, cal, s_pm[r], rec + r * blocks * AR, j0, 0, nr, lane, nodes, U, V, X);
+    const RowTab rt{d.low, d.df, d.cal_row, nullptr};
+    float* sums = reinterpret_cast<float*>(a.partials) + d.part_off + (r0 * d.nw_total + w) * NS;
+    auto store = [&](const RowState<NDET>& R, int r) {
+      float v[NS];
 #pragma unroll
       for (int q = 0; q < NDET; ++q) {
-        v[S * q] = U[q];
-        v[S * q + 1] = V[q];
-        if constexpr (CAL) v[S * q + 2] = X[q];
+        v[S * q] = R.U[q];
+        v[S * q + 1] = R.V[q];
+        if constexpr (CAL) v[S * q + 2] = R.X[q];
       }
       const float s = warp_fold<NS>(v, lane);
       constexpr int W = FoldP<NS>::W;
-      if (lane % W == 0 && lane / W < NS)
-        reinterpret_cast<float*>(a.partials)[d.part_off + ((r0 + r) * d.nw_total + w) * NS + lane / W] = s;
+      if (lane % W == 0 && lane / W < NS) sums[(int64_t)r * d.nw_total * NS + lane / W] = s;
+    };
+    while (true) {
+      int i = 0;
+      if (lane == 0) i = atomicAdd(&s_next, NR);
+      i = __shfl_sync(0xffffffffu, i, 0);
+      if (i >= n) break;
+      if constexpr (CAL) {
+        const int r = s_order[i];
+        const int nr = s_cut[r] - j0 < nbins ? s_cut[r] - j0 : nbins;
+        if (nr <= 0) break;  // no longer row follows
+        float4* nodes = s_nodes + (t >> 5) * NDET * kMaxCalNodes;
+        cal_nodes_fill<NDET, true>(a.theta + (p0 + r) * a.stride + a.cal_par, d.nn, d.calQ, lane, nodes);
+        RowState<NDET> R;
+        fused_row_sums<NDET, CAL>(rt, tab, cal, s_pm[r], rec + r * blocks * AR, j0, 0, nr, lane, nodes, R);
+        store(R, r);
+      } else {
+        RowState<NDET> R[NR];
+        const PropMixed* P[NR];
+        const float* rc[NR];
+        int rows[NR], nr[NR];
+#pragma unroll
+        for (int k = 0; k < NR; ++k) {
+          const int r = s_order[i + k < n ? i + k : i];
+          const int left = s_cut[r] - j0;
+          rows[k] = r;
+          nr[k] = i + k >= n || left <= 0 ? 0 : left < nbins ? left : nbins;
+          P[k] = &s_pm[r];
+          rc[k] = rec + r * blocks * AR;
+        }
+        if (nr[0] == 0) break;
+        fused_shared_sums<NDET, NR>(rt, tab, P, rc, j0, nr, lane, R);
+#pragma unroll
+        for (int k = 0; k < NR; ++k)
+          if (nr[k] > 0) store(R[k], rows[k]);
+      }
     }
     __syncthreads();  // all warps are done with this task's rows
   }
@@ -539,6 +583,7 @@ cudaError_t multi_prepare(Multi* m, int64_t n_per) {
     d.tab = mixed ? (const void*)c->d_tab_delta : (const void*)c->d_tab_f64;
     d.anchor = c->d_anchor;
     d.blk = c->d_tab_block;
+    d.low = c->d_tab_low;
     d.df = (float)c->df;
     d.row_elems = mixed ? c->row_delta : c->row_doubles;
     int CH = c->window;

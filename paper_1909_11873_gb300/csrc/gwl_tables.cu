@@ -32,7 +32,7 @@ __global__ void k_table_rows(const double* __restrict__ freqs, const double* __r
                              const double* __restrict__ psd, int64_t M, int n_det, double df, double t_ref,
                              float* __restrict__ tab_m, int row_f, double* __restrict__ tab_d, int row_d,
                              float* __restrict__ tab_x, int row_x, float* __restrict__ tab_b,
-                             float* __restrict__ anc, double* __restrict__ hterm) {
+                             float* __restrict__ tab_l, float* __restrict__ anc, double* __restrict__ hterm) {
   const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= M) return;
   const double f = freqs[j];
@@ -47,6 +47,7 @@ __global__ void k_table_rows(const double* __restrict__ freqs, const double* __r
   for (int m = 0; m < kNBasis; ++m) {
     split_f64(b[m] - ba[m], rx[m], rx[lo_off + m]);
     tab_b[block_index(j, m, n_det)] = rx[m];
+    tab_l[low_index(j, m)] = rx[lo_off + m];
   }
   for (int k = kNBasis; k < 4 * block_units(n_det); ++k) tab_b[block_index(j, k, n_det)] = 0.0f;  // G: k_scale_tables
   if (j == ja) {
@@ -213,7 +214,7 @@ cudaError_t launch_build_tables(gwl_ctx* c, const double* d_strain, const double
   if (e != cudaSuccess) return e;
   k_table_rows<<<(unsigned)nb, T, 0, st>>>(c->d_freqs, d_strain, d_psd, c->M, c->n_det, c->df, c->opt.t_ref,
                                             c->d_tab_mixed, c->row_floats, c->d_tab_f64, c->row_doubles,
-                                            c->d_tab_delta, c->row_delta, c->d_tab_block, c->d_anchor, c->d_H);
+                                            c->d_tab_delta, c->row_delta, c->d_tab_block, c->d_tab_low, c->d_anchor, c->d_H);
   c->launches++;
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
