@@ -418,7 +418,8 @@ __device__ __forceinline__ double coord_jac(const PriorInfo& pr, int i, double t
 // chain needs whole (g.Sigma g, v.g) are added in coordinate order on every lane.
 // (One thread per chain took 31 / 40 / 40 / 8 us for init, step, reflection and
 // move at 250 chains in 11-D: serial FP64 functions and triangular products on
-// two SMs.  Now @G1@.)
+// two SMs.  A warp per chain: 8.5, 13 with the step before's move, 14, and 5 us for
+// the last move; the walk of 10 steps 1279 -> 606 us, 568 with the maps below.)
 struct GmcArgs {
   const WalkScalars* sc;
   const double* chol;
@@ -431,6 +432,23 @@ struct GmcArgs {
   const double *l1, *g1, *l2;
   int32_t* mode;
 };
+
+// The step and the reflection have kGmcWarps warps per chain: the first does
+// what lanes can share, and the coordinate maps and their derivatives, FP64
+// functions of 2,000 cycles each, run on a warp per kind, so that they overlap
+// instead of following one another in one divergent warp: a step of 25 / 250 /
+// 1000 chains in 11-D 52.1 / 59.2 / 95.7 -> 49.2 / 56.6 / 72.4 us.
+constexpr int kGmcWarps = 4;
+// The warp that maps coordinate i.
+__device__ __forceinline__ int gmc_class(const PriorInfo& pr, int i) {
+  if (i >= pr.n_src) return 0;
+  switch (pr.kind[i]) {
+    case GWL_PRIOR_VOLUME: return 1;
+    case GWL_PRIOR_SINE: return 2;
+    case GWL_PRIOR_COSINE: return 3;
+    default: return 0;
+  }
+}
 
 // Normals of a step word times the step matrix, times a factor: s_dz[i] = f (L z)_i (one warp).
 __device__ __forceinline__ void gmc_draw(const GmcArgs& a, uint32_t chain, uint32_t word, int D, double* s_z,
@@ -509,34 +527,44 @@ __global__ void __launch_bounds__(32) k_gmc_end(GmcArgs a, int D) {
 // which keeps its distribution N(0, scale^2 L L^T); then x1 = u + v and
 // theta1 (NaN rows outside the cube).  The normals, which depend on no other
 // kernel of the step, are formed before the wait for the likelihood.
-__global__ void __launch_bounds__(32) k_gmc_step1(PriorInfo pr, GmcArgs a, uint32_t step, double rho) {
-  __shared__ double s_z[kMaxWalkDim + 1], s_dz[kMaxWalkDim];
+__global__ void __launch_bounds__(32 * kGmcWarps) k_gmc_step1(PriorInfo pr, GmcArgs a, uint32_t step, double rho) {
+  __shared__ double s_z[kMaxWalkDim + 1], s_dz[kMaxWalkDim], s_x[kMaxWalkDim];
+  __shared__ int s_in;
   cudaTriggerProgrammaticLaunchCompletion();
   const int64_t b = blockIdx.x;
-  const int D = pr.D, lane = threadIdx.x;
+  const int D = pr.D, lane = threadIdx.x & 31;
   const bool fresh = step > 1 && rho < 1.0;
-  if (step == 1) cudaGridDependencySynchronize();
-  if (fresh) gmc_draw(a, (uint32_t)b, step, D, s_z, s_dz);
-  if (step > 1) {
-    cudaGridDependencySynchronize();
-    gmc_end(a, b, D);
-  }
-  const double f = sqrt(1.0 - rho * rho) * a.sc->scale;
-  bool inside = true;
-  for (int i = lane; i < D; i += 32) {
-    const int64_t e = b * D + i;
-    double v = a.vel[e];
-    if (fresh) {
-      v = rho * v + f * s_dz[i];
-      a.vel[e] = v;
+  if (threadIdx.x < 32) {
+    if (step == 1) cudaGridDependencySynchronize();
+    if (fresh) gmc_draw(a, (uint32_t)b, step, D, s_z, s_dz);
+    if (step > 1) {
+      cudaGridDependencySynchronize();
+      gmc_end(a, b, D);
     }
-    double x = a.cu[e] + v;
-    if (coord_periodic(pr, i)) x -= floor(x);
-    else if (x < 0.0 || x > 1.0) inside = false;
-    a.x1[e] = x;
+    const double f = sqrt(1.0 - rho * rho) * a.sc->scale;
+    bool inside = true;
+    for (int i = lane; i < D; i += 32) {
+      const int64_t e = b * D + i;
+      double v = a.vel[e];
+      if (fresh) {
+        v = rho * v + f * s_dz[i];
+        a.vel[e] = v;
+      }
+      double x = a.cu[e] + v;
+      if (coord_periodic(pr, i)) x -= floor(x);
+      else if (x < 0.0 || x > 1.0) inside = false;
+      a.x1[e] = x;
+      s_x[i] = x;
+    }
+    inside = __all_sync(0xffffffffu, inside);
+    if (lane == 0) s_in = inside;
+  } else {
+    cudaGridDependencySynchronize();  // (theta1 may still be read by the kernels before)
   }
-  inside = __all_sync(0xffffffffu, inside);
-  for (int i = lane; i < D; i += 32) a.th1[b * D + i] = inside ? coord_map(pr, i, a.x1[b * D + i]) : NAN;
+  __syncthreads();
+  const bool inside = s_in;
+  for (int i = lane; i < D; i += 32)
+    if (gmc_class(pr, i) == (int)threadIdx.x >> 5) a.th1[b * D + i] = inside ? coord_map(pr, i, s_x[i]) : NAN;
 }
 
 // Accept x1, or reflect off the surface at x1 and set up the second trial.
@@ -549,62 +577,74 @@ __global__ void __launch_bounds__(32) k_gmc_step1(PriorInfo pr, GmcArgs a, uint3
 // so that it keeps the velocity distribution and undoes itself.  v' goes to
 // vel2 and theta2 = theta(x1 + v') is written for the chains that try x2.
 // mode: 0 moved to x1; 1 try x2; 2 stay and reverse v.
-__global__ void __launch_bounds__(32) k_gmc_reflect(PriorInfo pr, GmcArgs a) {
-  __shared__ double s_g[kMaxWalkDim], s_m[kMaxWalkDim];
+__global__ void __launch_bounds__(32 * kGmcWarps) k_gmc_reflect(PriorInfo pr, GmcArgs a) {
+  __shared__ double s_g[kMaxWalkDim], s_m[kMaxWalkDim], s_x[kMaxWalkDim];
+  __shared__ int s_in2;
   cudaTriggerProgrammaticLaunchCompletion();
   cudaGridDependencySynchronize();
   const int64_t b = blockIdx.x, o = b * pr.D;
-  const int D = pr.D, lane = threadIdx.x;
+  const int D = pr.D, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   bool inside = true;
   for (int i = lane; i < D; i += 32) inside = inside && !isnan(a.th1[o + i]);
   inside = __all_sync(0xffffffffu, inside);
-  for (int i = lane; i < D; i += 32) a.th2[o + i] = NAN;
-  if (inside && a.l1[b] >= a.sc->lstar) {  // move
-    for (int i = lane; i < D; i += 32) a.cu[o + i] = a.x1[o + i];
-    if (lane == 0) {
-      a.cl[b] = a.l1[b];
-      a.cn[b] += 1;
-      a.mode[b] = 0;
+  if (inside && a.l1[b] >= a.sc->lstar) {  // move (every warp of the CTA)
+    if (warp == 0) {
+      for (int i = lane; i < D; i += 32) {
+        a.cu[o + i] = a.x1[o + i];
+        a.th2[o + i] = NAN;
+      }
+      if (lane == 0) {
+        a.cl[b] = a.l1[b];
+        a.cn[b] += 1;
+        a.mode[b] = 0;
+      }
     }
     return;
   }
   for (int i = lane; i < D; i += 32) {
+    if (gmc_class(pr, i) != warp) continue;
     const double x = a.x1[o + i];
     s_g[i] = inside ? a.g1[o + i] * coord_jac(pr, i, a.th1[o + i])
                     : (coord_periodic(pr, i) ? 0.0 : (x > 1.0 ? 1.0 : (x < 0.0 ? -1.0 : 0.0)));
   }
-  __syncwarp();
-  for (int k = lane; k < D; k += 32) {  // m = L^T g
-    double t = 0.0;
-    for (int i = k; i < D; ++i) t += a.chol[i * D + k] * s_g[i];
-    s_m[k] = t;
+  __syncthreads();
+  if (warp == 0) {
+    for (int k = lane; k < D; k += 32) {  // m = L^T g
+      double t = 0.0;
+      for (int i = k; i < D; ++i) t += a.chol[i * D + k] * s_g[i];
+      s_m[k] = t;
+    }
+    __syncwarp();
+    double gsg = 0.0, vg = 0.0;
+    for (int k = 0; k < D; ++k) {
+      gsg += s_m[k] * s_m[k];
+      vg += a.vel[o + k] * s_g[k];
+    }
+    bool in2 = gsg > 0.0 && isfinite(gsg) && isfinite(vg);
+    if (in2) {
+      const double f = 2.0 * vg / gsg;
+      for (int i = lane; i < D; i += 32) {
+        double sgi = 0.0;  // (Sigma g)_i = (L m)_i
+        for (int k = 0; k <= i; ++k) sgi += a.chol[i * D + k] * s_m[k];
+        const double v2 = a.vel[o + i] - f * sgi;
+        double x = a.x1[o + i] + v2;
+        if (coord_periodic(pr, i)) x -= floor(x);
+        else if (x < 0.0 || x > 1.0) in2 = false;
+        a.x2[o + i] = x;
+        s_x[i] = x;
+        a.vel2[o + i] = v2;
+      }
+      in2 = __all_sync(0xffffffffu, in2);
+    }
+    if (lane == 0) {
+      s_in2 = in2;
+      a.mode[b] = in2 ? 1 : 2;
+    }
   }
-  __syncwarp();
-  double gsg = 0.0, vg = 0.0;
-  for (int k = 0; k < D; ++k) {
-    gsg += s_m[k] * s_m[k];
-    vg += a.vel[o + k] * s_g[k];
-  }
-  if (!(gsg > 0.0) || !isfinite(gsg) || !isfinite(vg)) {
-    if (lane == 0) a.mode[b] = 2;
-    return;
-  }
-  const double f = 2.0 * vg / gsg;
-  bool in2 = true;
-  for (int i = lane; i < D; i += 32) {
-    double sgi = 0.0;  // (Sigma g)_i = (L m)_i
-    for (int k = 0; k <= i; ++k) sgi += a.chol[i * D + k] * s_m[k];
-    const double v2 = a.vel[o + i] - f * sgi;
-    double x = a.x1[o + i] + v2;
-    if (coord_periodic(pr, i)) x -= floor(x);
-    else if (x < 0.0 || x > 1.0) in2 = false;
-    a.x2[o + i] = x;
-    a.vel2[o + i] = v2;
-  }
-  in2 = __all_sync(0xffffffffu, in2);
-  if (in2)
-    for (int i = lane; i < D; i += 32) a.th2[o + i] = coord_map(pr, i, a.x2[o + i]);
-  if (lane == 0) a.mode[b] = in2 ? 1 : 2;
+  __syncthreads();
+  const bool in2 = s_in2;
+  for (int i = lane; i < D; i += 32)
+    if (gmc_class(pr, i) == warp) a.th2[o + i] = in2 ? coord_map(pr, i, s_x[i]) : NAN;
 }
 
 // ---------------------------------------------------------------- nested-sampling state kernels
@@ -1222,11 +1262,11 @@ static cudaError_t launch_gmc(gwl_ctx* c, const double* live_u, const double* li
     c->launches++;
   }
   for (int s = 1; s <= walk_len && e == cudaSuccess; ++s) {
-    e = launch_pdl(k_gmc_step1, grid, block, 0, st, pr, a, (uint32_t)s, c->gmc_persistence);
+    e = launch_pdl(k_gmc_step1, grid, dim3(32 * kGmcWarps), 0, st, pr, a, (uint32_t)s, c->gmc_persistence);
     c->launches++;
     if (e != cudaSuccess) break;
     if ((e = launch_grad(c, pth, n_chains, plnl, g1, st)) != cudaSuccess) break;
-    e = launch_pdl(k_gmc_reflect, grid, block, 0, st, pr, a);
+    e = launch_pdl(k_gmc_reflect, grid, dim3(32 * kGmcWarps), 0, st, pr, a);
     c->launches++;
     if (e != cudaSuccess) break;
     e = launch_loglike(c, a.th2, n_chains, l2, st);
