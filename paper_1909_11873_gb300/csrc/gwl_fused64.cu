@@ -334,15 +334,16 @@ static size_t room64() {
 // CTAs each instead of 2 on every second SM).  A piece is a few blocks, so that a
 // row's sums end together on the warps: 32 bins up to 1.5 rows per SM, 64 up to
 // 3, 128 beyond (where the warp sums cost 4 % of a piece).  Segments of more than
-// kMaxBins64 bins take this form only with at least a row per warp: below that
-// their windows do better spread over the whole chip.
-// (16 s BNS, 2 detectors, 16385 bins, 250 rows: 741 us here against 628 there,
-// 1216 rows: 2640 against 2660.)
+// kMaxBins64 bins keep the separate kernels, whose (row, window) tasks spread over
+// the whole chip (us here against there: 16 s BNS, 2 detectors, 250 rows 741 / 628,
+// 1216 rows 2640 / 2660; 32 s BNS, 1300 rows 8556 / 8044; 128 s BNS, 1300 rows
+// 56314 / 51134, 2048 rows 82305 / 80386; 16 s BBH, 1 detector, 2000 rows 141 /
+// 185, or 147 after the autotuner).
 constexpr int64_t kMaxBins64 = 8192;
 
 bool fused64_used(const gwl_ctx* c, int64_t B) {
   if (c->opt.precision != GWL_FP64 || c->n_cal_nodes || B <= 0) return false;
-  return c->M <= kMaxBins64 || B >= 8 * (int64_t)c->num_sms;
+  return c->M <= kMaxBins64;
 }
 
 template <int NDET>
