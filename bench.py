@@ -16,7 +16,8 @@ by writing a 256 MB buffer between timed steps (the step inputs are < 1 MB).
 ``e2e`` is the same metric through gwl_loglike_host with page-locked host
 buffers, timed by the host clock around each call (the flush is issued and
 finished before the clock starts).  ``roofline`` refers to the dominant
-kernel (the windowed bin loop), timed by the library's CUDA events on the
+kernel (the one-kernel likelihood, or the windowed bin loop where the tuned
+shape takes the separate kernels), timed by the library's CUDA events on the
 launch stream, with every pipe's algorithmic work reported and the largest
 fraction taken as the bound.  ``cpu_baseline`` times the FP64 oracle on the
 host cores on a bounded sample and runs the oracle comparisons of the other
@@ -85,8 +86,8 @@ PIPES_CAL = {"fp32_flop": 56 + 75, "mufu": 6}
 FP32_LANES_PER_SM = 128
 MUFU_PER_SM_CLK = 16
 # The kernel sources whose change invalidates a stored DRAM-traffic capture.
-KERNEL_SOURCES = ("gwl_lnl.cu", "gwl_bins.cuh", "gwl_sched.cuh", "gwl_device.cuh", "gwl_ff.cuh", "gwl_internal.h")
-TRAFFIC_FILE = os.path.join(ROOT, "profiles", "traffic_k_window_mixed_c2.txt")
+KERNEL_SOURCES = ("gwl_fused.cu", "gwl_fused.cuh", "gwl_bins.cuh", "gwl_device.cuh", "gwl_ff.cuh", "gwl_internal.h")
+TRAFFIC_FILE = os.path.join(ROOT, "profiles", "traffic_k_fused_c2.txt")
 
 
 def parse():
@@ -637,7 +638,7 @@ def run_gwl(args):
         ms, launches = timed(ctx, args.steps, args.warmup, soak=args.soak_seconds, nvtx="timed_mixed")
     ctx.gwl_sync()
     clocks = clk.summary()
-    # the bin loop's own time (library CUDA events on the launch stream) over a separate pass
+    # the kernels' own times (library CUDA events on the launch stream) over a separate pass
     ctx.gwl_profile(True)
     for _ in range(args.steps):
         flush.fill_(1.0)
@@ -683,7 +684,9 @@ def run_gwl(args):
         "roofline": {"bound": "alu", "pipe": bound, "achieved": b.get("achieved_T"), "peak": b.get("peak_T"),
                      "unit": "Top/s" if bound == "mufu" else "TFLOP/s", "frac": b["frac"], "traffic": traffic,
                      "traffic_basis": traffic_basis,
-                     "kernel": "k_lanes<3>" if tuning.get("bin_kernel") == 3 else "k_window<3,mixed>", "kernel_ms": bins_ms,
+                     "kernel": ("k_lanes<3>" if tuning.get("bin_kernel") == 3 else
+                                "k_window<3,mixed>" if prof[gwl.KERNEL_PROLOGUE][1] else "k_fused<3>"),
+                     "kernel_ms": bins_ms,
                      "pairs_per_launch": int(pairs), "share_of_step": bins_ms / ms,
                      "pipes": r4({k: {"per": v.get("per_pair", v.get("per_eval_bytes")), "frac": v["frac"]}
                                   for k, v in pipes.items()}),

@@ -465,7 +465,8 @@ int gwl_test_ffdelta_blocks(gwl_ctx* ctx, int enable, int64_t* count);
  * (mixed) or FP64 summation order, within the parity tolerances. */
 typedef struct gwl_tuning {
   int window;        /* likelihood bin loop: bins per window; 0 keeps (set) */
-  int ctas_per_sm;   /* likelihood bin loop: grid = ctas_per_sm x SMs; 0 keeps */
+  int ctas_per_sm;   /* likelihood bin loop: grid = ctas_per_sm x SMs; 0 keeps (the one-kernel
+                        forms, which most calls take, choose their own grid) */
   int grad_window;   /* gradient bin loop: bins per window; 0 keeps */
   double ms_loglike; /* gwl_autotune output: best time of one gwl_loglike call
                         (ms) at the tuned batch; gwl_get_tuning: last tuned value or 0 */

@@ -492,17 +492,6 @@ __device__ __forceinline__ void anchored_sums_cal(const float* __restrict__ sm, 
   }
 }
 
-// The same without calibration.
-template <int NDET>
-__device__ __forceinline__ void anchored_sums(const float* __restrict__ sm, int row_elems,
-                                              const float* __restrict__ anc0, float df,
-                                              const PropMixed* __restrict__ P, int j0, int jend, int lane,
-                                              float (&U)[NDET], float (&V)[NDET],
-                                              unsigned long long* __restrict__ ffc = nullptr) {
-  float X[NDET];
-  anchored_sums_cal<NDET, false>(sm, row_elems, anc0, df, P, j0, jend, lane, U, V, nullptr, 0, nullptr, X, ffc);
-}
-
 template <int NDET>
 __device__ __forceinline__ void phase_f64(const double (&v)[RowD<NDET>::n], const double (&c)[kNBasis],
                                           const double (&tau)[NDET], double (&sn)[NDET], double (&cs)[NDET],

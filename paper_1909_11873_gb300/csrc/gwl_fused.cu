@@ -4,10 +4,10 @@
 // What bounds it: the dependent float-pair chains of the coefficients (latency,
 // about half of the kernel) and then the issue of the bin sums, of which the
 // hardware sine and cosine are the largest pipe.  Measured back to back on the
-// 8 s, 3-detector batch of 8192 rows (704-bin windows): 18.3-18.8 us a call
-// against 32.1-33.3 us with the clearing, prologue and bin-loop kernels; with
-// the calibration model, 4096 rows: 22.0 against 35.4 us; 4 s, 1 detector, 1000
-// rows: 12.3 against 24.7 us; one row: 8.5 against 18.8 us.
+// 8 s, 3-detector batch of 8192 rows (704-bin windows): 17.9 us a call against
+// 32.1-33.3 us with the clearing, prologue and bin-loop kernels; with the
+// calibration model, 4096 rows: 21.1 against 35.4 us; 4 s, 1 detector, 1000
+// rows: 11.7 against 24.7 us; one row: 8.6 against 18.8 us.
 #include "gwl_fused.cuh"
 
 namespace gwl {
@@ -93,15 +93,15 @@ constexpr size_t kSmemPerSm = 228 * 1024;  // 1 KB of it goes to each resident C
 // line is drawn by the number of windows (us per call, 640-bin windows, one
 // kernel against three):
 //   8 s BBH, 3 detectors (one window in use)   B = 1 / 250 / 1900 / 8192 / 20000:
-//     8.5 / 10.8 / 12.2 / 19.2 / 47.0 against 16.6 / 19.2 / 22.4 / 33.7 / 58.0
+//     8.6 / 10.5 / 12.2 / 19.8 / 49.0 against 16.6 / 19.2 / 22.4 / 33.7 / 58.0
 //   8 s, every row in all 13 windows           B = 1 / 250 / 1900 / 8192:
-//     17.6 / 23.3 / 60.6 / 190 against 26.6 / 39.4 / 97.5 / 291
+//     21.1 / 26.0 / 67.1 / 210 against 26.6 / 39.4 / 97.5 / 291
 //   16 s BNS, 2 detectors, 26 windows          B = 1 / 250 / 1900 / 8192:
-//     30.5 / 40.2 / 107 / 320 against 33.2 / 50.4 / 139 / 476
+//     34.1 / 43.8 / 118 / 348 against 33.2 / 50.4 / 139 / 476
 //   32 s BNS, 3 detectors, 51 windows          B = 1 / 64 / 250 / 1900:
-//     59.4 / 61.7 / 73.7 / 229 against 48.4 / 57.5 / 82.1 / 278
+//     59.4 / 61.7 / 73.7 / 250 against 48.4 / 57.5 / 82.1 / 278
 //   128 s BNS, 406 windows                     B = 64 / 1000 / 1900 / 4000:
-//     327 / 1014 / 1388 / 2479 against 248 / 895 / 1529 / 3109
+//     327 / 1014 / 1540 / 2721 against 248 / 895 / 1529 / 3109
 // so segments of up to 32 windows take it at any batch, longer ones where the
 // batch gives every warp of two CTAs per SM a row.
 bool fused_shape(const gwl_ctx* c, int64_t B, int* grid, int* rows, int* nwc) {

@@ -7,6 +7,12 @@
 // template, regrouped so that per bin and detector only the phase, one
 // sincos and four multiply-adds remain.
 //
+// Most calls take one kernel: gwl_fused.cu (mixed) or gwl_fused64.cu (FP64).
+// The kernels of this file serve the rest: segments of more than 32 windows in
+// small batches, windows too large for the one-kernel form, calibrated or long
+// FP64 segments, the FP64-phase arm, the lane layout's prologue, and the walk
+// steps of those.
+//
 // Work decomposition: a clearing kernel zeroes the work counters; a prologue
 // kernel turns each parameter row into its coefficients (four warps per 32
 // rows); the bins are cut into windows of W bins, and each CTA of the
