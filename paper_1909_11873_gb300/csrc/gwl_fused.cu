@@ -93,15 +93,15 @@ constexpr size_t kSmemPerSm = 228 * 1024;  // 1 KB of it goes to each resident C
 // line is drawn by the number of windows (us per call, 640-bin windows, one
 // kernel against three):
 //   8 s BBH, 3 detectors (one window in use)   B = 1 / 250 / 1900 / 8192 / 20000:
-//     8.6 / 10.5 / 12.2 / 19.8 / 49.0 against 16.6 / 19.2 / 22.4 / 33.7 / 58.0
+//     8.6 / 10.4 / 12.2 / 19.6 / 48.2 against 16.6 / 19.2 / 22.4 / 33.7 / 58.0
 //   8 s, every row in all 13 windows           B = 1 / 250 / 1900 / 8192:
-//     21.1 / 26.0 / 67.1 / 210 against 26.6 / 39.4 / 97.5 / 291
+//     21.1 / 26.0 / 65.2 / 203 against 26.6 / 39.4 / 97.5 / 291
 //   16 s BNS, 2 detectors, 26 windows          B = 1 / 250 / 1900 / 8192:
-//     34.1 / 43.8 / 118 / 348 against 33.2 / 50.4 / 139 / 476
+//     34.1 / 43.8 / 112 / 330 against 33.2 / 50.4 / 139 / 476
 //   32 s BNS, 3 detectors, 51 windows          B = 1 / 64 / 250 / 1900:
-//     59.4 / 61.7 / 73.7 / 250 against 48.4 / 57.5 / 82.1 / 278
+//     59.4 / 61.7 / 73.7 / 243 against 48.4 / 57.5 / 82.1 / 278
 //   128 s BNS, 406 windows                     B = 64 / 1000 / 1900 / 4000:
-//     327 / 1014 / 1540 / 2721 against 248 / 895 / 1529 / 3109
+//     327 / 1014 / 1492 / 2720 against 248 / 895 / 1529 / 3109
 // so segments of up to 32 windows take it at any batch, longer ones where the
 // batch gives every warp of two CTAs per SM a row.
 bool fused_shape(const gwl_ctx* c, int64_t B, int* grid, int* rows, int* nwc) {
