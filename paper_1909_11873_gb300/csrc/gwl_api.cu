@@ -109,13 +109,6 @@ int ensure_bytes(gwl_ctx* c, void** p, int64_t* cap, int64_t need) {
   return GWL_OK;
 }
 
-// The gradient's counters (new ones are not clear).
-int ensure_gwork(gwl_ctx* c) {
-  const int64_t need = gwl::grad_work_ints(c) * (int64_t)sizeof(int);
-  if (need > c->gwork_cap) c->gwork_clean = 0;
-  return ensure_bytes(c, (void**)&c->d_gwork, &c->gwork_cap, need);
-}
-
 int ensure_io(gwl_ctx* c, int64_t n) {
   if (n <= c->io_cap) return GWL_OK;
   dev_free(c, c->d_io, c->io_cap);
@@ -293,6 +286,7 @@ int gwl_create(const double* freqs, int64_t n_bins, const double* strain, const 
         cudaSuccess) { rc = cuda_fail(e, "alloc"); break; }
     if ((e = dev_alloc(c, &c->d_tab_f64, n_bins * c->row_doubles)) != cudaSuccess) { rc = cuda_fail(e, "alloc"); break; }
     if ((e = dev_alloc(c, &c->d_status, 4)) != cudaSuccess) { rc = cuda_fail(e, "alloc"); break; }
+    if ((e = dev_alloc(c, &c->d_gwork, gwl::grad_work_max(c))) != cudaSuccess) { rc = cuda_fail(e, "alloc"); break; }
     if ((e = cudaMalloc(&c->d_wscal, 64)) != cudaSuccess) { rc = cuda_fail(e, "alloc"); break; }
     if ((e = cudaMalloc(&d_strain, sizeof(double) * 2 * n_det * n_bins)) != cudaSuccess) { rc = cuda_fail(e, "alloc"); break; }
     if ((e = cudaMalloc(&d_psd, sizeof(double) * n_det * n_bins)) != cudaSuccess) { rc = cuda_fail(e, "alloc"); break; }
@@ -307,7 +301,8 @@ int gwl_create(const double* freqs, int64_t n_bins, const double* strain, const 
         (e = cudaMemcpy(c->d_geom, geom, sizeof(double) * 9 * n_det, cudaMemcpyHostToDevice)) != cudaSuccess ||
         (e = cudaMemcpy(d_strain, strain, sizeof(double) * 2 * n_det * n_bins, cudaMemcpyHostToDevice)) != cudaSuccess ||
         (e = cudaMemcpy(d_psd, psd, sizeof(double) * n_det * n_bins, cudaMemcpyHostToDevice)) != cudaSuccess ||
-        (e = cudaMemset(c->d_status, 0, 4 * sizeof(int))) != cudaSuccess) {
+        (e = cudaMemset(c->d_status, 0, 4 * sizeof(int))) != cudaSuccess ||
+        (e = cudaMemset(c->d_gwork, 0, sizeof(int) * gwl::grad_work_max(c))) != cudaSuccess) {
       rc = cuda_fail(e, "copy inputs");
       break;
     }
@@ -432,7 +427,6 @@ int gwl_grad(gwl_ctx* c, const double* theta_dev, int64_t B, double* lnl_dev, do
   if ((rc = ensure_scratch(c, B))) return rc;
   if ((rc = ensure_bytes(c, &c->d_pgrad, &c->pgrad_cap, gwl::prop_grad_bytes(c) * B))) return rc;
   if ((rc = ensure_bytes(c, &c->d_gpartials, &c->gpartials_cap, gwl::grad_partials_bytes(c, B)))) return rc;
-  if ((rc = ensure_gwork(c))) return rc;
   cudaStream_t st = (cudaStream_t)stream;
   c->last_stream = st;
   cudaError_t e = gwl::launch_grad(c, theta_dev, B, lnl_dev, grad_dev, st);
@@ -474,7 +468,6 @@ int ns_replace(gwl_ctx* c, const double* live_u, const double* live_lnl, int64_t
       return rc;
     if ((rc = ensure_bytes(c, &c->d_pgrad, &c->pgrad_cap, gwl::prop_grad_bytes(c) * n_chains))) return rc;
     if ((rc = ensure_bytes(c, &c->d_gpartials, &c->gpartials_cap, gwl::grad_partials_bytes(c, n_chains)))) return rc;
-    if ((rc = ensure_gwork(c))) return rc;
   }
   double* pu = c->d_walk;
   double* pth = pu + n_chains * D;
@@ -523,7 +516,6 @@ int ns_run_resumable(gwl_ctx* c, int64_t K, int64_t n_chains, int walk_len, uint
       return rc;
     if ((rc = ensure_bytes(c, &c->d_pgrad, &c->pgrad_cap, gwl::prop_grad_bytes(c) * nb))) return rc;
     if ((rc = ensure_bytes(c, &c->d_gpartials, &c->gpartials_cap, gwl::grad_partials_bytes(c, nb)))) return rc;
-    if ((rc = ensure_gwork(c))) return rc;
   }
   cudaStream_t st = (cudaStream_t)stream;
   c->last_stream = st;
@@ -713,6 +705,7 @@ int gwl_sync(gwl_ctx* c) {
   if (e != cudaSuccess) return cuda_fail(e, "gwl_sync status");
   if (st) {
     cudaMemset(c->d_status, 0, sizeof(int));
+    c->gwork_dirty = true;  // nothing is taken for granted after a kernel that left early
     if (st & gwl::kStatusTimeout) return fail(GWL_ERR_TIMEOUT, "a kernel's bounded wait ran out");
   }
   return GWL_OK;
@@ -911,9 +904,9 @@ void gwl_destroy(gwl_ctx* c) {
   dev_free(c, c->d_work, c->work_cap);
   dev_free(c, c->d_blist, c->blist_cap);
   dev_free(c, c->d_status, 4);
+  dev_free(c, c->d_gwork, gwl::grad_work_max(c));
   dev_free(c, c->d_ffc, 1);
   if (c->d_pgrad) cudaFree(c->d_pgrad);
-  if (c->d_gwork) cudaFree(c->d_gwork);
   if (c->d_walk) cudaFree(c->d_walk);
   if (c->d_gmc) cudaFree(c->d_gmc);
   if (c->d_wscal) cudaFree(c->d_wscal);

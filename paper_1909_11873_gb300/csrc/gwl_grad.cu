@@ -831,11 +831,8 @@ int64_t grad_partials_bytes(const gwl_ctx* c, int64_t B) {
 int64_t prop_grad_bytes(const gwl_ctx* c) {
   return c->opt.precision == GWL_MIXED ? (int64_t)sizeof(PropGrad<float>) : (int64_t)sizeof(PropGrad<double>);
 }
-// Counters of the gradient's bin loops (run_grad), in ints.
-int64_t grad_work_ints(const gwl_ctx* c) {
-  const int CH = grad_window_of(c);
-  return 1 + 3 * ((c->M + CH - 1) / CH);
-}
+// Counters of the gradient's bin loops (run_grad) with the smallest window, 32 bins, in ints.
+int64_t grad_work_max(const gwl_ctx* c) { return 1 + 3 * ((c->M + 31) / 32); }
 
 // Directions per CTA of the role-form tangent prologue, and how many of its
 // CTAs an SM holds (from the kernel's registers and shared memory).
@@ -863,20 +860,26 @@ static cudaError_t run_grad(gwl_ctx* c, const double* theta, int64_t B, double* 
   const int CH = grad_window_of(c);
   const int nw_total = (int)((c->M + CH - 1) / CH);
   // The counters (largest cut, window counters, histogram, the moments' window
-  // counters) are the gradient's own, and every call leaves them cleared (the
-  // combination kernel, after the bin loops): with a clearing launch before the
-  // prologue the call took 44.0 us against 40.6 at 4096 rows, 25.2 against 23.1
-  // at 250.  They are cleared here when they are
-  // new, after a change of the window count and after a call that failed.
+  // counters) are the gradient's own: all of the buffer is clear between calls.
+  // gwl_create clears it, for every window count, and every call clears what it
+  // has used (the combination kernel, after the bin loops): with a clearing
+  // launch before the prologue the call took 44.0 us against 40.6 at 4096 rows,
+  // 25.2 against 23.1 at 250.  After a call that failed half-way or a reported
+  // timeout it is cleared here; a clearing that is only recorded in a graph
+  // vouches for nothing until the graph runs, so it leaves the mark.
   const int nwork = 1 + 3 * nw_total;
   int* work = c->d_gwork;
   int* hist = work + 1 + nw_total;
   cudaError_t e = cudaSuccess;
-  if (c->gwork_clean != nwork) {
-    e = cudaMemsetAsync(work, 0, sizeof(int) * (size_t)nwork, st);
+  bool stays_dirty = false;
+  if (c->gwork_dirty) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if ((e = cudaStreamIsCapturing(st, &cap)) != cudaSuccess) return e;
+    stays_dirty = cap != cudaStreamCaptureStatusNone;
+    e = cudaMemsetAsync(work, 0, sizeof(int) * (size_t)grad_work_max(c), st);
     if (e != cudaSuccess) return e;
   }
-  c->gwork_clean = 0;
+  c->gwork_dirty = true;
   {
     ProfScope ps(c, GWL_KERNEL_PROLOGUE, st);
     // the role form, three directions per CTA, while its CTAs fit one wave
@@ -964,7 +967,7 @@ static cudaError_t run_grad(gwl_ctx* c, const double* theta, int64_t B, double* 
                    2 * c->n_cal_nodes, lnl, grad, work, nwork);
     c->launches++;
   }
-  if (e == cudaSuccess) c->gwork_clean = nwork;
+  if (e == cudaSuccess) c->gwork_dirty = stays_dirty;
   return e;
 }
 

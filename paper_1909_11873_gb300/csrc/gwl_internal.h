@@ -59,9 +59,8 @@ struct gwl_ctx {
   int64_t io_cap = 0;            // in doubles
   void* d_pgrad = nullptr;       // per-proposal tangents of the gradient prologue
   int64_t pgrad_cap = 0;         // in bytes
-  int* d_gwork = nullptr;        // counters of the gradient's bin loops
-  int64_t gwork_cap = 0;         // in bytes
-  int gwork_clean = 0;           // ints of them that the last call left cleared (0: unknown)
+  int* d_gwork = nullptr;        // [grad_work_max] counters of the gradient's bin loops, clear between calls
+  bool gwork_dirty = false;      // a call may have left some of them set
   void* d_gpartials = nullptr;   // per-window sums of the gradient bin loop
   int64_t gpartials_cap = 0;     // in bytes
   int* d_blist = nullptr;        // lane bin loop: bucket lists of proposals [chunks][B]
@@ -168,7 +167,7 @@ size_t calgrad_smem(const gwl_ctx* c, int CH);
 cudaError_t launch_grad(gwl_ctx* c, const double* theta, int64_t B, double* lnl, double* grad, cudaStream_t st);
 int64_t grad_partials_bytes(const gwl_ctx* c, int64_t B);
 int64_t prop_grad_bytes(const gwl_ctx* c);
-int64_t grad_work_ints(const gwl_ctx* c);
+int64_t grad_work_max(const gwl_ctx* c);
 
 // a7 / a9: random walks and nested sampling
 cudaError_t launch_walk(gwl_ctx* c, const double* live_u, const double* live_lnl, int64_t K, const void* scalars,
