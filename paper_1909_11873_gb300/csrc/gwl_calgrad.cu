@@ -204,7 +204,8 @@ __global__ void __launch_bounds__(256, 1) k_cal_moments(CalGradArgs a) {
       fence_proxy_async_smem();
       calgrad_stage<MIXED>(a, sm, j0, j1, &bar);
     }
-    if (!mbar_wait_bounded(&bar, parity, a.status)) return;
+    // a wait that ran out ends the whole CTA's work, by way of the wait at its end
+    if (__syncthreads_or(!mbar_wait_bounded(&bar, parity, a.status))) break;
     parity ^= 1u;
     const Elem* crows = sm + a.cal_smem;
     drain_window(ctr, a.B, 1, a.pc, j0, lane, [&](int64_t p, int ncut) {
