@@ -6,16 +6,18 @@
 // busy over the SMs.  In the separate kernels the bin loop's warps race for
 // rows: with about a thousand rows the SMs that pass the prologue's wait first
 // take 16 each and others none, and a row's windows follow one another.  Here
-// every SM gets the same number of rows, and a row is cut into pieces of 32 to
-// 128 bins that the warps of a CTA, or of a cluster of CTAs, share.  The arithmetic per row and bin is that
-// of prologue_rows and bin_f64; the FP64 sums are added in another order (piece
-// by piece, in bin order across pieces, the same on every call).
+// every SM gets the same number of rows, and a row is cut into pieces of 128
+// bins that the warps of a CTA, or of a cluster of CTAs, share.  The arithmetic per row and bin is that
+// of prologue_rows and bin_f64; the FP64 sums are added in another order: a
+// piece's four blocks of 32 bins lane by lane, a fixed fold of the lanes, then
+// the pieces in bin order.  However the work is split, that order stays, so a
+// row's lnL has the same bits in every batch.
 //
 // Measured back to back (us a call, 8 s BBH, 3 detectors, one kernel against
 // three, 384-bin windows), at 1 / 32 / 150 / 250 / 1021 / 2000 / 8192 rows:
-// 20.5 / 21.2 / 32.5 / 49.6 / 92.3 / 173 / 551 against 56.9 / 71.0 / 125 / 165 /
-// 173 / 205 / 609; rows over the whole band (8 s BNS), 1 / 64 / 250 / 1000:
-// 50.6 / 164 / 517 / 1662 against 81.5 / 206 / 511 / 1643.
+// 15.6 / 17.3 / 29.7 / 45.2 / 114.7 / 209.6 / 725 against 65.6 / 76.6 / 139 / 157
+// / 201 / 218 / 727; rows over the whole band (8 s BNS), 1 / 64 / 250 / 1000:
+// 45.1 / 145 / 510 / 1655 against 79.9 / 205 / 510 / 1638.
 #include <cmath>
 
 #include "gwl_bins.cuh"
@@ -23,14 +25,16 @@
 namespace gwl {
 
 constexpr int kRows64 = 32;  // rows per CTA at most (one per lane in the prologue)
+constexpr int kPiece = 128;  // bins per piece
 
 struct Fused64Args {
   SegInfo seg;
   const double* tab;  // FP64 rows
   int row_elems;      // doubles per row
-  int piece;          // bins per item (a multiple of 32)
   int np;             // pieces a CTA stages together
-  int C;              // CTAs per group of rows (a cluster)
+  int lc;             // log2 of C, the CTAs per group of rows (a cluster)
+  int keep;           // pieces whose sums a CTA holds (np, or all of its own where C > 1)
+  int team;           // warps that share an item: 1, 2 or 4
   int* status;
 };
 
@@ -46,6 +50,7 @@ struct Smem64 {
   PropF64 pf[kRows64];
   int ncut[kRows64], flag[kRows64];
   int next, maxcut, fail;
+  int item[4][2];
   alignas(8) uint64_t bar;
 };
 
@@ -144,16 +149,23 @@ __device__ __forceinline__ void coeffs64(const SegInfo& s, int R, Smem64<NDET>& 
   __syncthreads();
 }
 
-// warp_fold (gwl_fused.cuh) on doubles: value v's warp sum on lanes [4 v, 4 v + 4) (at most eight values).
+// warp_fold (gwl_fused.cuh) on doubles (at most eight values): value v's warp sum
+// on lanes [v W, v W + W), W = 32 / P, P the power of two at or above the count.
+template <int N>
+struct Fold64 {
+  static constexpr int P = N <= 2 ? 2 : N <= 4 ? 4 : 8;
+  static constexpr int W = 32 / P;
+};
 template <int N>
 __device__ __forceinline__ double warp_fold64(const double (&v)[N], int lane) {
   static_assert(N <= 8, "at most eight sums");
-  double t[8];
+  constexpr int P = Fold64<N>::P;
+  double t[P];
 #pragma unroll
-  for (int k = 0; k < 8; ++k) t[k] = k < N ? v[k] : 0.0;
+  for (int k = 0; k < P; ++k) t[k] = k < N ? v[k] : 0.0;
   int off = 16;
 #pragma unroll
-  for (int h = 4; h >= 1; h >>= 1, off >>= 1) {
+  for (int h = P / 2; h >= 1; h >>= 1, off >>= 1) {
     const bool up = (lane & off) != 0;
 #pragma unroll
     for (int k = 0; k < h; ++k) {
@@ -162,9 +174,20 @@ __device__ __forceinline__ double warp_fold64(const double (&v)[N], int lane) {
       t[k] = keep + __shfl_xor_sync(0xffffffffu, send, off);
     }
   }
-  t[0] += __shfl_xor_sync(0xffffffffu, t[0], 2);
-  t[0] += __shfl_xor_sync(0xffffffffu, t[0], 1);
+#pragma unroll
+  for (; off >= 1; off >>= 1) t[0] += __shfl_xor_sync(0xffffffffu, t[0], off);
   return t[0];
+}
+
+// The U and V of detector d with one bin's sine and cosine, as bin_f64 adds them.
+__device__ __forceinline__ void add_bin64(double gr, double gi, double sn, double cs, double& U, double& V) {
+  U = fma(gr, cs, fma(gi, sn, U));
+  V = fma(gi, cs, fma(-gr, sn, V));
+}
+
+// Barrier of team q, of n threads.
+__device__ __forceinline__ void team_sync(int q, int n) {
+  asm volatile("bar.sync %0, %1;" ::"r"(1 + q), "r"(n) : "memory");
 }
 
 // A double in the shared memory of the cluster's CTA `rank`, at this CTA's address p.
@@ -179,9 +202,27 @@ __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.aligned;\n barrier.cluster.wait.aligned;" ::: "memory");
 }
 
+// K_d and the <h|h> term of detector d, one row per lane (one warp).
+template <int NDET>
+__device__ __forceinline__ void amplitudes64(const SegInfo& s, Smem64<NDET>& sm, int d, int lane) {
+  const int nc = sm.ncut[lane];
+  const double H = nc > 0 ? s.H[(int64_t)d * s.M + nc - 1] : 0.0;
+  const double amp = sm.amp[lane], Pr = sm.P[2 * d][lane], Pi = sm.P[2 * d + 1][lane];
+  const double sa = sm.ang[0][lane], ca = sm.ang[1][lane];
+  sm.Kr[d][lane] = amp * (Pr * ca - Pi * sa);
+  sm.Ki[d][lane] = amp * (Pr * sa + Pi * ca);
+  sm.hterm[d][lane] = amp * amp * (Pr * Pr + Pi * Pi) * H;
+}
+
 // A cluster of C CTAs takes the same R rows: every CTA forms their coefficients
-// and sums every C-th piece of the bins, the first CTA adds the CTAs' sums (from
-// their shared memory, in rank order) and writes lnL.
+// and sums every C-th piece of the bins, the first CTA adds the pieces' sums (from
+// the CTAs' shared memory) and writes lnL.
+//
+// An item is a (row, piece) on one warp or, with few rows, on a team of two or
+// four: a block takes a lone warp 3.5 us, nearly all of it in the phase and its
+// sine and cosine.  A team's warps form those of two blocks or one each, and
+// then, each for its detectors, add the four blocks' terms in the order in which
+// one warp would.
 template <int NDET>
 __global__ void __launch_bounds__(256, 1) k_fused64(const __grid_constant__ Fused64Args a,
                                                     const double* __restrict__ theta, int64_t B, int R,
@@ -190,20 +231,22 @@ __global__ void __launch_bounds__(256, 1) k_fused64(const __grid_constant__ Fuse
   __shared__ Smem64<NDET> sm;
   constexpr int NS = Smem64<NDET>::NS;
   double* rows = reinterpret_cast<double*>(smem_raw);  // [np][piece] rows of this CTA's pieces
-  double* part = rows + (int64_t)a.np * a.piece * a.row_elems;  // [R][np][NS]
-  const int t = threadIdx.x, lane = t & 31;
-  const int C = a.C, rank = (int)blockIdx.x % C;
-  // this CTA's pieces g C np + rank + C i (i < np) of group g, one thread
+  double* part = rows + (int64_t)a.np * kPiece * a.row_elems;  // [R][keep][NS]
+  const int t = threadIdx.x, lane = t & 31, team = a.team;
+  const int group = (t >> 5) / team, tw = (t >> 5) % team;
+  double* trig = part + R * a.keep * NS + group * (4 * NS * 32);  // (teams) [4 blocks][sine, cosine][32] of this one
+  const int C = 1 << a.lc, rank = (int)blockIdx.x & (C - 1);
+  // this CTA's pieces p0 + C i (i < count), one thread
   auto stage = [&](int64_t p0, int count) {
     uint32_t bytes = 0;
     for (int pass = 0; pass < 2; ++pass) {
       for (int i = 0; i < count; ++i) {
-        const int64_t j0 = (p0 + (int64_t)C * i) * a.piece;
-        const int64_t n = a.seg.M - j0 < a.piece ? a.seg.M - j0 : a.piece;
+        const int64_t j0 = (p0 + (int64_t)C * i) * kPiece;
+        const int64_t n = a.seg.M - j0 < kPiece ? a.seg.M - j0 : kPiece;
         if (n <= 0) break;
         const uint32_t nb = (uint32_t)n * (uint32_t)a.row_elems * 8u;
         if (pass == 0) bytes += nb;
-        else bulk_g2s(rows + (int64_t)i * a.piece * a.row_elems, a.tab + j0 * a.row_elems, nb, &sm.bar);
+        else bulk_g2s(rows + (int64_t)i * kPiece * a.row_elems, a.tab + j0 * a.row_elems, nb, &sm.bar);
       }
       if (pass == 0) mbar_arrive_expect_tx(&sm.bar, bytes);
     }
@@ -216,14 +259,14 @@ __global__ void __launch_bounds__(256, 1) k_fused64(const __grid_constant__ Fuse
     stage(rank, a.np);
   }
   cudaGridDependencySynchronize();  // theta's writer and lnl's earlier users are done
-  const int64_t row0 = (int64_t)(blockIdx.x / C) * R;
+  const int64_t row0 = (int64_t)(blockIdx.x >> a.lc) * R;
   const int n = B - row0 < R ? (int)(B - row0) : R;
   coeffs64<NDET>(a.seg, n, sm, theta + (row0 + lane) * a.seg.stride);
-  for (int i = t; i < NS * kRows64; i += 256) (&sm.acc[0][0])[i] = 0.0;
   const int maxcut = sm.maxcut;
-  const int all = (maxcut + a.piece - 1) / a.piece;  // pieces of the longest row
+  const int all = (maxcut + kPiece - 1) / kPiece;  // pieces of the longest row
   uint32_t parity = 0;
   bool pending = true;
+  int turn = 0;  // (teams) which of sm.item's slots is next
   for (int p0 = rank; p0 - rank < all; p0 += C * a.np) {
     // own pieces that hold bins (none where the rows end before this rank's first one)
     const int np = p0 < all ? min(a.np, (all - p0 + C - 1) / C) : 0;
@@ -239,77 +282,134 @@ __global__ void __launch_bounds__(256, 1) k_fused64(const __grid_constant__ Fuse
     }
     __syncthreads();
     if (sm.fail) break;  // (every thread: the barriers below are still met)
-    const int nk = p0 == 0 ? NDET : 0;  // the first CTA's first items are the detectors' amplitudes
-    while (true) {
-      int item = 0;
-      if (lane == 0) item = atomicAdd(&sm.next, 1);
-      item = __shfl_sync(0xffffffffu, item, 0) - nk;
-      if (item >= n * np) break;
-      if (item < 0) {
-        const int d = item + nk, nc = sm.ncut[lane];
-        const double H = nc > 0 ? a.seg.H[(int64_t)d * a.seg.M + nc - 1] : 0.0;
-        const double amp = sm.amp[lane], Pr = sm.P[2 * d][lane], Pi = sm.P[2 * d + 1][lane];
-        const double sa = sm.ang[0][lane], ca = sm.ang[1][lane];
-        sm.Kr[d][lane] = amp * (Pr * ca - Pi * sa);
-        sm.Ki[d][lane] = amp * (Pr * sa + Pi * ca);
-        sm.hterm[d][lane] = amp * amp * (Pr * Pr + Pi * Pi) * H;
-        continue;
-      }
-      const int pc = item / n, r = item - pc * n;  // all rows' first pieces first: the last ones are the longest rows'
-      int nb = sm.ncut[r] - (p0 + C * pc) * a.piece;  // the piece's bins below the row's cut
-      if (nb <= 0) continue;
-      if (nb > a.piece) nb = a.piece;
-      double c[kNBasis], tau[NDET], U[NDET], V[NDET], v[NS];
+    const int s0 = C > 1 ? (p0 - rank) >> a.lc : 0;  // where the first piece's sums go
+    // all rows' first pieces first: the last ones are the longest rows'
+    if (team > 1) {
+      const int nk = p0 == 0 ? 1 : 0;  // the first CTA's first item is the detectors' amplitudes
+      while (true) {
+        if (tw == 0 && lane == 0) sm.item[group][turn] = atomicAdd(&sm.next, 1);
+        team_sync(group, 32 * team);  // (and every warp of the team is done with the last item's trig)
+        const int item = sm.item[group][turn] - nk;
+        turn ^= 1;
+        if (item >= n * np) break;
+        if (item < 0) {
+          for (int d = tw; d < NDET; d += team) amplitudes64<NDET>(a.seg, sm, d, lane);
+          continue;
+        }
+        const int pc = item / n, r = item - pc * n;
+        const int nb = sm.ncut[r] - (p0 + C * pc) * kPiece;  // the piece's bins below the row's cut, or more
+        if (nb <= 0) continue;
+        const double* pr = rows + (int64_t)pc * kPiece * a.row_elems;
+        double c[kNBasis], tau[NDET];
 #pragma unroll
-      for (int m = 0; m < kNBasis; ++m) c[m] = sm.pf[r].c[m];
+        for (int m = 0; m < kNBasis; ++m) c[m] = sm.pf[r].c[m];
 #pragma unroll
-      for (int d = 0; d < NDET; ++d) {
-        tau[d] = sm.pf[r].tau[d];
-        U[d] = V[d] = 0.0;
-      }
-      const double* pr = rows + (int64_t)pc * a.piece * a.row_elems;
-      for (int j = lane; j < nb; j += 32) {
-        double x[RowD<NDET>::n];
-        load_row<NDET>(pr + (int64_t)j * a.row_elems, x);
-        bin_f64<NDET>(x, c, tau, U, V);
-      }
+        for (int d = 0; d < NDET; ++d) tau[d] = sm.pf[r].tau[d];
+        for (int b = tw; b < kPiece / 32 && 32 * b + lane < nb; b += team) {
+          double x[RowD<NDET>::n], sn[NDET], cs[NDET];
+          load_row<NDET>(pr + (int64_t)(32 * b + lane) * a.row_elems, x);
+          phase_f64<NDET>(x, c, tau, sn, cs);
 #pragma unroll
-      for (int d = 0; d < NDET; ++d) {
-        v[2 * d] = U[d];
-        v[2 * d + 1] = V[d];
+          for (int d = 0; d < NDET; ++d) {
+            trig[(b * NS + 2 * d) * 32 + lane] = sn[d];
+            trig[(b * NS + 2 * d + 1) * 32 + lane] = cs[d];
+          }
+        }
+        team_sync(group, 32 * team);
+        for (int d = tw; d < NDET; d += team) {
+          double v[2] = {0.0, 0.0};
+#pragma unroll
+          for (int b = 0; b < kPiece / 32; ++b)
+            if (32 * b + lane < nb) {
+              const double* g = pr + (int64_t)(32 * b + lane) * a.row_elems + 9 + 2 * d;
+              add_bin64(g[0], g[1], trig[(b * NS + 2 * d) * 32 + lane], trig[(b * NS + 2 * d + 1) * 32 + lane], v[0], v[1]);
+            }
+          const double sum = warp_fold64<2>(v, lane);
+          if (lane % 16 == 0) part[(r * a.keep + s0 + pc) * NS + 2 * d + lane / 16] = sum;
+        }
       }
-      const double sum = warp_fold64<NS>(v, lane);
-      if (lane % 4 == 0 && lane / 4 < NS) part[(r * a.np + pc) * NS + lane / 4] = sum;
+    } else {
+      const int nk = p0 == 0 ? NDET : 0;  // the first CTA's first items are the detectors' amplitudes
+      while (true) {
+        int item = 0;
+        if (lane == 0) item = atomicAdd(&sm.next, 1);
+        item = __shfl_sync(0xffffffffu, item, 0) - nk;
+        if (item >= n * np) break;
+        if (item < 0) {
+          amplitudes64<NDET>(a.seg, sm, item + nk, lane);
+          continue;
+        }
+        const int pc = item / n, r = item - pc * n;
+        int nb = sm.ncut[r] - (p0 + C * pc) * kPiece;  // the piece's bins below the row's cut
+        if (nb <= 0) continue;
+        if (nb > kPiece) nb = kPiece;
+        double c[kNBasis], tau[NDET], U[NDET], V[NDET], v[NS];
+#pragma unroll
+        for (int m = 0; m < kNBasis; ++m) c[m] = sm.pf[r].c[m];
+#pragma unroll
+        for (int d = 0; d < NDET; ++d) {
+          tau[d] = sm.pf[r].tau[d];
+          U[d] = V[d] = 0.0;
+        }
+        const double* pr = rows + (int64_t)pc * kPiece * a.row_elems;
+        for (int j = lane; j < nb; j += 32) {
+          double x[RowD<NDET>::n];
+          load_row<NDET>(pr + (int64_t)j * a.row_elems, x);
+          bin_f64<NDET>(x, c, tau, U, V);
+        }
+#pragma unroll
+        for (int d = 0; d < NDET; ++d) {
+          v[2 * d] = U[d];
+          v[2 * d + 1] = V[d];
+        }
+        const double sum = warp_fold64<NS>(v, lane);
+        constexpr int W = Fold64<NS>::W;
+        if (lane % W == 0 && lane / W < NS) part[(r * a.keep + s0 + pc) * NS + lane / W] = sum;
+      }
     }
     __syncthreads();
-    // the pieces' sums in bin order (one thread per row and sum)
-    for (int i = t; i < n * NS; i += 256) {
-      const int r = i / NS, k = i - r * NS;
-      double x = sm.acc[k][r];
+    if (C == 1) {  // the pieces' sums in bin order (one thread per row and sum)
+      for (int i = t; i < n * NS; i += 256) {
+        const int r = i / NS, k = i - r * NS;
+        double x = p0 == 0 ? 0.0 : sm.acc[k][r];
 #pragma unroll 1
-      for (int pc = 0; pc < np && (p0 + C * pc) * a.piece < sm.ncut[r]; ++pc) x += part[(r * a.np + pc) * NS + k];
-      sm.acc[k][r] = x;
+        for (int pc = 0; pc < np && (p0 + pc) * kPiece < sm.ncut[r]; ++pc) x += part[(r * a.keep + pc) * NS + k];
+        sm.acc[k][r] = x;
+      }
+      __syncthreads();
     }
-    __syncthreads();
   }
   if (pending) mbar_wait_bounded(&sm.bar, parity, a.status);  // no copy may outlive the CTA
-  if (C > 1) cluster_sync();  // every CTA's sums are in place
-  else __syncthreads();
+  if (C > 1) {
+    cluster_sync();  // every CTA's sums are in place
+    if (rank == 0) {  // the same order, each CTA's pieces from its shared memory
+      for (int i = t; i < n * NS; i += 256) {
+        const int r = i / NS, k = i - r * NS, m = (sm.ncut[r] + kPiece - 1) / kPiece;
+        double x = 0.0;
+        for (int p = 0; p < m; p += 8) {
+          double v[8];
+#pragma unroll
+          for (int u = 0; u < 8; ++u)
+            v[u] = p + u < m ? cluster_load(&part[(r * a.keep + ((p + u) >> a.lc)) * NS + k], (uint32_t)((p + u) & (C - 1)))
+                             : 0.0;
+#pragma unroll
+          for (int u = 0; u < 8; ++u) x += v[u];
+        }
+        sm.acc[k][r] = x;
+      }
+    }
+  }
+  __syncthreads();
   if (rank == 0 && t < n) {
     double l = -INFINITY;
     if (!sm.flag[t]) {
       l = 0.0;
       if (sm.ncut[t] > 0) {
-        auto sum = [&](int k) {
-          double x = sm.acc[k][t];
-          for (int q = 1; q < C; ++q) x += cluster_load(&sm.acc[k][t], (uint32_t)q);
-          return x;
-        };
         double hh = 0.0;
 #pragma unroll
         for (int d = 0; d < NDET; ++d) {
           hh += sm.hterm[d][t];
-          l += sm.Kr[d][t] * sum(2 * d) - sm.Ki[d][t] * sum(2 * d + 1);
+          l += sm.Kr[d][t] * sm.acc[2 * d][t] - sm.Ki[d][t] * sm.acc[2 * d + 1][t];
         }
         l -= 0.5 * hh;
       }
@@ -331,14 +431,20 @@ static size_t room64() {
 // (a cluster): of C = 1, 2, 4 and 8 the one with the fewest rows per SM, R / C, is
 // taken, the smallest C among equals, so that neither a handful of rows nor a batch
 // just above the number of SMs leaves SMs idle (160 rows on 152 SMs: 5 rows on 4
-// CTAs each instead of 2 on every second SM).  A piece is a few blocks, so that a
-// row's sums end together on the warps: 32 bins up to 1.5 rows per SM, 64 up to
-// 3, 128 beyond (where the warp sums cost 4 % of a piece).  Segments of more than
-// kMaxBins64 bins keep the separate kernels, whose (row, window) tasks spread over
-// the whole chip (us here against there: 16 s BNS, 2 detectors, 250 rows 741 / 628,
-// 1216 rows 2640 / 2660; 32 s BNS, 1300 rows 8556 / 8044; 128 s BNS, 1300 rows
-// 56314 / 51134, 2048 rows 82305 / 80386; 16 s BBH, 1 detector, 2000 rows 141 /
-// 185, or 147 after the autotuner).
+// CTAs each instead of 2 on every second SM).  Clusters of more CTAs than a row has
+// pieces leave CTAs idle, so C stays below twice the pieces of a row in the middle of
+// the mass prior (8 s BBH, 3 pieces: 100 rows 29.4 us on single CTAs, 39.6 on clusters
+// of eight; 16 rows 16.0 on clusters of four, 30.1 of eight; 8 s BNS, 63 pieces: 100
+// rows 234 us on clusters of eight, 271 on single CTAs).
+//
+// An item is a (row, piece); few rows have fewer items than the SM has warps, and then
+// four warps share one up to 1.5 rows per SM, two up to 3 (one row, 8 s BBH: 15.7 us,
+// 32.9 with a warp per item; 380 rows: 54.0 us, 54.7 with teams of four, 56.0 without).
+// Segments of more than kMaxBins64 bins keep the separate kernels, whose (row, window)
+// tasks spread over the whole chip (us here against there: 16 s BNS, 2 detectors, 250
+// rows 696 / 625, 1216 rows 2610 / 2654; 32 s BNS, 3 detectors, 1300 rows 8495 / 8019;
+// where rows use a small part of their bins the one kernel would win: 16 s BBH, 3
+// detectors, 250 rows 80 / 201, 2000 rows 399 / 411).
 constexpr int64_t kMaxBins64 = 8192;
 
 bool fused64_used(const gwl_ctx* c, int64_t B) {
@@ -346,36 +452,55 @@ bool fused64_used(const gwl_ctx* c, int64_t B) {
   return c->M <= kMaxBins64;
 }
 
+// In-band bins of a row at the middle of the mass prior (the whole segment
+// where the prior does not say).
+static int64_t mid_cut(const gwl_ctx* c) {
+  if (c->opt.fcut_mode != GWL_FCUT_ISCO) return c->M;
+  auto mid = [&](int k) {
+    const int i = c->seg.param_pos[k];
+    return i < 0 ? c->opt.fixed_theta[k] : 0.5 * (c->opt.prior_lo[i] + c->opt.prior_hi[i]);
+  };
+  const double q = mid(1), M = mid(0) * std::pow(q / ((1.0 + q) * (1.0 + q)), -0.6);
+  const double x = (1.0 / (kSix32 * kPi * kTsun * M) - c->f0) / c->df + 1.0;
+  return x > 1.0 && x < (double)c->M ? (int64_t)x : x <= 1.0 ? 1 : c->M;
+}
+
 template <int NDET>
 static cudaError_t run_fused64(gwl_ctx* c, const double* theta, int64_t B, double* lnl, cudaStream_t st) {
   const int64_t sms = c->num_sms;
   const int64_t waves = (B + sms * kRows64 - 1) / (sms * kRows64);
   int64_t R = (B + sms * waves - 1) / (sms * waves);
-  int C = 1;
+  int lc = 0;
+  const int64_t mid = (mid_cut(c) + kPiece - 1) / kPiece;  // pieces of a row in the middle of the prior
   if (waves == 1)
-    for (int k = 2; k <= 8; k *= 2) {
+    for (int k = 1; k <= 3 && 1 << k < 2 * mid; ++k) {
       // clusters resident together: one per TPC (two SMs); four of four or two of eight in a GPC of 18-20 SMs
-      const int64_t groups = k == 2 ? sms / 2 : k == 4 ? sms * 4 / 19 : sms * 2 / 19;
+      const int64_t groups = k == 1 ? sms / 2 : k == 2 ? sms * 4 / 19 : sms * 2 / 19;
       const int64_t r = (B + groups - 1) / groups;
-      if (r <= kRows64 && r * C < R * k) {
+      if (r <= kRows64 && r << lc < R << k) {
         R = r;
-        C = k;
+        lc = k;
       }
     }
+  const int C = 1 << lc;
   const int grid = (int)((B + R - 1) / R) * C;
   Fused64Args a;
   a.seg = c->seg;
   a.tab = c->d_tab_f64;
   a.row_elems = c->row_doubles;
-  a.C = C;
-  a.piece = 2 * R <= 3 * C ? 32 : R <= 3 * C ? 64 : 128;
-  // the pieces that fit beside their sums
-  const size_t per_piece = sizeof(double) * ((size_t)a.piece * a.row_elems + (size_t)R * 2 * NDET);
-  const int64_t own = ((c->M + a.piece - 1) / a.piece + C - 1) / C;
-  const int64_t fit = (int64_t)(room64<NDET>() / per_piece);
+  a.lc = lc;
+  a.team = 2 * R <= 3 * C ? 4 : R <= 3 * C ? 2 : 1;
+  // the pieces that fit beside their sums (of one staging or, in a cluster, of all) and the teams' sines and cosines
+  constexpr int NS = 2 * NDET;
+  const int64_t own = ((c->M + kPiece - 1) / kPiece + C - 1) / C;
+  const size_t per_row = sizeof(double) * (size_t)R * NS, rows = sizeof(double) * (size_t)kPiece * a.row_elems;
+  const size_t fixed = (a.team > 1 ? sizeof(double) * (8 / a.team) * 4 * NS * 32 : 0) + (C > 1 ? per_row * own : 0);
+  const size_t per_piece = rows + (C > 1 ? 0 : per_row);
+  const int64_t fit = (int64_t)((room64<NDET>() - fixed) / per_piece);
   a.np = (int)(fit < own ? fit : own);
+  a.keep = C > 1 ? (int)own : a.np;
   a.status = c->d_status;
-  const size_t smem = (size_t)a.np * per_piece;
+  const size_t smem = fixed + (size_t)a.np * per_piece;
   cudaError_t e = raise_smem_limit((const void*)k_fused64<NDET>, c->device, smem);
   if (e != cudaSuccess) return e;
   ProfScope ps(c, GWL_KERNEL_BINS, st);
