@@ -1050,8 +1050,9 @@ static cudaError_t run_pipeline(gwl_ctx* c, const double* theta, int64_t B, doub
                                 bool cleared = false) {
   const int seg = lanes_seg(c, B);
   int grid, rows, nwc;
-  if (!cleared && !seg && fused_shape(c, B, &grid, &rows, &nwc)) return launch_fused(c, theta, B, lnl, grid, rows, nwc, st);
-  if (!cleared && fused64_used(c, B)) return launch_fused64(c, theta, B, lnl, st);
+  // (whatever the caller has cleared: a row's lnL is the same in a walk and in a batch)
+  if (!seg && fused_shape(c, B, &grid, &rows, &nwc)) return launch_fused(c, theta, B, lnl, grid, rows, nwc, st);
+  if (fused64_used(c, B)) return launch_fused64(c, theta, B, lnl, st);
   int* pdone = c->d_work + 1 + 2 * nw_max(c);
   int* bcount = pdone + B;
   const Buckets bk = seg ? Buckets{bcount, c->d_blist, seg} : Buckets{nullptr, nullptr, 32};
