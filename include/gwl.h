@@ -512,14 +512,16 @@ int gwl_get_tuning(const gwl_ctx* ctx, gwl_tuning* out);
 /* Autotuner: times gwl_loglike (what & GWL_TUNE_LOGLIKE) over every window in
  * {128, 192, ..., 1536} bins that fits in shared memory (at most the segment),
  * every ctas_per_sm in {1, 2, 3, 4} and both bin-loop layouts (GWL_BINS_WARP,
- * and GWL_BINS_LANE with chunks of 32 and 64 bins where it is available),
- * and gwl_grad
- * (what & GWL_TUNE_GRAD) over the same windows (those whose calibration
+ * and GWL_BINS_LANE with chunks of 32 and 64 bins where it is available) --
+ * of these only what the kernel that the batch takes reads: the one-kernel
+ * forms keep the context's ctas_per_sm, and the FP64 one its window too --
+ * and gwl_grad (what & GWL_TUNE_GRAD) over the same windows (those whose calibration
  * scratch fits, with the calibration model), on the caller's batch
  * theta_dev (B x theta_stride, device, row-major, read only) on `stream`, and keeps
- * the fastest shape of each in the context.  Each shape is timed with CUDA
- * events as the best of two runs of three back-to-back calls after one
- * warm-up call.  Outputs go to a device buffer the call allocates and frees;
+ * the fastest shape of each in the context (for gwl_loglike, of the shapes
+ * within 1 % of the fastest the one that was set, else the first).  Each shape is timed with CUDA
+ * events as the best of two runs of back-to-back calls (three or more, about
+ * 0.3 ms) after a warm-up.  Outputs go to a device buffer the call allocates and frees;
  * scratch grows to the largest need of the shapes tried and is kept.  The
  * results are not used; windows whose per-window partial sums would exceed
  * 2 GB at this batch are skipped.  The call synchronises
