@@ -278,10 +278,14 @@ int gwl_create(const double* freqs, int64_t n_bins, const double* strain, const 
     if ((e = dev_alloc(c, &c->d_H, (int64_t)n_det * n_bins)) != cudaSuccess) { rc = cuda_fail(e, "alloc"); break; }
     if ((e = dev_alloc(c, &c->d_tab_mixed, n_bins * c->row_floats)) != cudaSuccess) { rc = cuda_fail(e, "alloc"); break; }
     if ((e = dev_alloc(c, &c->d_tab_delta, n_bins * c->row_delta)) != cudaSuccess) { rc = cuda_fail(e, "alloc"); break; }
-    if ((e = dev_alloc(c, &c->d_tab_block, (n_bins + gwl::kAnchor - 1) / gwl::kAnchor * gwl::block_floats(n_det))) !=
-        cudaSuccess) { rc = cuda_fail(e, "alloc"); break; }
-    if ((e = dev_alloc(c, &c->d_tab_low, (n_bins + gwl::kAnchor - 1) / gwl::kAnchor * gwl::kLowFloats)) !=
-        cudaSuccess) { rc = cuda_fail(e, "alloc"); break; }
+    if (opt->precision == GWL_MIXED) {  // the blocked tables: 80 to 96 bytes per bin that no other mode reads
+      const int64_t nb = (n_bins + gwl::kAnchor - 1) / gwl::kAnchor;
+      if ((e = dev_alloc(c, &c->d_tab_block, nb * gwl::block_floats(n_det))) != cudaSuccess ||
+          (e = dev_alloc(c, &c->d_tab_low, nb * gwl::kLowFloats)) != cudaSuccess) {
+        rc = cuda_fail(e, "alloc");
+        break;
+      }
+    }
     if ((e = dev_alloc(c, &c->d_anchor, (n_bins + gwl::kAnchor - 1) / gwl::kAnchor * gwl::kAnchorRowFloats)) !=
         cudaSuccess) { rc = cuda_fail(e, "alloc"); break; }
     if ((e = dev_alloc(c, &c->d_tab_f64, n_bins * c->row_doubles)) != cudaSuccess) { rc = cuda_fail(e, "alloc"); break; }

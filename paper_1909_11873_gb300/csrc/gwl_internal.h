@@ -26,8 +26,8 @@ struct gwl_ctx {
   float* d_tab_delta = nullptr;  // [M][delta_row_floats]: basis deltas from the block anchor, G_d
   float* d_anchor = nullptr;     // [ceil(M / kAnchor)][kAnchorRowFloats]
   int row_delta = 0;
-  float* d_tab_low = nullptr;    // [ceil(M / kAnchor)][kLowFloats]: the float-float blocks' low parts, blocked
-  float* d_tab_block = nullptr;  // [ceil(M / kAnchor)][block_floats]: the FP32-delta bins' part, blocked
+  float* d_tab_low = nullptr;    // [ceil(M / kAnchor)][kLowFloats]: the float-float blocks' low parts, blocked (mixed contexts)
+  float* d_tab_block = nullptr;  // [ceil(M / kAnchor)][block_floats]: the FP32-delta bins' part, blocked (mixed contexts)
   double* d_tab_f64 = nullptr;   // [M][f64_row_doubles]
   int row_floats = 0, row_doubles = 0;
 

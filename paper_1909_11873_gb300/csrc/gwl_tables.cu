@@ -46,10 +46,13 @@ __global__ void k_table_rows(const double* __restrict__ freqs, const double* __r
 #pragma unroll
   for (int m = 0; m < kNBasis; ++m) {
     split_f64(b[m] - ba[m], rx[m], rx[lo_off + m]);
-    tab_b[block_index(j, m, n_det)] = rx[m];
-    tab_l[low_index(j, m)] = rx[lo_off + m];
+    if (tab_b) {  // (mixed contexts)
+      tab_b[block_index(j, m, n_det)] = rx[m];
+      tab_l[low_index(j, m)] = rx[lo_off + m];
+    }
   }
-  for (int k = kNBasis; k < 4 * block_units(n_det); ++k) tab_b[block_index(j, k, n_det)] = 0.0f;  // G: k_scale_tables
+  if (tab_b)
+    for (int k = kNBasis; k < 4 * block_units(n_det); ++k) tab_b[block_index(j, k, n_det)] = 0.0f;  // G: k_scale_tables
   if (j == ja) {
     float* ra = anc + (j / kAnchor) * kAnchorRowFloats;
 #pragma unroll
@@ -145,8 +148,10 @@ __global__ void k_scale_tables(int64_t M, int n_det, double sg, float* __restric
     tab_m[j * row_f + 19 + 2 * d] = (float)tab_d[j * row_d + 10 + 2 * d];
     tab_x[j * row_x + kNBasis + 2 * d] = tab_m[j * row_f + 18 + 2 * d];
     tab_x[j * row_x + kNBasis + 2 * d + 1] = tab_m[j * row_f + 19 + 2 * d];
-    tab_b[block_index(j, kNBasis + 2 * d, n_det)] = tab_m[j * row_f + 18 + 2 * d];
-    tab_b[block_index(j, kNBasis + 2 * d + 1, n_det)] = tab_m[j * row_f + 19 + 2 * d];
+    if (tab_b) {
+      tab_b[block_index(j, kNBasis + 2 * d, n_det)] = tab_m[j * row_f + 18 + 2 * d];
+      tab_b[block_index(j, kNBasis + 2 * d + 1, n_det)] = tab_m[j * row_f + 19 + 2 * d];
+    }
     H[(int64_t)d * M + j] *= sg * sg;
   }
 }
@@ -208,10 +213,12 @@ cudaError_t launch_cal_tables(gwl_ctx* c, const double* d_xnode, cudaStream_t st
 cudaError_t launch_build_tables(gwl_ctx* c, const double* d_strain, const double* d_psd, cudaStream_t st) {
   const int T = 256;
   const int64_t nb = (c->M + T - 1) / T;
-  // the bins past the last one in its block
-  const int64_t last = (c->M - 1) / kAnchor * block_floats(c->n_det);
-  cudaError_t e = cudaMemsetAsync(c->d_tab_block + last, 0, sizeof(float) * block_floats(c->n_det), st);
-  if (e != cudaSuccess) return e;
+  cudaError_t e;
+  if (c->d_tab_block) {  // the bins past the last one in its block
+    const int64_t last = (c->M - 1) / kAnchor * block_floats(c->n_det);
+    e = cudaMemsetAsync(c->d_tab_block + last, 0, sizeof(float) * block_floats(c->n_det), st);
+    if (e != cudaSuccess) return e;
+  }
   k_table_rows<<<(unsigned)nb, T, 0, st>>>(c->d_freqs, d_strain, d_psd, c->M, c->n_det, c->df, c->opt.t_ref,
                                             c->d_tab_mixed, c->row_floats, c->d_tab_f64, c->row_doubles,
                                             c->d_tab_delta, c->row_delta, c->d_tab_block, c->d_tab_low, c->d_anchor, c->d_H);
