@@ -181,6 +181,20 @@ int walk_supported(const gwl_ctx* c, const char* what) {
   return GWL_OK;
 }
 
+// In-band bins of a row at the middle of the mass prior (the whole segment where
+// the prior does not say): what the rules of the launch shapes take a row's length
+// to be.
+int64_t mid_prior_cut(const gwl_ctx* c) {
+  if (c->opt.fcut_mode != GWL_FCUT_ISCO) return c->M;
+  auto mid = [&](int k) {
+    const int i = c->seg.param_pos[k];
+    return i < 0 ? c->opt.fixed_theta[k] : 0.5 * (c->opt.prior_lo[i] + c->opt.prior_hi[i]);
+  };
+  const double q = mid(1), M = mid(0) * std::pow(q / ((1.0 + q) * (1.0 + q)), -0.6);
+  const double x = (1.0 / (gwl::kSix32 * gwl::kPi * gwl::kTsun * M) - c->f0) / c->df + 1.0;
+  return x > 1.0 && x < (double)c->M ? (int64_t)x : x <= 1.0 ? 1 : c->M;
+}
+
 // The device address of a page-locked host buffer (device-accessible under
 // unified addressing), or null for pageable memory.
 template <class T>
@@ -352,6 +366,7 @@ int gwl_create(const double* freqs, int64_t n_bins, const double* strain, const 
       s.param_pos[k] = -1;
     }
     for (int i = 0; i < opt->n_dim; ++i) s.param_pos[opt->param_map[i]] = i;
+    c->mid_cut = mid_prior_cut(c);
   } while (false);
   if (d_strain) cudaFree(d_strain);
   if (d_psd) cudaFree(d_psd);

@@ -83,36 +83,66 @@ static size_t fused_static(const gwl_ctx* c) {
 }
 constexpr size_t kSmemPerSm = 228 * 1024;  // 1 KB of it goes to each resident CTA's system part
 
-// The launch shape of the fused kernel for a batch of B: CTAs, rows per CTA and
-// windows staged together; false where the separate kernels run.
+// Groups of nwc windows that a row in the middle of the mass prior has.
+int fused_groups(const gwl_ctx* c, int nwc) {
+  const int64_t nw = (c->mid_cut + lnl_window(c) - 1) / lnl_window(c);
+  return (int)((nw + nwc - 1) / nwc);
+}
+
+// Whether the one-kernel form is the faster one for R rows per CTA, per_sm CTAs
+// per SM, nwc windows staged together.
 //
-// Up to a row for each warp (B <= 8 SMs) one CTA per SM, with all its shared
-// memory for windows; past that two CTAs per SM, in whole waves of at most 32
-// rows each.  A CTA walks through its rows' windows by itself, while the
-// separate bin loop spreads (row, window) pairs over the whole chip, so the
-// line is drawn by the number of windows (us per call, 640-bin windows, one
-// kernel against three):
-//   8 s BBH, 3 detectors (one window in use)   B = 1 / 250 / 1900 / 8192 / 20000:
-//     8.6 / 10.4 / 12.2 / 19.6 / 48.2 against 16.6 / 19.2 / 22.4 / 33.7 / 58.0
-//   8 s, every row in all 13 windows           B = 1 / 250 / 1900 / 8192:
-//     21.1 / 26.0 / 65.2 / 203 against 26.6 / 39.4 / 97.5 / 291
-//   16 s BNS, 2 detectors, 26 windows          B = 1 / 250 / 1900 / 8192:
-//     34.1 / 43.8 / 112 / 330 against 33.2 / 50.4 / 139 / 476
-//   32 s BNS, 3 detectors, 51 windows          B = 1 / 64 / 250 / 1900:
-//     59.4 / 61.7 / 73.7 / 243 against 48.4 / 57.5 / 82.1 / 278
-//   128 s BNS, 406 windows                     B = 64 / 1000 / 1900 / 4000:
-//     327 / 1014 / 1492 / 2720 against 248 / 895 / 1529 / 3109
-// so segments of up to 32 windows take it at any batch, longer ones where the
-// batch gives every warp of two CTAs per SM a row.
-bool fused_shape(const gwl_ctx* c, int64_t B, int* grid, int* rows, int* nwc) {
+// A CTA walks through its rows' windows by itself, a group of nwc after another,
+// while the separate bin loop spreads (row, window) pairs over the whole chip.
+// Up to four groups (three with the calibration model) the one kernel wins at
+// any batch.  Beyond, each group costs 4-6 us of staging and barriers, which have
+// to be shared by enough (row, window) items: a CTA with fewer of them than warps
+// leaves the others idle.  How many are enough depends on the other side: it is
+// slow where its windows leave room for one CTA per SM, and fast in small batches,
+// which leave the one-kernel form SMs without a row.  The lines below are drawn
+// through 760 calls timed both ways (1-4 detectors, 4 to 128 s, 256- to 1344-bin
+// windows, 1 to 6000 rows, with and without calibration), among them, in us a
+// call, one kernel against three:
+//   8 s BBH, 3 detectors, 1 group               B = 1 / 400 / 1216 / 4096: 9 / 10 / 11 / 14 against 17 / 19 / 21 / 27
+//   8 s, every row in all 13 windows, 3 groups  B = 1 / 400 / 1216 / 4096: 20 / 32 / 50 / 109 against 28 / 59 / 84 / 177
+//   16 s BNS, 2 detectors, 640-bin windows      B = 1 / 400 / 1217 / 4096: 33 / 48 / 98 / 192 against 33 / 70 / 115 / 278
+//   16 s BNS, 2 detectors, 1280-bin windows     B = 1 / 400 / 1217 / 4096: 38 / 52 / 94 / 182 against 29 / 55 / 93 / 223
+//   32 s BNS, 3 detectors, 1280-bin windows     B = 1 / 152 / 400 / 1216: 89 / 91 / 103 / 171 against 36 / 89 / 129 / 273
+//   32 s BNS, 3 detectors, 640-bin windows      B = 1 / 400 / 1217 / 2400: 63 / 105 / 211 / 251 against 47 / 114 / 213 / 364
+//   16 s BNS, calibrated, 640-bin windows       B = 1 / 400 / 1216 / 1600 / 2400: 68 / 109 / 179 / 251 / 278
+//                                                                      against 37 / 97 / 184 / 228 / 317
+// Small batches on segments of more than 32 windows go to the separate kernels.
+static bool fused_pays(const gwl_ctx* c, int64_t B, int per_sm, int R, int nwc) {
+  if (fused_window_count(c) > 32 && per_sm == 1) return false;
+  const bool cal = c->n_cal_nodes > 0;
+  const int G = fused_groups(c, nwc);
+  if (G <= (cal ? 3 : 4)) return true;
+  const int items = R * nwc, rounds = (items + 7) / 8;  // of the eight warps
+  // whether two CTAs of k_window fit an SM: its window, and its own arrays
+  const size_t window = (size_t)lnl_window(c) * lnl_row_bytes(c) +
+                        (size_t)(lnl_window(c) / kAnchor) * kAnchorRowFloats * sizeof(float);
+  const bool two = window + 2304 + (cal ? 3328 : 1024) * c->n_det + 1024 <= kSmemPerSm / 2;
+  // (a few calibrated rows, one window at a time, would be 1.3-1.9 times faster in three kernels up to six groups too)
+  if (!two) return per_sm == 2 || items >= (cal && nwc == 1 ? 6 : 4) || (cal && G <= 6 && nwc == 1);
+  if (per_sm == 2) return cal ? items >= 17 || (items >= 7 && 10 * items >= 64 * rounds) : items >= 6 || G <= 16;
+  if (cal)
+    return 4 * B >= c->num_sms &&
+           ((G <= 5 && items >= 3) || (items >= 8 && 20 * items >= 152 * rounds) || (items >= 20 && 10 * items >= 64 * rounds));
+  return items >= (B >= c->num_sms ? 3 : 2 * B >= c->num_sms ? 5 : 6);
+}
+
+// The launch shape of the fused kernel for a batch of B: CTAs, rows per CTA and
+// windows staged together; false where it does not fit.  Up to a row for each warp
+// (B <= 8 SMs) one CTA per SM, with all its shared memory for windows; past that
+// two CTAs per SM, in whole waves of at most 32 rows each.
+static bool fused_fits(const gwl_ctx* c, int64_t B, int* grid, int* rows, int* nwc, int* per_sm) {
   if (c->opt.precision != GWL_MIXED || B <= 0) return false;
-  if (fused_window_count(c) > 32 && B <= 8 * (int64_t)c->num_sms) return false;
-  const int per_sm = B <= 8 * (int64_t)c->num_sms ? 1 : 2;
-  const int64_t slots = per_sm * (int64_t)c->num_sms;
+  *per_sm = B <= 8 * (int64_t)c->num_sms ? 1 : 2;
+  const int64_t slots = *per_sm * (int64_t)c->num_sms;
   const int64_t waves = (B + slots * kFusedRows - 1) / (slots * kFusedRows);
   const int64_t R = (B + slots * waves - 1) / (slots * waves);
   const int64_t G = (B + R - 1) / R;
-  const int w = fused_windows(c, (int)R, (per_sm == 1 ? 227 * 1024 : kSmemPerSm / 2 - 1024) - fused_static(c) - 128);
+  const int w = fused_windows(c, (int)R, (*per_sm == 1 ? 227 * 1024 : kSmemPerSm / 2 - 1024) - fused_static(c) - 128);
   if (w == 0) return false;
   *grid = (int)G;
   *rows = (int)R;
@@ -120,10 +150,26 @@ bool fused_shape(const gwl_ctx* c, int64_t B, int* grid, int* rows, int* nwc) {
   return true;
 }
 
+// The same, false too where the separate kernels are the faster ones.  (Of the
+// batches that are not the lane layout's: with GWL_BINS_AUTO, the default, those
+// are the ones below 2048 rows, and calibrated ones; from 2048 rows on the
+// one-kernel form runs with GWL_BINS_WARP, which the autotuner sets where it is
+// the faster one.)
+bool fused_shape(const gwl_ctx* c, int64_t B, int* grid, int* rows, int* nwc) {
+  int per_sm;
+  return fused_fits(c, B, grid, rows, nwc, &per_sm) && fused_pays(c, B, per_sm, *rows, *nwc);
+}
+
 // Whether gwl_loglike takes the fused kernel for a batch of B.
 bool fused_used(const gwl_ctx* c, int64_t B) {
   int grid, rows, nwc;
   return !lanes_seg(c, B) && fused_shape(c, B, &grid, &rows, &nwc);
+}
+
+// Whether a walk of n chains may (its own line is with it).
+bool fused_possible(const gwl_ctx* c, int64_t n) {
+  int grid, rows, nwc, per_sm;
+  return !lanes_seg(c, n) && fused_fits(c, n, &grid, &rows, &nwc, &per_sm);
 }
 
 FusedArgs fused_args(const gwl_ctx* c, int nwc) {

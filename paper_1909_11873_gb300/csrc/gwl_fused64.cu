@@ -452,26 +452,13 @@ bool fused64_used(const gwl_ctx* c, int64_t B) {
   return c->M <= kMaxBins64;
 }
 
-// In-band bins of a row at the middle of the mass prior (the whole segment
-// where the prior does not say).
-static int64_t mid_cut(const gwl_ctx* c) {
-  if (c->opt.fcut_mode != GWL_FCUT_ISCO) return c->M;
-  auto mid = [&](int k) {
-    const int i = c->seg.param_pos[k];
-    return i < 0 ? c->opt.fixed_theta[k] : 0.5 * (c->opt.prior_lo[i] + c->opt.prior_hi[i]);
-  };
-  const double q = mid(1), M = mid(0) * std::pow(q / ((1.0 + q) * (1.0 + q)), -0.6);
-  const double x = (1.0 / (kSix32 * kPi * kTsun * M) - c->f0) / c->df + 1.0;
-  return x > 1.0 && x < (double)c->M ? (int64_t)x : x <= 1.0 ? 1 : c->M;
-}
-
 template <int NDET>
 static cudaError_t run_fused64(gwl_ctx* c, const double* theta, int64_t B, double* lnl, cudaStream_t st) {
   const int64_t sms = c->num_sms;
   const int64_t waves = (B + sms * kRows64 - 1) / (sms * kRows64);
   int64_t R = (B + sms * waves - 1) / (sms * waves);
   int lc = 0;
-  const int64_t mid = (mid_cut(c) + kPiece - 1) / kPiece;  // pieces of a row in the middle of the prior
+  const int64_t mid = (c->mid_cut + kPiece - 1) / kPiece;  // pieces of a row in the middle of the prior
   if (waves == 1)
     for (int k = 1; k <= 3 && 1 << k < 2 * mid; ++k) {
       // clusters resident together: one per TPC (two SMs); four of four or two of eight in a GPC of 18-20 SMs

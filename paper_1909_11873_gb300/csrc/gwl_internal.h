@@ -16,6 +16,7 @@ struct gwl_ctx {
   int n_det = 0;
   double f0 = 0.0, df = 0.0;
   gwl_options opt{};
+  int64_t mid_cut = 0;           // in-band bins of a row at the middle of the mass prior (launch shapes)
   gwl::SegInfo seg{};  // device pointers inside
 
   // device tables (owned)
@@ -146,6 +147,8 @@ bool fused_shape(const gwl_ctx* c, int64_t B, int* grid, int* rows, int* nwc);
 int fused_window_count(const gwl_ctx* c);
 int fused_windows(const gwl_ctx* c, int R, size_t room);
 bool fused_used(const gwl_ctx* c, int64_t B);
+bool fused_possible(const gwl_ctx* c, int64_t n);
+int fused_groups(const gwl_ctx* c, int nwc);
 // the FP64 one-kernel form (gwl_fused64.cu)
 bool fused64_used(const gwl_ctx* c, int64_t B);
 cudaError_t launch_fused64(gwl_ctx* c, const double* theta, int64_t B, double* lnl, cudaStream_t st);

@@ -1321,13 +1321,21 @@ static auto for_model(const gwl_ctx* c, F f) {
   }
 }
 
-// Whether the random walk of n chains runs as one kernel: where gwl_loglike of
-// n rows would (gwl_fused.cu gives the line and both sides).
+// Whether the random walk of n chains runs as one kernel.  It saves the launches
+// of a step as well, so it wins where gwl_loglike's rows already take the separate
+// kernels (us a step, one kernel against three launches: 16 s BNS, 4 detectors,
+// 1280-bin windows, 1 / 152 / 1217 chains 54 / 55 / 110 against 64 / 88 / 203; 16 s
+// BNS, calibrated, 400 chains 121 against 531), but for a few chains with many
+// groups of windows (32 s BNS, 3 detectors, 1280-bin windows, 1 / 40 / 152 chains:
+// 88 / 90 / 91 against 68 / 73 / 127), and small rounds on segments of more than 32
+// windows, which keep the separate kernels.
 static bool walk_fused_shape(const gwl_ctx* c, int64_t n, WalkShape* o) {
-  if (c->walk_kind != GWL_WALK_RANDOM || !fused_used(c, n)) return false;
-  return for_model(c, [&](auto nd, auto cal) {
+  if (c->walk_kind != GWL_WALK_RANDOM || !fused_possible(c, n)) return false;
+  if (fused_window_count(c) > 32 && n <= 8 * (int64_t)c->num_sms) return false;
+  const bool fits = for_model(c, [&](auto nd, auto cal) {
     return walk_shape_of<decltype(nd)::value, decltype(cal)::value>(c, n, o);
   });
+  return fits && (n >= c->num_sms || c->n_cal_nodes || fused_groups(c, o->nwc) <= 8);
 }
 
 template <int NDET, bool CAL, int NW>
@@ -1362,8 +1370,7 @@ static cudaError_t launch_walk_fused(gwl_ctx* c, const WalkScalars& val, const W
 }
 
 // ns_replace's walk in the one-kernel form, its scalars passed by value; false
-// where the separate kernels run (the line is fused_shape's: the walk's step is
-// that likelihood).
+// where the separate kernels run.
 bool launch_walk_direct(gwl_ctx* c, const double* live_u, const double* live_lnl, int64_t K, int64_t worst,
                         double lstar, uint64_t seed, uint64_t counter, int64_t n_chains, int walk_len, double scale,
                         const double* chol, double* out_u, double* out_lnl, int32_t* out_nacc, int32_t* out_start,
