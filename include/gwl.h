@@ -462,11 +462,18 @@ int gwl_test_ffdelta_blocks(gwl_ctx* ctx, int enable, int64_t* count);
  * `window` frequency bins staged in shared memory, drained by warps of 32
  * lanes, one proposal per warp; the grid is sized in CTAs per SM).  The
  * result of gwl_loglike/gwl_grad depends on the shape only through the FP32
- * (mixed) or FP64 summation order, within the parity tolerances. */
+ * (mixed) or FP64 summation order, within the parity tolerances.  A row's
+ * result does not depend on the rows beside it.  With one shape set it does
+ * not depend on the size of its batch either, but for the order in which the
+ * mixed path adds in FP64 the FP32 sums of a row's windows (on segments of more
+ * than 32 windows it differs between small and large batches) and, with
+ * GWL_BINS_AUTO, for the layout.  The FP64 path adds in an order of its own
+ * where it runs as one kernel (segments of up to 8192 bins, no calibration),
+ * and so do its walks; its multi-event batches add window by window. */
 typedef struct gwl_tuning {
   int window;        /* likelihood bin loop: bins per window; 0 keeps (set) */
   int ctas_per_sm;   /* likelihood bin loop: grid = ctas_per_sm x SMs; 0 keeps (the one-kernel
-                        forms, which most calls take, choose their own grid) */
+                        forms choose their own grid) */
   int grad_window;   /* gradient bin loop: bins per window; 0 keeps */
   double ms_loglike; /* gwl_autotune output: best time of one gwl_loglike call
                         (ms) at the tuned batch; gwl_get_tuning: last tuned value or 0 */
@@ -531,10 +538,10 @@ int gwl_autotune(gwl_ctx* ctx, const double* theta_dev, int64_t B, int what, gwl
 
 /* Kernel classes for gwl_profile_read. */
 #define GWL_KERNEL_PROLOGUE 0 /* per-proposal coefficients */
-#define GWL_KERNEL_BINS 1     /* windowed bin loop of gwl_loglike */
+#define GWL_KERNEL_BINS 1     /* windowed bin loop of gwl_loglike, or its one kernel */
 #define GWL_KERNEL_COMBINE 2  /* per-proposal combination */
 #define GWL_KERNEL_GRAD 3     /* windowed bin loop of gwl_grad */
-#define GWL_KERNEL_WALK 4     /* random-walk proposal/accept steps of ns_replace */
+#define GWL_KERNEL_WALK 4     /* random-walk proposal/accept steps of ns_replace, or the whole walk in one kernel */
 #define GWL_KERNEL_CALGRAD 5  /* calibration-moment pass of gwl_grad (calibration model) */
 #define GWL_KERNEL_KINDS 6
 

@@ -182,8 +182,9 @@ __global__ void __launch_bounds__(256, 1) k_cal_moments(CalGradArgs a) {
   }
   __syncthreads();
   // This grid may run beside the gradient's bin loop, whose CTAs let it launch
-  // once they have seen the prologue complete: it reads nothing of theirs.  It
-  // waits for them at its end, so that the combination, which waits for this
+  // once they have seen the prologue complete: what it reads is the prologue's,
+  // in place by that wait of theirs (a bin loop that let it in earlier would
+  // open a race), and nothing of their own.  It waits for them at its end, so that the combination, which waits for this
   // grid, finds both done.
   const int maxn = *a.maxcut;
   int nw = (maxn + a.CH - 1) / a.CH;

@@ -525,8 +525,14 @@ __global__ void __launch_bounds__(32) k_gmc_end(GmcArgs a, int D) {
 // velocity is partly refreshed,
 //   v <- rho v + sqrt(1 - rho^2) scale L z  (z: the normals of this step's word),
 // which keeps its distribution N(0, scale^2 L L^T); then x1 = u + v and
-// theta1 (NaN rows outside the cube).  The normals, which depend on no other
-// kernel of the step, are formed before the wait for the likelihood.
+// theta1 (NaN rows outside the cube).  The normals are formed before the wait
+// for the likelihood: all they read is the step matrix and the scalars, written
+// before the walk.  That these are in place rests on the gradient of the step
+// before, whose first kernel is an ordinary launch (it starts when everything
+// before it is complete) and whose last one lets its successor in only at its
+// end.  If the gradient's kernels all became programmatic dependents, a step
+// could start beside the kernels that write them, and the draw would have to
+// follow the wait.
 __global__ void __launch_bounds__(32 * kGmcWarps) k_gmc_step1(PriorInfo pr, GmcArgs a, uint32_t step, double rho) {
   __shared__ double s_z[kMaxWalkDim + 1], s_dz[kMaxWalkDim], s_x[kMaxWalkDim];
   __shared__ int s_in;
