@@ -93,6 +93,18 @@ int ensure_scratch(gwl_ctx* c, int64_t B) {
   return GWL_OK;
 }
 
+// Whether that scratch has still to grow for a batch of B.
+bool scratch_short(const gwl_ctx* c, int64_t B) {
+  return B > c->prop_cap || gwl::work_needed(c, B) > c->work_cap || gwl::lanes_list_ints(c, B) > c->blist_cap ||
+         gwl::partials_needed(c, B) > c->partials_cap;
+}
+bool capturing(cudaStream_t st) {
+  cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &s) == cudaSuccess) return s != cudaStreamCaptureStatusNone;
+  cudaGetLastError();
+  return false;
+}
+
 int ensure_bytes(gwl_ctx* c, void** p, int64_t* cap, int64_t need) {
   if (need <= *cap) return GWL_OK;
   const int64_t n = need > 2 * *cap ? need : 2 * *cap;
@@ -384,10 +396,21 @@ int gwl_loglike(gwl_ctx* c, const double* theta_dev, int64_t B, double* lnl_dev,
   if (B < 0) return fail(GWL_ERR_ARG, "B < 0");
   if (B == 0) return GWL_OK;
   if (!theta_dev || !lnl_dev) return fail(GWL_ERR_ARG, "null device pointer");
-  if (!gwl::fused_used(c, B) && !gwl::fused64_used(c, B) && (rc = ensure_scratch(c, B))) return rc;  // the one-kernel form needs no scratch
   cudaStream_t st = (cudaStream_t)stream;
+  cudaError_t e;
+  bool anyway = false;
+  if (!gwl::fused_used(c, B) && !gwl::fused64_used(c, B)) {
+    // the separate kernels need scratch; where it cannot grow (nothing may be allocated during a capture, or the
+    // device is full), a batch that fits the one-kernel form takes that one, which needs none
+    anyway = scratch_short(c, B) && gwl::fused_possible(c, B) && capturing(st);
+    if (!anyway && (rc = ensure_scratch(c, B))) {
+      if (rc != GWL_ERR_NOMEM || !gwl::fused_possible(c, B)) return rc;
+      cudaGetLastError();
+      anyway = true;
+    }
+  }
   c->last_stream = st;
-  cudaError_t e = gwl::launch_loglike(c, theta_dev, B, lnl_dev, st);
+  e = anyway ? gwl::launch_fused_possible(c, theta_dev, B, lnl_dev, st) : gwl::launch_loglike(c, theta_dev, B, lnl_dev, st);
   if (e != cudaSuccess) return cuda_fail(e, "gwl_loglike");
   return GWL_OK;
 }
@@ -467,16 +490,25 @@ int ns_replace(gwl_ctx* c, const double* live_u, const double* live_lnl, int64_t
   if (n_chains == 0) return GWL_OK;
   if (!live_u || !live_lnl || !chol || !out_u || !out_lnl || !out_nacc) return fail(GWL_ERR_ARG, "null device pointer");
   const int D = (int)gwl::theta_stride(c);
-  cudaError_t e = cudaSuccess;
-  if (gwl::launch_walk_direct(c, live_u, live_lnl, K, worst, lnl_star, seed, counter, n_chains, walk_len, scale, chol,
-                              out_u, out_lnl, out_nacc, out_start, (cudaStream_t)stream, &e)) {
-    c->last_stream = (cudaStream_t)stream;
-    return e == cudaSuccess ? GWL_OK : cuda_fail(e, "ns_replace");
-  }
-  if ((rc = ensure_scratch(c, n_chains))) return rc;
-  if ((rc = ensure_bytes(c, (void**)&c->d_walk, &c->walk_cap, (int64_t)sizeof(double) * n_chains * (2 * D + 1))))
-    return rc;
   cudaStream_t st = (cudaStream_t)stream;
+  cudaError_t e = cudaSuccess;
+  auto direct = [&](bool anyway) {
+    if (!gwl::launch_walk_direct(c, live_u, live_lnl, K, worst, lnl_star, seed, counter, n_chains, walk_len, scale, chol,
+                                 out_u, out_lnl, out_nacc, out_start, anyway, st, &e))
+      return false;
+    c->last_stream = st;
+    rc = e == cudaSuccess ? GWL_OK : cuda_fail(e, "ns_replace");
+    return true;
+  };
+  // as in gwl_loglike, the one-kernel form also where it is the slower one but needs no scratch and no copy
+  if (direct(false) || (capturing(st) && direct(true))) return rc;
+  rc = ensure_scratch(c, n_chains);
+  if (!rc) rc = ensure_bytes(c, (void**)&c->d_walk, &c->walk_cap, (int64_t)sizeof(double) * n_chains * (2 * D + 1));
+  if (rc) {
+    const int why = rc;
+    if (why == GWL_ERR_NOMEM) cudaGetLastError();
+    return why == GWL_ERR_NOMEM && direct(true) ? rc : why;
+  }
   c->last_stream = st;
   unsigned char hs[64];
   gwl::set_walk_scalars(hs, lnl_star, scale, worst, counter);

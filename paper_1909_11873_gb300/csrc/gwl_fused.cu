@@ -111,9 +111,7 @@ int fused_groups(const gwl_ctx* c, int nwc) {
 //   32 s BNS, 3 detectors, 640-bin windows      B = 1 / 400 / 1217 / 2400: 63 / 105 / 211 / 251 against 47 / 114 / 213 / 364
 //   16 s BNS, calibrated, 640-bin windows       B = 1 / 400 / 1216 / 1600 / 2400: 68 / 109 / 179 / 251 / 278
 //                                                                      against 37 / 97 / 184 / 228 / 317
-// Small batches on segments of more than 32 windows go to the separate kernels.
 static bool fused_pays(const gwl_ctx* c, int64_t B, int per_sm, int R, int nwc) {
-  if (fused_window_count(c) > 32 && per_sm == 1) return false;
   const bool cal = c->n_cal_nodes > 0;
   const int G = fused_groups(c, nwc);
   if (G <= (cal ? 3 : 4)) return true;
@@ -134,10 +132,12 @@ static bool fused_pays(const gwl_ctx* c, int64_t B, int per_sm, int R, int nwc) 
 // The launch shape of the fused kernel for a batch of B: CTAs, rows per CTA and
 // windows staged together; false where it does not fit.  Up to a row for each warp
 // (B <= 8 SMs) one CTA per SM, with all its shared memory for windows; past that
-// two CTAs per SM, in whole waves of at most 32 rows each.
+// two CTAs per SM, in whole waves of at most 32 rows each.  Small batches on segments
+// of more than 32 windows always go to the separate kernels.
 static bool fused_fits(const gwl_ctx* c, int64_t B, int* grid, int* rows, int* nwc, int* per_sm) {
   if (c->opt.precision != GWL_MIXED || B <= 0) return false;
   *per_sm = B <= 8 * (int64_t)c->num_sms ? 1 : 2;
+  if (fused_window_count(c) > 32 && *per_sm == 1) return false;
   const int64_t slots = *per_sm * (int64_t)c->num_sms;
   const int64_t waves = (B + slots * kFusedRows - 1) / (slots * kFusedRows);
   const int64_t R = (B + slots * waves - 1) / (slots * waves);
@@ -166,7 +166,7 @@ bool fused_used(const gwl_ctx* c, int64_t B) {
   return !lanes_seg(c, B) && fused_shape(c, B, &grid, &rows, &nwc);
 }
 
-// Whether a walk of n chains may (its own line is with it).
+// Whether it could (a walk of n chains has a line of its own).
 bool fused_possible(const gwl_ctx* c, int64_t n) {
   int grid, rows, nwc, per_sm;
   return !lanes_seg(c, n) && fused_fits(c, n, &grid, &rows, &nwc, &per_sm);
@@ -217,6 +217,13 @@ cudaError_t launch_fused(gwl_ctx* c, const double* theta, int64_t B, double* lnl
     default: return cal ? run_fused<4, true>(c, theta, B, lnl, grid, rows, nwc, st)
                         : run_fused<4, false>(c, theta, B, lnl, grid, rows, nwc, st);
   }
+}
+
+// The one-kernel form wherever it fits, the faster one or not.
+cudaError_t launch_fused_possible(gwl_ctx* c, const double* theta, int64_t B, double* lnl, cudaStream_t st) {
+  int grid, rows, nwc, per_sm;
+  if (!fused_fits(c, B, &grid, &rows, &nwc, &per_sm)) return cudaErrorInvalidValue;
+  return launch_fused(c, theta, B, lnl, grid, rows, nwc, st);
 }
 
 }  // namespace gwl

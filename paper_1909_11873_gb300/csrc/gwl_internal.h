@@ -148,6 +148,7 @@ int fused_window_count(const gwl_ctx* c);
 int fused_windows(const gwl_ctx* c, int R, size_t room);
 bool fused_used(const gwl_ctx* c, int64_t B);
 bool fused_possible(const gwl_ctx* c, int64_t n);
+cudaError_t launch_fused_possible(gwl_ctx* c, const double* theta, int64_t B, double* lnl, cudaStream_t st);
 int fused_groups(const gwl_ctx* c, int nwc);
 // the FP64 one-kernel form (gwl_fused64.cu)
 bool fused64_used(const gwl_ctx* c, int64_t B);
@@ -177,11 +178,12 @@ cudaError_t launch_walk(gwl_ctx* c, const double* live_u, const double* live_lnl
                         uint64_t seed, int64_t n_chains, int walk_len, const double* chol, double* out_u,
                         double* out_lnl, int32_t* out_nacc, int32_t* out_start, double* pu, double* pth,
                         double* plnl, cudaStream_t st);
-// the one-kernel walk with its scalars by value and no scratch (false: not used for this shape)
+// the one-kernel walk with its scalars by value and no scratch (false: not used for this shape; anyway: also where
+// the separate kernels are the faster ones)
 bool launch_walk_direct(gwl_ctx* c, const double* live_u, const double* live_lnl, int64_t K, int64_t worst,
                         double lstar, uint64_t seed, uint64_t counter, int64_t n_chains, int walk_len, double scale,
                         const double* chol, double* out_u, double* out_lnl, int32_t* out_nacc, int32_t* out_start,
-                        cudaStream_t st, cudaError_t* e);
+                        bool anyway, cudaStream_t st, cudaError_t* e);
 size_t walk_scalars_bytes();
 size_t gmc_scratch_doubles(int64_t n_chains, int D);
 void set_walk_scalars(void* host_buf, double lstar, double scale, int64_t worst, uint64_t counter);

@@ -1335,13 +1335,12 @@ static auto for_model(const gwl_ctx* c, F f) {
 // groups of windows (32 s BNS, 3 detectors, 1280-bin windows, 1 / 40 / 152 chains:
 // 88 / 90 / 91 against 68 / 73 / 127), and small rounds on segments of more than 32
 // windows, which keep the separate kernels.
-static bool walk_fused_shape(const gwl_ctx* c, int64_t n, WalkShape* o) {
+static bool walk_fused_shape(const gwl_ctx* c, int64_t n, WalkShape* o, bool anyway = false) {
   if (c->walk_kind != GWL_WALK_RANDOM || !fused_possible(c, n)) return false;
-  if (fused_window_count(c) > 32 && n <= 8 * (int64_t)c->num_sms) return false;
   const bool fits = for_model(c, [&](auto nd, auto cal) {
     return walk_shape_of<decltype(nd)::value, decltype(cal)::value>(c, n, o);
   });
-  return fits && (n >= c->num_sms || c->n_cal_nodes || fused_groups(c, o->nwc) <= 8);
+  return fits && (anyway || n >= c->num_sms || c->n_cal_nodes || fused_groups(c, o->nwc) <= 8);
 }
 
 template <int NDET, bool CAL, int NW>
@@ -1380,9 +1379,9 @@ static cudaError_t launch_walk_fused(gwl_ctx* c, const WalkScalars& val, const W
 bool launch_walk_direct(gwl_ctx* c, const double* live_u, const double* live_lnl, int64_t K, int64_t worst,
                         double lstar, uint64_t seed, uint64_t counter, int64_t n_chains, int walk_len, double scale,
                         const double* chol, double* out_u, double* out_lnl, int32_t* out_nacc, int32_t* out_start,
-                        cudaStream_t st, cudaError_t* e) {
+                        bool anyway, cudaStream_t st, cudaError_t* e) {
   WalkShape sh;
-  if (!walk_fused_shape(c, n_chains, &sh)) return false;
+  if (!walk_fused_shape(c, n_chains, &sh, anyway)) return false;
   WalkScalars v;
   v.lstar = lstar;
   v.scale = scale;
