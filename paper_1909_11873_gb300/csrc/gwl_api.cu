@@ -93,11 +93,6 @@ int ensure_scratch(gwl_ctx* c, int64_t B) {
   return GWL_OK;
 }
 
-// Whether that scratch has still to grow for a batch of B.
-bool scratch_short(const gwl_ctx* c, int64_t B) {
-  return B > c->prop_cap || gwl::work_needed(c, B) > c->work_cap || gwl::lanes_list_ints(c, B) > c->blist_cap ||
-         gwl::partials_needed(c, B) > c->partials_cap;
-}
 bool capturing(cudaStream_t st) {
   cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(st, &s) == cudaSuccess) return s != cudaStreamCaptureStatusNone;
@@ -400,9 +395,10 @@ int gwl_loglike(gwl_ctx* c, const double* theta_dev, int64_t B, double* lnl_dev,
   cudaError_t e;
   bool anyway = false;
   if (!gwl::fused_used(c, B) && !gwl::fused64_used(c, B)) {
-    // the separate kernels need scratch; where it cannot grow (nothing may be allocated during a capture, or the
-    // device is full), a batch that fits the one-kernel form takes that one, which needs none
-    anyway = scratch_short(c, B) && gwl::fused_possible(c, B) && capturing(st);
+    // the separate kernels need scratch; a batch that fits the one-kernel form takes that one, which needs none,
+    // during a capture (nothing may be allocated, and a graph must not hold scratch that a later call replaces)
+    // and where the device is full
+    anyway = gwl::fused_possible(c, B) && capturing(st);
     if (!anyway && (rc = ensure_scratch(c, B))) {
       if (rc != GWL_ERR_NOMEM || !gwl::fused_possible(c, B)) return rc;
       cudaGetLastError();

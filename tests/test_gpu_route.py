@@ -106,4 +106,12 @@ def test_first_calls_under_capture():
     assert float((lnl - ref).abs().max()) < 1e-10
     assert torch.equal(out[2], want[2]) and torch.equal(out[3], want[3]) and torch.equal(out[0], want[0])
     assert float((out[1] - want[1]).abs().max()) < 1e-10
+    # the graph holds no scratch: it gives the same after calls that have replaced the context's
+    first = [lnl.clone()] + [o.clone() for o in out]
+    for rows in (u, u.repeat(100, 1)):
+        g.loglike(ctx, rows)
+    g.grad(ctx, u.repeat(100, 1))
+    graph.replay()
+    torch.cuda.synchronize()
+    assert all(torch.equal(a, b) for a, b in zip(first, [lnl] + out))
     ctx.gwl_sync()
